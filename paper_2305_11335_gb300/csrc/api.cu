@@ -1217,17 +1217,20 @@ int dpc_decision_graph(const dpc_batch* b, const int32_t* rho, const double* del
   // dimension); rows of empty instances keep the padding written first
   CallPlan P = make_plan(b, insts, 0, 1, true);
   if ((rc = prepare(w, P, b, insts, nullptr, flags))) return rc;
-  launch_decision_init(b->n_inst, k, top, gamma, rho_bins, delta_bins,
+  const size_t members = P.classes.empty() ? 0 : P.classes[0].members.size();
+  launch_decision_init(b->n_inst, k, members < (size_t)b->n_inst, top, gamma, rho_bins, delta_bins,
                        (unsigned long long*)hist, w->stream);
   for (const ClassPlan& c : P.classes) {
     const ClassView cv = view_of(w, c, insts);
     if (k > 0 &&
         (rc = w->reserve_buf(&w->scr, &w->scr_bytes, decision_scratch_bytes(cv.ninst, k))))
       return rc;
-    launch_class_init(cv, c.g, c.ib, c.bcap, w->status, w->stream);
     launch_chunks(cv, w->chunk_inst, w->chunk_pos, w->stream);
-    launch_decision(rho, delta, cv, k, top, gamma, rho_bins, delta_bins, delta_lo,
-                    (unsigned long long*)hist, w->scr, w->stream);
+    if (launch_decision(rho, delta, cv, k, top, gamma, rho_bins, delta_bins, delta_lo,
+                        (unsigned long long*)hist, w->scr, w->status, w->stream)) {
+      cudaGetLastError();
+      return DPC_ERR_CUDA;
+    }
   }
   return finish(w, flags);
 }

@@ -192,10 +192,11 @@ void launch_dep_far(int dp, bool fp64, const float* spts, const unsigned long lo
 // ---- decision graph (decision.cu) -------------------------------------------------
 // top-k by gamma = rho * delta and the (rho, delta) histogram of every instance
 // of the class (rho, delta indexed by output index; top/gamma [n_inst][k] and
-// hist [n_inst][rho_bins][delta_bins] by batch row, InstDev::row)
-void launch_decision(const int32_t* rho, const double* delta, const ClassView& cv, int k,
+// hist [n_inst][rho_bins][delta_bins] by batch row, InstDev::row); 0, or -1
+// when a launch failed
+int launch_decision(const int32_t* rho, const double* delta, const ClassView& cv, int k,
                      int32_t* top, double* gamma, int rho_bins, int delta_bins, double delta_lo,
-                     unsigned long long* hist, void* scratch, cudaStream_t st);
+                     unsigned long long* hist, void* scratch, int* status, cudaStream_t st);
 // device scratch launch_decision needs for a class of ninst instances
 size_t decision_scratch_bytes(uint32_t ninst, int k);
 // ---- priority range search (range.cu) -------------------------------------------
@@ -226,8 +227,9 @@ void launch_prange_scatter(const unsigned long long* keys, uint64_t total,
                            int* status, cudaStream_t st);
 
 int decision_max_topk();
-// padding of every top-k row (-1, NaN) and zero histograms for n_inst rows
-void launch_decision_init(int n_inst, int k, int32_t* top, double* gamma, int rho_bins,
+// padding of every top-k row (-1, NaN; `pad`: some rows have no points) and
+// zero histograms for n_inst rows
+void launch_decision_init(int n_inst, int k, bool pad, int32_t* top, double* gamma, int rho_bins,
                           int delta_bins, unsigned long long* hist, cudaStream_t st);
 
 // ---- labels (labels.cu) -------------------------------------------------------------
