@@ -248,8 +248,8 @@ int dpc_decision_graph(const dpc_batch* b, const int32_t* rho, const double* del
  * search kd-tree): for each query, the points of one instance inside a closed
  * axis-parallel box whose priority -- the density rho -- is above a
  * threshold:  { i : lo[a] <= x_i[a] <= hi[a] for a < d, and rho_i > rho_q }.
- * The search runs on the same radix tree as the dependent-point step,
- * entering a subtree only if its largest density is above rho_q and its
+ * The search runs on a 32-ary hierarchy of bounding boxes over the sorted
+ * points, entering a node only if its largest density is above rho_q and its
  * bounding box meets the query box.
  *   pts, dtype, b  the points, as for dpc_density (the first cutoff of every
  *                  instance sizes the search grid; results do not depend on it)
@@ -268,10 +268,7 @@ int dpc_decision_graph(const dpc_batch* b, const int32_t* rho, const double* del
  * (DPC_ERR_DATA with DPC_FLAG_SYNC_CHECK).  With max_out > 0 the call reads
  * the number of matches back once per dimension class, so it synchronizes
  * `stream`; more than 2^32 - 1 matches in one class returns DPC_ERR_OVERFLOW.
- * Flags: DPC_FLAG_SYNC_CHECK only.  The environment variable
- * DPC_RANGE_STACK (1..2048) caps the per-warp node stack; a smaller cap sends
- * more subtrees to the per-lane walk (for testing that path; results do not
- * depend on it). */
+ * Flags: DPC_FLAG_SYNC_CHECK only. */
 int dpc_priority_range(const void* pts, int dtype, const dpc_batch* b, const int32_t* rho,
                        int32_t n_query, const int32_t* q_inst, const double* q_box,
                        const int32_t* q_rho, int32_t max_out, int64_t* count, int32_t* ids,

@@ -1253,7 +1253,7 @@ int dpc_priority_range(const void* pts, int dtype, const dpc_batch* b, const int
   if ((rc = get_workspace((cudaStream_t)stream, &w))) return rc;
   std::lock_guard<std::mutex> lk(g_mu);
   // classes by dimension; the first cutoff of every instance sizes its grid
-  // (the tree does not depend on it)
+  // (the results do not depend on it)
   CallPlan P = make_plan(b, insts, 0, 1, false);
   if ((rc = prepare(w, P, b, insts, nullptr, flags))) return rc;
   cudaStream_t st = w->stream;
@@ -1275,18 +1275,13 @@ int dpc_priority_range(const void* pts, int dtype, const dpc_batch* b, const int
   a.rowmap = nullptr;
   a.one_row = -1;
   a.count = (long long*)count;
-  a.stack_cap = 0;
-  if (const char* e = std::getenv("DPC_RANGE_STACK")) a.stack_cap = std::atoi(e);
   launch_prange_init(a, ids, max_out, w->status, st);
   std::vector<int32_t> map_host((size_t)b->n_inst);
   for (const ClassPlan& c : P.classes) {
     const ClassView cv = view_of(w, c, insts);
     bin_class(w, pts, dtype, P, c, cv, b, insts);
-    tree_step(w, cv);
     launch_keys_from_rho(rho, w->sid, cv.N, w->skey, st);
-    launch_tree_maxkey(w->skey, w->spts, c.dp, cv.N, w->nodes, w->leaf_parent, w->visit, w->nbox,
-                       true, st);
-    w->boxes_ready = true;
+    launch_prange_boxes(c.dp, w->spts, w->skey, cv, w->nbox, st);
     if (c.uploaded()) {
       std::fill(map_host.begin(), map_host.end(), -1);
       for (size_t j = 0; j < c.members.size(); ++j) map_host[c.members[j]] = (int32_t)j;
@@ -1299,15 +1294,22 @@ int dpc_priority_range(const void* pts, int dtype, const dpc_batch* b, const int
       a.rowmap = nullptr;
       a.one_row = c.members[0];
     }
-    launch_prange(c.dp, false, w->spts, w->sid, w->skey, cv, w->nodes, w->nbox, w->roots, a, cnt,
-                  nullptr, nullptr, w->status, st);
+    // the warp's buffer serves up to prange_top_ids() ids in one pass
+    const bool top = max_out > 0 && max_out <= prange_top_ids();
+    if (top) cudaMemsetAsync(off + nq, 0, sizeof(unsigned long long), st);
+    launch_prange(c.dp, top ? 2 : 0, w->spts, w->skey, cv, w->nbox, a, cnt, nullptr, nullptr, ids, max_out,
+                  off + nq, w->status, st);
     if (max_out == 0) continue;
-    launch_prange_scan(cnt, nq, off, st);
+    if (!top) launch_prange_scan(cnt, nq, off, st);
     unsigned long long total = 0;
     if (cudaMemcpyAsync(&total, off + nq, sizeof(total), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess) {
       cudaGetLastError();
       return DPC_ERR_CUDA;
+    }
+    if (top) {
+      if (total >= (1ull << 32)) return DPC_ERR_OVERFLOW;
+      continue;
     }
     if (total == 0) continue;
     if (total >= (1ull << 32)) return DPC_ERR_OVERFLOW;
@@ -1322,8 +1324,8 @@ int dpc_priority_range(const void* pts, int dtype, const dpc_batch* b, const int
     char* s2 = (char*)w->scr2;
     unsigned long long* keys_a = (unsigned long long*)(s2 + k_a);
     unsigned long long* keys_b = (unsigned long long*)(s2 + k_b);
-    launch_prange(c.dp, true, w->spts, w->sid, w->skey, cv, w->nodes, w->nbox, w->roots, a, cnt, off,
-                  keys_a, w->status, st);
+    launch_prange(c.dp, 1, w->spts, w->skey, cv, w->nbox, a, cnt, off, keys_a, ids, max_out, nullptr,
+                  w->status, st);
     // sort the keys (query << 31 | id): 31 id bits under ib query bits
     int ib = 0;
     while (ib < 32 && (1ull << ib) < nq) ++ib;

@@ -209,18 +209,21 @@ struct PrangeArgs {
   const int32_t* rowmap;    // [n_inst] class-local index or -1; null: one_row only
   int32_t one_row;          // the batch row of a single-instance class
   long long* count;         // [nq] matches (device output)
-  int stack_cap;            // shared stack entries per warp (0: all); smaller
-                            //   values send more subtrees to the per-lane walk
 };
 void launch_prange_init(const PrangeArgs& a, int32_t* ids, int max_out, int* status,
                         cudaStream_t st);
-// one class: count (fill = false: cnt[q] for the class's queries, 0 for the
-// others, and count[q]) or fill (keys (q << 31 | id) at off[q]..)
-void launch_prange(int dp, bool fill, const float* spts, const uint32_t* sid,
-                   const unsigned long long* skey, const ClassView& cv, const Node* nodes,
-                   const float* nbox, const uint32_t* roots, const PrangeArgs& a, uint32_t* cnt,
-                   const unsigned long long* off, unsigned long long* keys, int* status,
-                   cudaStream_t st);
+// the box hierarchy of one class (rec: at least 22 words per chunk)
+void launch_prange_boxes(int dp, const float* spts, const unsigned long long* skey,
+                         const ClassView& cv, float* rec, cudaStream_t st);
+// one class.  mode 0 (count): cnt[q] for the class's queries, 0 for the
+// others, and count[q]; 1 (fill): keys (q << 31 | id) at off[q]..; 2 (top):
+// count[q], the max_out <= prange_top_ids() smallest ids of each query, and
+// the class's matches added to *total
+void launch_prange(int dp, int mode, const float* spts, const unsigned long long* skey,
+                   const ClassView& cv, float* rec, const PrangeArgs& a, uint32_t* cnt,
+                   const unsigned long long* off, unsigned long long* keys, int32_t* ids,
+                   int max_out, unsigned long long* total, int* status, cudaStream_t st);
+int prange_top_ids();
 void launch_prange_scan(const uint32_t* cnt, uint32_t nq, unsigned long long* off, cudaStream_t st);
 void launch_prange_scatter(const unsigned long long* keys, uint64_t total,
                            const unsigned long long* off, uint32_t nq, int max_out, int32_t* ids,
