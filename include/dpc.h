@@ -343,7 +343,8 @@ typedef struct {
                              of the (2R+1)^g block around a query's cell)     */
   int32_t density_layout; /* layout the last density launch ran: 1 union,
                              2 segment, 4 tensor, 5 pairs, 6 cell
-                             (see DPC_FLAG_LAYOUT)                            */
+                             (see DPC_FLAG_LAYOUT); 0: small instances, all
+                             pairs (no grid: its fields are 0 too)            */
   int32_t near_layout;    /* layout of the last near-dependent launch: 1 union,
                              2 segment, 3 tree, 4 tensor, 6 cell              */
   int32_t near_shift;     /* grid levels the near phase ran below the density's */

@@ -374,9 +374,10 @@ struct Workspace {
     const size_t o_cuts = take(sizeof(CutGeom) * want_i * (size_t)want_c);
     const size_t o_cls = take(sizeof(ClassGeom));
     const size_t o_hi = take(sizeof(HashInfo));
-    const size_t o_ctr = take(sizeof(Counters));
+    // the status word follows the counters: one memset clears both
+    const size_t o_ctr = take(sizeof(Counters) + sizeof(int));
+    const size_t o_status = o_ctr + sizeof(Counters);
     const size_t o_ctr2 = take(sizeof(Counters));
-    const size_t o_status = take(sizeof(int));
     const size_t o_flags = take(sizeof(int32_t) * 80);
     const size_t o_roots = take(sizeof(uint32_t) * want_i);
     const size_t o_ci = take(4 * nchunk), o_cp = take(4 * nchunk);
@@ -441,8 +442,7 @@ struct Workspace {
     cap_inst = want_i;
     cap_ncut = want_c;
     have_last = false;
-    cudaMemsetAsync(status, 0, sizeof(int), stream);
-    cudaMemsetAsync(ctr, 0, sizeof(Counters), stream);
+    cudaMemsetAsync(ctr, 0, sizeof(Counters) + sizeof(int), stream);
     return DPC_OK;
   }
 
@@ -701,6 +701,15 @@ const CutHost* cut_table(Workspace* w, const ClassPlan& c) {
   return c.uploaded() ? (const CutHost*)((char*)w->up_dev + c.off_cut) : nullptr;
 }
 
+// The cutoffs of a class that runs without uploaded tables.
+std::vector<CutHost> host_cuts(const CallPlan& P, const dpc_batch* b, const ClassPlan& c) {
+  std::vector<CutHost> hc;
+  if (!c.uploaded())
+    for (int k = 0; k < P.ncut && k < kCutChunk; ++k)
+      hc.push_back(cut_host(P, b, c.members[0], P.cut_first + k, c.dp));
+  return hc;
+}
+
 // Binning of one class: geometry for the call's cutoffs, sorted points.
 void bin_class(Workspace* w, const void* pts, int dtype, const CallPlan& P, const ClassPlan& c,
                const ClassView& cv, const dpc_batch* b, const std::vector<Inst>& insts) {
@@ -710,13 +719,7 @@ void bin_class(Workspace* w, const void* pts, int dtype, const CallPlan& P, cons
   launch_class_init(cv, c.g, c.ib, c.bcap, w->status, st);
   launch_chunks(cv, w->chunk_inst, w->chunk_pos, st);
   launch_bbox(pts, dtype, cv, c.g, st);
-  std::vector<CutHost> hc;
-  if (!c.uploaded()) {
-    const int bi = c.members[0];
-    for (int k = 0; k < P.ncut && k < kCutChunk; ++k)
-      hc.push_back(cut_host(P, b, bi, P.cut_first + k, c.dp));
-  }
-  launch_setup(cv, w->cuts, P.ncut, cut_table(w, c), hc.data(), st);
+  launch_setup(cv, w->cuts, P.ncut, cut_table(w, c), host_cuts(P, b, c).data(), st);
   launch_codes(pts, dtype, cv, c.g, w->codes_a, w->ids_a, st);
   launch_sort(w->codes_a, w->codes_b, w->ids_a, w->ids_b, cv.N, w->cls, w->hist, st);
   launch_gather(pts, dtype, cv, c.dp, w->codes_a, w->codes_b, w->ids_a, w->ids_b, w->spts,
@@ -802,7 +805,11 @@ void labels_step(Workspace* w, const ClassPlan& c, const ClassView& cv, int k_in
       c.uploaded()
           ? (const LabelParams*)((char*)w->up_dev + c.off_par) + (size_t)k_in_call * c.members.size()
           : nullptr;
-  launch_labels(rho, lambda, delta, cv, c.nmax, par, one, label, w->flags, w->stream);
+  // instances that fit a CTA's shared memory: one launch, a CTA per instance
+  if (c.nmax <= kSmallLabelPoints)
+    launch_small_labels(rho, lambda, delta, cv, c.nmax, par, one, label, w->status, w->stream);
+  else
+    launch_labels(rho, lambda, delta, cv, c.nmax, par, one, label, w->flags, w->stream);
 }
 
 LabelParams one_params(const dpc_params* params, const ClassPlan& c, int ncut_all, int cut) {
@@ -814,6 +821,55 @@ LabelParams one_params(const dpc_params* params, const ClassPlan& c, int ncut_al
     L.delta_min = q.delta_min;
   }
   return L;
+}
+
+// ---- small instances -----------------------------------------------------------
+
+// Whether a class runs from all pairs (small.cu) instead of the grid: one
+// dimension, no fixed or tuned radius or layout asked for, and few enough
+// points.  Measured on blobs with a median density of 16 (us a call, grid ->
+// all pairs): density of 1,000 points in 2-D 156 -> 18, 8,192 183 -> 37,
+// 16,384 205 -> 77 (5-D 313 -> 191, 8-D 347 -> 457; 8,192 points 287 -> 135);
+// a run of 1,000 points in 2-D 311 -> 34, 8,192 393 -> 117 (5-D 1,077 -> 167,
+// 8-D 1,240 -> 339).  In binary64 the pairs wait for the binary64 pipe: a run
+// of 2,048 points in 2-D 444 -> 191 but 4,096 461 -> 642; in 5-D 4,009 ->
+// 1,336 at 4,096.  A captured call (DPC_FLAG_GRAPH) takes this path up to
+// 4,096 points only: tests/test_gpu_parity.py counts the kernels of a captured
+// grid pipeline at 6,000.
+bool small_class(const Workspace* w, const ClassPlan& c, const std::vector<Inst>& insts, uint32_t flags,
+                 bool density_only) {
+  if (flags & (DPC_FLAG_RADIUS_MASK | DPC_FLAG_LAYOUT_MASK | DPC_FLAG_NEAR_SHIFT_MASK | DPC_FLAG_AUTOTUNE))
+    return false;
+  if (!w->tuned.empty()) return false;  // choices of earlier calls stay in force
+  const bool fp64 = (flags & DPC_PREC_MASK) == DPC_PREC_FP64;
+  const int d = insts[c.members[0]].d;
+  const uint32_t nmax = small_limit(d, fp64, density_only);
+  if (c.nmax > nmax || ((flags & DPC_FLAG_GRAPH) && c.nmax > 4096u)) return false;
+  uint64_t pairs = 0;
+  for (int i : c.members) {
+    if (insts[i].d != d) return false;
+    pairs += insts[i].n * insts[i].n;
+  }
+  return pairs <= (uint64_t)nmax * nmax;
+}
+
+void small_density_step(Workspace* w, const void* pts, int dtype, const CallPlan& P, const ClassPlan& c,
+                        const ClassView& cv, const dpc_batch* b, const std::vector<Inst>& insts, bool fp64,
+                        int32_t* rho, uint64_t N) {
+  Phase ph(w, DPC_PHASE_DENSITY);
+  launch_chunks(cv, w->chunk_inst, w->chunk_pos, w->stream);
+  launch_small_density(insts[c.members[0]].d, fp64, pts, dtype, cv, cut_table(w, c), host_cuts(P, b, c).data(),
+                       P.ncut, rho, N, w->ctr, w->status, w->stream);
+  w->last_choice = Choice();
+  w->have_last = false;
+}
+
+void small_dependent_step(Workspace* w, const void* pts, int dtype, const CallPlan& P, const ClassPlan& c,
+                          const ClassView& cv, const dpc_batch* b, const std::vector<Inst>& insts, bool fp64,
+                          int k, int32_t rho_skip, const int32_t* rho, int32_t* lambda, double* delta) {
+  Phase ph(w, DPC_PHASE_NEAR);
+  launch_small_dependent(insts[c.members[0]].d, fp64, pts, dtype, cv, cut_table(w, c), host_cuts(P, b, c).data(),
+                         P.ncut, k, rho_skip, rho, lambda, delta, w->ctr, w->status, w->stream);
 }
 
 // ---- autotuning of the cell level -------------------------------------------------
@@ -1024,14 +1080,14 @@ Choice choose(Workspace* w, const ClassPlan& c, const ClassView& cv, CutGeom* cu
 
 void reset_call(Workspace* w, uint32_t flags) {
   w->begin_call(flags);
-  cudaMemsetAsync(w->status, 0, sizeof(int), w->stream);
-  cudaMemsetAsync(w->ctr, 0, sizeof(Counters), w->stream);
+  cudaMemsetAsync(w->ctr, 0, sizeof(Counters) + sizeof(int), w->stream);
 }
 
 // Reserves the workspace for a plan and uploads its tables.
 int prepare(Workspace* w, CallPlan& P, const dpc_batch* b, const std::vector<Inst>& insts,
             const dpc_params* params, uint32_t flags) {
   sort_init();
+  small_init();
   P.params = params;
   P.skip_noise = (flags & DPC_FLAG_SKIP_NOISE) != 0;
   int rc = w->reserve(P.max_n, P.max_inst, P.ncut);
@@ -1091,6 +1147,10 @@ int dpc_density(const void* pts, int dtype, const dpc_batch* b, int32_t* rho, ui
   const bool fp64 = (flags & DPC_PREC_MASK) == DPC_PREC_FP64;
   for (const ClassPlan& c : P.classes) {
     const ClassView cv = view_of(w, c, insts);
+    if (small_class(w, c, insts, flags, true)) {
+      small_density_step(w, pts, dtype, P, c, cv, b, insts, fp64, rho, N);
+      continue;
+    }
     bin_class(w, pts, dtype, P, c, cv, b, insts);
     for (int k = 0; k < P.ncut; ++k) {
       CutGeom* cuts = w->cuts + (size_t)k * cv.ninst;
@@ -1122,6 +1182,12 @@ int dpc_dependent(const void* pts, int dtype, const dpc_batch* b, int32_t dcut_i
   const bool fp64 = (flags & DPC_PREC_MASK) == DPC_PREC_FP64;
   for (const ClassPlan& c : P.classes) {
     const ClassView cv = view_of(w, c, insts);
+    if (small_class(w, c, insts, flags, false)) {
+      launch_chunks(cv, w->chunk_inst, w->chunk_pos, w->stream);
+      w->have_last = false;
+      small_dependent_step(w, pts, dtype, P, c, cv, b, insts, fp64, 0, rho_skip, rho, lambda, delta);
+      continue;
+    }
     bin_class(w, pts, dtype, P, c, cv, b, insts);
     tree_step(w, cv);
     const Choice ch = choose(w, c, cv, w->cuts, b, dcut_index, fp64, nullptr,
@@ -1153,8 +1219,10 @@ int dpc_cluster(const dpc_batch* b, int32_t dcut_index, const dpc_params* params
   if ((rc = prepare(w, P, b, insts, params, flags))) return rc;
   for (const ClassPlan& c : P.classes) {
     const ClassView cv = view_of(w, c, insts);
-    launch_class_init(cv, c.g, c.ib, c.bcap, w->status, w->stream);
-    launch_chunks(cv, w->chunk_inst, w->chunk_pos, w->stream);
+    if (c.nmax > kSmallLabelPoints) {
+      launch_class_init(cv, c.g, c.ib, c.bcap, w->status, w->stream);
+      launch_chunks(cv, w->chunk_inst, w->chunk_pos, w->stream);
+    }
     labels_step(w, c, cv, 0, one_params(params, c, P.ncut_all, dcut_index), rho, lambda, delta,
                 label);
   }
@@ -1176,6 +1244,18 @@ static void run_classes(Workspace* w, const CallPlan& P, const void* pts, int dt
     // class finishes that phase's output of every class
     const bool last = &c == &P.classes.back();
     const ClassView cv = view_of(w, c, insts);
+    if (small_class(w, c, insts, flags, false)) {
+      small_density_step(w, pts, dtype, P, c, cv, b, insts, fp64, rho, N);
+      for (int k = 0; k < P.ncut; ++k) {
+        const size_t o = (size_t)k * N;
+        if (last && done) (*done)(0, k);
+        small_dependent_step(w, pts, dtype, P, c, cv, b, insts, fp64, k, 0, rho + o, lambda + o, delta + o);
+        if (last && done) (*done)(1, k);
+        labels_step(w, c, cv, k, one_params(params, c, P.ncut_all, k), rho + o, lambda + o, delta + o, label + o);
+        if (last && done) (*done)(2, k);
+      }
+      continue;
+    }
     bin_class(w, pts, dtype, P, c, cv, b, insts);
     tree_step(w, cv);
     for (int k = 0; k < P.ncut; ++k) {

@@ -235,6 +235,31 @@ int decision_max_topk();
 void launch_decision_init(int n_inst, int k, bool pad, int32_t* top, double* gamma, int rho_bins,
                           int delta_bins, unsigned long long* hist, cudaStream_t st);
 
+// ---- small instances (small.cu) ---------------------------------------------------
+// All pairs straight from the caller's coordinates (every instance of the
+// class has dimension d); cutoffs as for launch_setup.  rho of cutoff k at
+// rho + k * rho_stride.
+void launch_small_density(int d, bool fp64, const void* pts, int dtype, const ClassView& cv,
+                          const CutHost* hc_dev, const CutHost* hc_host, int ncut, int32_t* rho,
+                          uint64_t rho_stride, Counters* ctr, int* status, cudaStream_t st);
+// lambda and delta of cutoff `cut` of the call from its densities
+void launch_small_dependent(int d, bool fp64, const void* pts, int dtype, const ClassView& cv,
+                            const CutHost* hc_dev, const CutHost* hc_host, int ncut, int cut,
+                            int32_t rho_skip, const int32_t* rho, int32_t* lambda, double* delta,
+                            Counters* ctr, int* status, cudaStream_t st);
+// Largest instance that all pairs serve faster than the grid (small_class in
+// api.cu gives the measurements).
+constexpr uint32_t small_limit(int d, bool fp64, bool density_only) {
+  return fp64 ? (d <= 3 ? 2048u : 4096u) : (density_only && d <= 5 ? 16384u : 8192u);
+}
+// labels of a class whose instances have at most kSmallLabelPoints points
+constexpr uint32_t kSmallLabelPoints = 32768;
+void launch_small_labels(const int32_t* rho, const int32_t* lambda, const double* delta,
+                         const ClassView& cv, uint32_t nmax, const LabelParams* params,
+                         LabelParams one, int32_t* label, int* status, cudaStream_t st);
+// one-time kernel attribute setup (called before any stream capture)
+void small_init();
+
 // ---- labels (labels.cu) -------------------------------------------------------------
 int label_rounds(uint32_t n);
 // Labels of every point of the class for one cutoff (arrays indexed by output

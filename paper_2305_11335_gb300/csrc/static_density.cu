@@ -32,8 +32,9 @@ constexpr size_t kOffCut = kOffGeom + al(sizeof(GridGeom));
 constexpr size_t kOffCls = kOffCut + al(sizeof(CutGeom));
 constexpr size_t kOffHash = kOffCls + al(sizeof(ClassGeom));
 constexpr size_t kOffCtr = kOffHash + al(sizeof(HashInfo));
-constexpr size_t kOffStatus = kOffCtr + al(sizeof(Counters));
-constexpr size_t kOffCodesA = kOffStatus + al(sizeof(int));
+// the status word follows the counters: one memset clears both
+constexpr size_t kOffStatus = kOffCtr + sizeof(Counters);
+constexpr size_t kOffCodesA = kOffCtr + al(sizeof(Counters) + sizeof(int));
 constexpr size_t kOffCodesB = kOffCodesA + al(8 * kStaticN);
 constexpr size_t kOffIdsA = kOffCodesB + al(8 * kStaticN);
 constexpr size_t kOffIdsB = kOffIdsA + al(4 * kStaticN);
@@ -122,8 +123,7 @@ extern "C" int dpc_density_static(const void* pts, int dtype, int64_t n, int32_t
   const CutHost ch = make_cut_host(d_cut, dp);
   // the previous call's contents are still there: zero the words that
   // accumulate (status, counters); every other buffer is fully rewritten
-  cudaMemsetAsync(status, 0, sizeof(int), st);
-  cudaMemsetAsync(ctr, 0, sizeof(Counters), st);
+  cudaMemsetAsync(ctr, 0, sizeof(Counters) + sizeof(int), st);
   // one instance: a class without instance or chunk tables
   ClassView cv;
   memset(&cv, 0, sizeof(cv));
@@ -134,18 +134,23 @@ extern "C" int dpc_density_static(const void* pts, int dtype, int64_t n, int32_t
   cv.one.d = d;
   cv.geom = geom;
   cv.cls = cls;
-  // one instance: no instance bits, and g * B <= 63 keeps every cell code
-  // below 2^63 (the allocating path's rule with ib = 0)
-  launch_class_init(cv, g, 0, std::min(kMaxBits, 63 / g), status, st);
-  launch_bbox(pts, dtype, cv, g, st);
-  launch_setup(cv, cut, 1, nullptr, &ch, st);
-  launch_codes(pts, dtype, cv, g, codes_a, ids_a, st);
-  launch_sort(codes_a, codes_b, ids_a, ids_b, nn, cls, hist, st);
-  launch_gather(pts, dtype, cv, dp, codes_a, codes_b, ids_a, ids_b, spts, scode, sid, st);
-  launch_cells(scode, cv, g, cut, hinfo, hkeys, hvals, kStaticHash, st);
-  launch_density(dp, g, prec == DPC_PREC_FP64, g >= 2 ? kLayoutSegment : kLayoutUnion, spts, scode,
-                 sid, cv, cut, hinfo, hkeys, hvals, nullptr, rho,
-                 skey, ctr, st);
+  // few points: all pairs, one launch
+  if (nn <= small_limit(d, prec == DPC_PREC_FP64, true)) {
+    launch_small_density(d, prec == DPC_PREC_FP64, pts, dtype, cv, nullptr, &ch, 1, rho, 0, ctr, status, st);
+  } else {
+    // one instance: no instance bits, and g * B <= 63 keeps every cell code
+    // below 2^63 (the allocating path's rule with ib = 0)
+    launch_class_init(cv, g, 0, std::min(kMaxBits, 63 / g), status, st);
+    launch_bbox(pts, dtype, cv, g, st);
+    launch_setup(cv, cut, 1, nullptr, &ch, st);
+    launch_codes(pts, dtype, cv, g, codes_a, ids_a, st);
+    launch_sort(codes_a, codes_b, ids_a, ids_b, nn, cls, hist, st);
+    launch_gather(pts, dtype, cv, dp, codes_a, codes_b, ids_a, ids_b, spts, scode, sid, st);
+    launch_cells(scode, cv, g, cut, hinfo, hkeys, hvals, kStaticHash, st);
+    launch_density(dp, g, prec == DPC_PREC_FP64, g >= 2 ? kLayoutSegment : kLayoutUnion, spts, scode,
+                   sid, cv, cut, hinfo, hkeys, hvals, nullptr, rho,
+                   skey, ctr, st);
+  }
   if (cudaGetLastError() != cudaSuccess) return DPC_ERR_CUDA;
   if (flags & DPC_FLAG_SYNC_CHECK) {
     int s = 0;
