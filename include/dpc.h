@@ -312,7 +312,7 @@ int dpc_run_host(const void* pts_host, int dtype, const dpc_batch* b, const dpc_
  *   rho     device, int32 [n]: the same densities dpc_density writes for this
  *           point set and cutoff
  *   flags   precision (DPC_PREC_*) and DPC_FLAG_SYNC_CHECK as for dpc_density
- * All scratch memory is one fixed array of about 7 MB compiled into the
+ * All scratch memory is one fixed array of about 8 MB compiled into the
  * library, so every GPU that loads the library holds it until the process
  * exits.  The first call on a device looks up that array's device address
  * (cudaGetSymbolAddress, with that device current); make that first call

@@ -163,6 +163,7 @@ struct ClassPlan {
   int dp = 0, g = 0;
   std::vector<int> members;  // batch indices
   uint32_t N = 0, nchunk = 0, nmax = 0;
+  int dmax = 1;  // largest dimension of its instances
   int ib = 0, bcap = kMaxBits;
   // offsets of this class's tables in the upload block (multi-instance only)
   size_t off_inst = 0, off_cut = 0, off_par = 0;
@@ -189,6 +190,7 @@ std::vector<ClassPlan> plan_classes(const std::vector<Inst>& insts, bool all_one
       c.N += (uint32_t)in.n;
       c.nchunk += (uint32_t)((in.n + 31) / 32);
       c.nmax = std::max(c.nmax, (uint32_t)in.n);
+      c.dmax = std::max(c.dmax, in.d);
     }
     if (c.members.empty()) continue;
     int ib = 0;
@@ -208,6 +210,8 @@ struct Choice {
   int nlay = 0;  // near-phase layout
   int ns = 0;    // near-phase grid levels below the density's
   int sc = 0;    // segment layouts: cells a segment's union may hold (0: one cell)
+  uint32_t dfill = 0, nfill = 0;  // points per cell from which a tensor layout runs (0: always)
+  int nsparse = kLayoutUnion;     // near layout below nfill
 };
 
 struct Workspace {
@@ -221,6 +225,7 @@ struct Workspace {
 
   GridGeom* geom = nullptr;   // [cap_inst]
   CutGeom* cuts = nullptr;    // [cap_ncut][cap_inst]
+  CutGeom* geo = nullptr;     // [cap_inst] geometry shared by the cutoffs of a group
   ClassGeom* cls = nullptr;
   HashInfo* hinfo = nullptr;
   Counters* ctr = nullptr;
@@ -245,7 +250,7 @@ struct Workspace {
   bool boxes_ready = false; // nbox matches the current binning
   uint32_t* leaf_parent = nullptr;
   uint32_t* visit = nullptr;
-  uint2* pieces = nullptr;        // 128-point pieces of the cells (tensor-core density)
+  uint4* pieces = nullptr;        // pieces of up to 128 points (tensor-core layouts)
   uint32_t* qpos = nullptr;
   float* qs1 = nullptr;
   double* qs1d = nullptr;
@@ -289,6 +294,7 @@ struct Workspace {
 
   // for dpc_get_stats: the last class and cutoff that ran
   Choice last_choice;
+  uint32_t last_points = 0;  // points of the class last_cut belongs to
   const CutGeom* last_cut = nullptr;
   const GridGeom* last_geom = nullptr;
   bool have_last = false;
@@ -372,6 +378,7 @@ struct Workspace {
     auto take = [&](size_t b) { size_t o = off; off += align_up(b); return o; };
     const size_t o_geom = take(sizeof(GridGeom) * want_i);
     const size_t o_cuts = take(sizeof(CutGeom) * want_i * (size_t)want_c);
+    const size_t o_geo = take(sizeof(CutGeom) * want_i);
     const size_t o_cls = take(sizeof(ClassGeom));
     const size_t o_hi = take(sizeof(HashInfo));
     // the status word follows the counters: one memset clears both
@@ -392,7 +399,7 @@ struct Workspace {
     const size_t o_nodes = take(sizeof(Node) * N);
     const size_t o_nbox = take(4 * (size_t)kRecWordsMax * N);
     const size_t o_lp = take(4 * N), o_visit = take(4 * N);
-    const size_t o_pieces = take(8 * N);
+    const size_t o_pieces = take(sizeof(uint4) * N);
     const size_t o_qpos = take(4 * N), o_qs1 = take(4 * N), o_qs1d = take(8 * N);
     const size_t o_qpos2 = take(4 * N), o_qs1_2 = take(4 * N), o_qs1d2 = take(8 * N);
     void* p = nullptr;
@@ -406,6 +413,7 @@ struct Workspace {
     char* b = (char*)p;
     geom = (GridGeom*)(b + o_geom);
     cuts = (CutGeom*)(b + o_cuts);
+    geo = (CutGeom*)(b + o_geo);
     cls = (ClassGeom*)(b + o_cls);
     hinfo = (HashInfo*)(b + o_hi);
     ctr = (Counters*)(b + o_ctr);
@@ -431,7 +439,7 @@ struct Workspace {
     nbox = (float*)(b + o_nbox);
     leaf_parent = (uint32_t*)(b + o_lp);
     visit = (uint32_t*)(b + o_visit);
-    pieces = (uint2*)(b + o_pieces);
+    pieces = (uint4*)(b + o_pieces);
     qpos = (uint32_t*)(b + o_qpos);
     qs1 = (float*)(b + o_qs1);
     qs1d = (double*)(b + o_qs1d);
@@ -727,6 +735,16 @@ void bin_class(Workspace* w, const void* pts, int dtype, const CallPlan& P, cons
   (void)insts;
 }
 
+// Points per occupied cell from which the default layouts of 5-8 dimensions use
+// tensor tiles: a tile serves up to 128 queries at the cost of one, but sparse
+// cells leave its rows empty and every piece pays its lookups and waits.
+// Densities of 1e5 points in 5-D at 4 cutoffs (2-4 points per cell): 1.17 ms
+// with tiles from 1 point on, 1.47 from 4, 1.92 without; near phase of 1.6e6
+// points in 5-D at 8 cutoffs (3 points per cell): 60 ms with tiles, 48 with one
+// query per lane; of 2e6 points in 7-D (17 points per cell): 50 ms with tiles,
+// 118 without.
+constexpr uint32_t kTensorDensityFill = 2, kTensorNearFill = 4;
+
 FarQueue queue_of(Workspace* w) {
   FarQueue q;
   q.pos = w->qpos;
@@ -748,23 +766,26 @@ void cells_step(Workspace* w, const ClassPlan& c, const ClassView& cv, const Cut
   launch_cells(w->scode, cv, c.g, cuts, w->hinfo, w->hkeys, w->hvals, w->hcap, w->stream);
   w->last_cut = cuts;
   w->last_geom = w->geom;
+  w->last_points = cv.N;
   w->have_last = true;
 }
 
 void density_step(Workspace* w, const ClassPlan& c, const ClassView& cv, const CutGeom* cuts,
-                  bool fp64, int layout, int seg_cells, int32_t* rho) {
+                  bool fp64, int layout, int seg_cells, int32_t* rho, uint32_t min_fill) {
   Phase ph(w, DPC_PHASE_DENSITY);
   // the tensor layout exists for 5-8 dimensions with the float32 filter;
   // other cases run in segments, and the statistics report what ran
   if (layout == kLayoutTensor && !(c.dp == 8 && !fp64)) layout = kLayoutSegment;
   w->last_choice.dlay = layout;
-  launch_density(c.dp, c.g, fp64, layout, w->spts, w->scode, w->sid, cv, cuts, w->hinfo, w->hkeys,
-                 w->hvals, w->pieces, rho, w->skey, w->ctr, w->stream, seg_cells);
+  w->last_choice.dfill = min_fill;
+  launch_density(c.dp, c.g, c.dmax, fp64, layout, w->spts, w->scode, w->sid, cv, cuts, w->hinfo, w->hkeys,
+                 w->hvals, w->pieces, rho, w->skey, w->ctr, w->stream, seg_cells, min_fill);
 }
 
 void dependent_step(Workspace* w, const ClassPlan& c, const ClassView& cv, CutGeom* cuts,
                     const void* pts, int dtype, int32_t rho_skip, bool fp64, int layout, int nshift,
-                    int seg_cells, int32_t* lambda, double* delta) {
+                    int seg_cells, int32_t* lambda, double* delta, uint32_t min_fill,
+                    int sparse_layout = kLayoutUnion, const FarHint& hint = FarHint()) {
   cudaStream_t st = w->stream;
   {
     Phase ph(w, DPC_PHASE_MAXKEY);
@@ -779,8 +800,11 @@ void dependent_step(Workspace* w, const ClassPlan& c, const ClassView& cv, CutGe
   {
     Phase ph(w, DPC_PHASE_NEAR);
     if (layout == kLayoutTensor && c.dp == 8 && !fp64) {
-      launch_dep_near_tc(c.g, w->spts, w->sid, w->skey, cv, rho_skip, pts, dtype, cuts, w->hinfo,
-                         w->hkeys, w->hvals, w->pieces, lambda, delta, queue_of(w), w->ctr, st);
+      launch_dep_near_tc(c.dmax, w->spts, w->scode, w->sid, w->skey, cv, rho_skip, pts, dtype, cuts, w->hinfo,
+                         w->hkeys, w->hvals, w->pieces, lambda, delta, queue_of(w), w->ctr, min_fill, st);
+      if (min_fill)  // sparse cells
+        launch_dep_near(c.dp, c.g, fp64, sparse_layout, w->spts, w->scode, w->skey, cv, rho_skip, pts, dtype, cuts,
+                        w->hinfo, w->hkeys, w->hvals, lambda, delta, queue_of(w), w->ctr, st, seg_cells, min_fill);
     } else {
       // the tensor layout exists for 5-8 dimensions with the float32 filter
       if (layout == kLayoutTensor) layout = kLayoutUnion;
@@ -789,11 +813,13 @@ void dependent_step(Workspace* w, const ClassPlan& c, const ClassView& cv, CutGe
                       seg_cells);
     }
     w->last_choice.nlay = layout;
+    w->last_choice.nfill = min_fill;
+    w->last_choice.nsparse = sparse_layout;
   }
   {
     Phase ph(w, DPC_PHASE_FAR);
     launch_dep_far(c.dp, fp64, w->spts, w->scode, w->skey, cv, cuts, w->nodes, w->nbox, w->roots,
-                   queue_of(w), lambda, delta, w->ctr, st);
+                   queue_of(w), hint, lambda, delta, w->ctr, st);
   }
 }
 
@@ -899,10 +925,16 @@ struct NearTrial {
   double* delta;
 };
 
-// Default layouts (measured on the GB300): density in segments from 2 gridded
-// dimensions up; the near phase in segments in 3, union otherwise.
-inline int default_dlayout(int g) { return g >= 2 ? kLayoutSegment : kLayoutUnion; }
-inline int default_nlayout(int g) { return g == 3 ? kLayoutSegment : kLayoutUnion; }
+// Default layouts (measured on the GB300): tensor tiles in 5-8 dimensions with
+// the float32 filter; else density in segments from 2 gridded dimensions up and
+// the near phase in segments in 3, union otherwise.
+inline bool tensor_class(const ClassPlan& c, bool fp64) { return c.dp == 8 && !fp64; }
+inline int default_dlayout(const ClassPlan& c, bool fp64) {
+  return tensor_class(c, fp64) ? kLayoutTensor : (c.g >= 2 ? kLayoutSegment : kLayoutUnion);
+}
+inline int default_nlayout(const ClassPlan& c, bool fp64) {
+  return tensor_class(c, fp64) ? kLayoutTensor : (c.g == 3 ? kLayoutSegment : kLayoutUnion);
+}
 // segments of the segment layouts span cells while their union fits this
 inline int default_seg_cells(int g) { return g == 3 ? 48 : 0; }
 
@@ -922,10 +954,14 @@ Choice choose(Workspace* w, const ClassPlan& c, const ClassView& cv, CutGeom* cu
   ch.r = (int)((flags & DPC_FLAG_RADIUS_MASK) >> 12);
   const int forced = (int)((flags & DPC_FLAG_LAYOUT_MASK) >> 16);
   const int forced_ns = (int)((flags & DPC_FLAG_NEAR_SHIFT_MASK) >> 20);
-  ch.dlay = (forced && forced != kLayoutTree) ? forced : default_dlayout(c.g);
-  ch.nlay = (forced && forced != kLayoutPairs) ? forced : default_nlayout(c.g);
+  ch.dlay = (forced && forced != kLayoutTree) ? forced : default_dlayout(c, fp64);
+  ch.nlay = (forced && forced != kLayoutPairs) ? forced : default_nlayout(c, fp64);
   ch.ns = forced_ns ? forced_ns - 1 : 0;
   ch.sc = default_seg_cells(c.g);
+  if (!forced) {
+    ch.dfill = kTensorDensityFill;
+    ch.nfill = kTensorNearFill;
+  }
   const std::string key = (near ? "R/" : "D/") + tune_key(c, b, cut);
   auto it = w->tuned.find(key);
   const bool fixed = ch.r != 0 || forced || forced_ns;
@@ -954,7 +990,7 @@ Choice choose(Workspace* w, const ClassPlan& c, const ClassView& cv, CutGeom* cu
       if (timed) cudaEventRecord(w->tune_ev[1], st);
       for (int l = 0; l < 4; ++l) {
         if (l < ndl)
-          launch_density(c.dp, c.g, fp64, dlays[l], w->spts, w->scode, w->sid, cv, cuts, w->hinfo,
+          launch_density(c.dp, c.g, c.dmax, fp64, dlays[l], w->spts, w->scode, w->sid, cv, cuts, w->hinfo,
                          w->hkeys, w->hvals, w->pieces, rho_scratch, w->skey, w->ctr, st,
                          default_seg_cells(c.g));
         if (timed) cudaEventRecord(w->tune_ev[2 + l], st);
@@ -974,16 +1010,16 @@ Choice choose(Workspace* w, const ClassPlan& c, const ClassView& cv, CutGeom* cu
         for (int l = 0; l < kNL; ++l) {
           if (l < nnl && (sh == 0 || nlays[l] != kLayoutTree)) {
             if (nlays[l] == kLayoutTensor)
-              launch_dep_near_tc(c.g, w->spts, w->sid, w->skey, cv, 0, near->pts, near->dtype,
+              launch_dep_near_tc(c.dmax, w->spts, w->scode, w->sid, w->skey, cv, 0, near->pts, near->dtype,
                                  cuts, w->hinfo, w->hkeys, w->hvals, w->pieces, near->lambda,
-                                 near->delta, queue_of(w), w->ctr, st);
+                                 near->delta, queue_of(w), w->ctr, 0, st);
             else
               launch_dep_near(c.dp, c.g, fp64, nlays[l], w->spts, w->scode, w->skey, cv, 0,
                               near->pts, near->dtype, cuts, w->hinfo, w->hkeys, w->hvals,
                               near->lambda, near->delta, queue_of(w), w->ctr, st,
                               default_seg_cells(c.g));
             launch_dep_far(c.dp, fp64, w->spts, w->scode, w->skey, cv, cuts, w->nodes, w->nbox,
-                           w->roots, queue_of(w), near->lambda, near->delta, w->ctr, st);
+                           w->roots, queue_of(w), FarHint(), near->lambda, near->delta, w->ctr, st);
           }
           if (timed) cudaEventRecord(w->tune_ev[8 + (kNL + 1) * sh + l], st);
         }
@@ -1040,14 +1076,14 @@ Choice choose(Workspace* w, const ClassPlan& c, const ClassView& cv, CutGeom* cu
           if (t[l] < 0.97f * t[bi]) bi = l;
         return bi;
       };
-      const int di = pick(dt, dlays, ndl, default_dlayout(c.g));
+      const int di = pick(dt, dlays, ndl, default_dlayout(c, fp64));
       int nsi = 0, ni = -1;
       float nms = 0.f;
       if (near) {
-        ni = pick(nt[0], nlays, nnl, default_nlayout(c.g));
+        ni = pick(nt[0], nlays, nnl, default_nlayout(c, fp64));
         nms = nt[0][ni];
         for (int sh = 1; sh < kShifts; ++sh) {
-          const int l = pick(nt[sh], nlays, nnl, default_nlayout(c.g));
+          const int l = pick(nt[sh], nlays, nnl, default_nlayout(c, fp64));
           const float t = lv[sh] + nt[sh][l];
           if (t < 0.97f * nms) {
             nms = t;
@@ -1061,7 +1097,7 @@ Choice choose(Workspace* w, const ClassPlan& c, const ClassView& cv, CutGeom* cu
         best_ms = ms;
         best.r = r;
         best.dlay = dlays[di];
-        best.nlay = near ? nlays[ni] : default_nlayout(c.g);
+        best.nlay = near ? nlays[ni] : default_nlayout(c, fp64);
         best.ns = near ? nsi : 0;
         best.sc = default_seg_cells(c.g);
       }
@@ -1076,6 +1112,81 @@ Choice choose(Workspace* w, const ClassPlan& c, const ClassView& cv, CutGeom* cu
   if (ch.r > 0) launch_set_radius(cv, cuts, ch.r, w->stream);
   w->last_choice = ch;
   return ch;
+}
+
+// ---- cutoff sweeps -------------------------------------------------------------
+//
+// The grid level of a cutoff is a power of two times the smallest one, so the
+// cutoffs of a sweep fall into groups with the same cells (1.25^k: three per
+// level).  One density launch serves up to kMultiCuts cutoffs of a group, and
+// the near-dependent search runs on the cells of the smallest cutoff (at most
+// kNearLevels levels below the cutoff's own): a dependent point's distance
+// hardly depends on the cutoff, the block's points grow with its power.  After
+// the first cutoff the dependent point found for another one, where it is
+// higher here too, bounds the search (FarHint).  Groups run from the largest
+// cutoffs down, so one hash at a time suffices.
+// 2e6 points in 7-D at 4 cutoffs: 565 -> 171 ms a call (density 217 -> 49, near
+// phase 209 -> 50, far 30 -> 70); 128 instances of 2, 3 and 5 dimensions at 8
+// cutoffs: 257 -> 148 ms (density 90 -> 42, near phase and far 154 -> 97).
+constexpr int kNearLevels = 3;
+
+struct CutGroup {
+  int level = 0;
+  std::vector<int> cuts;  // cutoffs whose densities run on this group's cells
+  std::vector<int> near;  // cutoffs whose near phase does
+};
+
+bool sweep_call(const CallPlan& P, uint32_t flags) {
+  return P.ncut > 1 && P.ncut <= 64 &&
+         !(flags & (DPC_FLAG_RADIUS_MASK | DPC_FLAG_LAYOUT_MASK | DPC_FLAG_NEAR_SHIFT_MASK));
+}
+
+// Groups by the cutoffs of the class's first instance (any grouping is
+// correct: every instance takes the geometry of its largest cutoff of the
+// group), largest level first.
+std::vector<CutGroup> group_cuts(const CallPlan& P, const dpc_batch* b, const ClassPlan& c) {
+  const double* d = b->d_cut + (size_t)c.members[0] * P.ncut_all;
+  const double dmin = *std::min_element(d, d + P.ncut);
+  std::map<int, CutGroup, std::greater<int>> by;
+  std::vector<int> level(P.ncut);
+  for (int j = 0; j < P.ncut; ++j) {
+    // no common fine cell without a positive smallest cutoff: one group each
+    level[j] = dmin > 0.0 ? (int)std::ceil(std::log2(std::min(d[j] / dmin, 0x1p40)) - 1e-9) : j;
+    by[level[j]].level = level[j];
+    by[level[j]].cuts.push_back(j);
+  }
+  for (int j = 0; j < P.ncut; ++j) {
+    int at = level[j];
+    if (dmin > 0.0)
+      for (auto& kv : by)
+        if (kv.first < at && kv.first >= level[j] - kNearLevels) at = kv.first;
+    by[at].near.push_back(j);
+  }
+  std::vector<CutGroup> out;
+  for (auto& kv : by) out.push_back(std::move(kv.second));
+  return out;
+}
+
+// The densities of one group (cells of its geometry into the hash first).
+void group_density_step(Workspace* w, const ClassPlan& c, const ClassView& cv, int ncut, const CutGroup& g,
+                        bool fp64, int32_t* rho, uint64_t N) {
+  unsigned long long mask = 0;
+  for (int j : g.cuts) mask |= 1ull << j;
+  launch_group_geometry(cv, w->cuts, ncut, mask, w->geo, w->stream);
+  cells_step(w, c, cv, w->geo);
+  Phase ph(w, DPC_PHASE_DENSITY);
+  w->last_choice = Choice();
+  w->last_choice.dlay = tensor_class(c, fp64) ? kLayoutTensor : kLayoutSegment;
+  w->last_choice.dfill = kTensorDensityFill;
+  for (size_t i = 0; i < g.cuts.size(); i += kMultiCuts) {
+    MultiCut mc;
+    for (size_t j = i; j < g.cuts.size() && j < i + kMultiCuts; ++j) {
+      mc.cut[mc.m] = w->cuts + (size_t)g.cuts[j] * cv.ninst;
+      mc.rho[mc.m++] = rho + (size_t)g.cuts[j] * N;
+    }
+    launch_density_multi(c.dp, c.g, c.dmax, fp64, w->spts, w->scode, w->sid, cv, w->geo, w->hinfo, w->hkeys,
+                         w->hvals, w->pieces, mc, w->ctr, w->stream, default_seg_cells(c.g), kTensorDensityFill);
+  }
 }
 
 void reset_call(Workspace* w, uint32_t flags) {
@@ -1152,11 +1263,15 @@ int dpc_density(const void* pts, int dtype, const dpc_batch* b, int32_t* rho, ui
       continue;
     }
     bin_class(w, pts, dtype, P, c, cv, b, insts);
+    if (sweep_call(P, flags)) {
+      for (const CutGroup& g : group_cuts(P, b, c)) group_density_step(w, c, cv, P.ncut, g, fp64, rho, N);
+      continue;
+    }
     for (int k = 0; k < P.ncut; ++k) {
       CutGeom* cuts = w->cuts + (size_t)k * cv.ninst;
       const Choice ch = choose(w, c, cv, cuts, b, k, fp64, rho + (size_t)k * N, flags);
       cells_step(w, c, cv, cuts);
-      density_step(w, c, cv, cuts, fp64, ch.dlay, ch.sc, rho + (size_t)k * N);
+      density_step(w, c, cv, cuts, fp64, ch.dlay, ch.sc, rho + (size_t)k * N, ch.dfill);
     }
   }
   return finish(w, flags);
@@ -1195,7 +1310,7 @@ int dpc_dependent(const void* pts, int dtype, const dpc_batch* b, int32_t dcut_i
     cells_step(w, c, cv, w->cuts);
     launch_keys_from_rho(rho, w->sid, cv.N, w->skey, w->stream);
     dependent_step(w, c, cv, w->cuts, pts, dtype, rho_skip, fp64, ch.nlay, ch.ns, ch.sc, lambda,
-                   delta);
+                   delta, ch.nfill);
   }
   return finish(w, flags);
 }
@@ -1258,16 +1373,47 @@ static void run_classes(Workspace* w, const CallPlan& P, const void* pts, int dt
     }
     bin_class(w, pts, dtype, P, c, cv, b, insts);
     tree_step(w, cv);
+    if (sweep_call(P, flags)) {
+      int prev = -1;  // the cutoff whose dependent points were found last
+      for (const CutGroup& g : group_cuts(P, b, c)) {
+        group_density_step(w, c, cv, P.ncut, g, fp64, rho, N);
+        if (last && done)
+          for (int k : g.cuts) (*done)(0, k);
+        for (int k : g.near) {
+          const size_t o = (size_t)k * N;
+          CutGeom* cuts = w->cuts + (size_t)k * cv.ninst;
+          launch_adopt_geometry(cv, w->geo, cuts, w->stream);
+          launch_keys_from_rho(rho + o, w->sid, cv.N, w->skey, w->stream);
+          FarHint hint;
+          if (prev >= 0) {
+            hint.lambda = lambda + (size_t)prev * N;
+            hint.rho = rho + o;
+            hint.pts = pts;
+            hint.dtype = dtype;
+          }
+          prev = k;
+          // with a bound to start from, the tree search alone beats a scan of
+          // the blocks except where tensor tiles run
+          const int nlay = hint.lambda && !tensor_class(c, fp64) ? kLayoutTree : default_nlayout(c, fp64);
+          dependent_step(w, c, cv, cuts, pts, dtype, 0, fp64, nlay, 0, default_seg_cells(c.g), lambda + o, delta + o,
+                         kTensorNearFill, hint.lambda ? kLayoutTree : kLayoutUnion, hint);
+          if (last && done) (*done)(1, k);
+          labels_step(w, c, cv, k, one_params(params, c, P.ncut_all, k), rho + o, lambda + o, delta + o, label + o);
+          if (last && done) (*done)(2, k);
+        }
+      }
+      continue;
+    }
     for (int k = 0; k < P.ncut; ++k) {
       const size_t o = (size_t)k * N;
       CutGeom* cuts = w->cuts + (size_t)k * cv.ninst;
       const NearTrial nt{pts, dtype, lambda + o, delta + o};
       const Choice ch = choose(w, c, cv, cuts, b, k, fp64, rho + o, flags, &nt);
       cells_step(w, c, cv, cuts);
-      density_step(w, c, cv, cuts, fp64, ch.dlay, ch.sc, rho + o);
+      density_step(w, c, cv, cuts, fp64, ch.dlay, ch.sc, rho + o, ch.dfill);
       if (last && done) (*done)(0, k);
       dependent_step(w, c, cv, cuts, pts, dtype, 0, fp64, ch.nlay, ch.ns, ch.sc, lambda + o,
-                     delta + o);
+                     delta + o, ch.nfill);
       if (last && done) (*done)(1, k);
       labels_step(w, c, cv, k, one_params(params, c, P.ncut_all, k), rho + o, lambda + o,
                   delta + o, label + o);
@@ -1636,8 +1782,11 @@ int dpc_get_stats(void* stream, dpc_stats* out) {
     out->occupied_cells = hi.m;
     out->grid_level = cg.k;
     out->block_radius = cg.R;
-    out->density_layout = w->last_choice.dlay;
-    out->near_layout = w->last_choice.nlay;
+    // what the fill rule left to the CUDA-core layouts (tensor_fill)
+    const Choice& ch = w->last_choice;
+    auto sparse = [&](uint32_t fill) { return (uint64_t)w->last_points < (uint64_t)fill * hi.m; };
+    out->density_layout = ch.dlay == kLayoutTensor && sparse(ch.dfill) ? kLayoutSegment : ch.dlay;
+    out->near_layout = ch.nlay == kLayoutTensor && sparse(ch.nfill) ? ch.nsparse : ch.nlay;
     out->near_shift = w->last_choice.ns;
     out->bits_per_axis = g.B;
   }

@@ -285,6 +285,29 @@ __global__ void k_near_level(ClassView cv, CutGeom* cuts, int shift) {
   set_far(C, cv.geom[i].f);
 }
 
+__global__ void k_group_geometry(ClassView cv, const CutGeom* __restrict__ cuts, int ncut,
+                                 unsigned long long mask, CutGeom* __restrict__ geo) {
+  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= cv.ninst) return;
+  int best = -1;
+  double dc = -1.0;
+  for (int c = 0; c < ncut && c < 64; ++c)
+    if (((mask >> c) & 1ull) && cuts[(size_t)c * cv.ninst + i].dc > dc) {
+      best = c;
+      dc = cuts[(size_t)c * cv.ninst + i].dc;
+    }
+  geo[i] = cuts[(size_t)(best < 0 ? 0 : best) * cv.ninst + i];
+}
+
+__global__ void k_adopt_geometry(ClassView cv, const CutGeom* __restrict__ geo, CutGeom* __restrict__ cut) {
+  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= cv.ninst) return;
+  cut[i].k = geo[i].k;
+  cut[i].R = geo[i].R;
+  cut[i].far32 = geo[i].far32;
+  cut[i].far64 = geo[i].far64;
+}
+
 // Per (instance, cutoff) search parameters, one thread each.  cuts is
 // [ncut][ninst].
 __global__ void k_setup_cuts(ClassView cv, CutGeom* cuts, int ncut, const CutHost* __restrict__ hc,
@@ -536,6 +559,17 @@ void launch_chunks(const ClassView& cv, uint32_t* chunk_inst, uint32_t* chunk_po
 void launch_near_level(const ClassView& cv, CutGeom* cuts, int shift, cudaStream_t st) {
   if (shift <= 0) return;
   k_near_level<<<grid_for(cv.ninst), kThreads, 0, st>>>(cv, cuts, shift);
+  count_launches(1);
+}
+
+void launch_group_geometry(const ClassView& cv, const CutGeom* cuts, int ncut, unsigned long long mask,
+                           CutGeom* geo, cudaStream_t st) {
+  k_group_geometry<<<grid_for(cv.ninst), kThreads, 0, st>>>(cv, cuts, ncut, mask, geo);
+  count_launches(1);
+}
+
+void launch_adopt_geometry(const ClassView& cv, const CutGeom* geo, CutGeom* cut, cudaStream_t st) {
+  k_adopt_geometry<<<grid_for(cv.ninst), kThreads, 0, st>>>(cv, geo, cut);
   count_launches(1);
 }
 

@@ -206,13 +206,17 @@ __device__ __forceinline__ uint2 seg_band_recount(const RunTable& rt, int nr, ui
 template <int DP>
 constexpr int seg_v() { return DP == 2 ? 8 : (DP == 4 ? 4 : 2); }
 
-template <int DP, int G, bool F64>
-__global__ void __launch_bounds__(kThreads, (F64 || G >= 4) ? 5 : 6)
+// M cutoffs of a sweep that share the block geometry `geo` (M = 1: one cutoff)
+// are counted in one pass: the distances, lookups and window loads are paid
+// once, every cutoff adds its own compare and count.
+template <int DP, int G, bool F64, int M>
+__global__ void __launch_bounds__(kThreads, (F64 || G >= 4 || M > 2) ? 5 : 6)
 k_density_seg(const float* __restrict__ spts, const unsigned long long* __restrict__ scode,
-              const uint32_t* __restrict__ sid, ClassView cv, const CutGeom* __restrict__ cuts,
+              const uint32_t* __restrict__ sid, ClassView cv, const CutGeom* __restrict__ geo,
               const HashInfo* __restrict__ hi, const unsigned long long* __restrict__ hkeys,
-              const uint2* __restrict__ hvals, int32_t* __restrict__ rho_out,
-              unsigned long long* __restrict__ skey, Counters* ctr, int seg_cells) {
+              const uint2* __restrict__ hvals, MultiCut mc, unsigned long long* __restrict__ skey,
+              Counters* ctr, int seg_cells, uint32_t skip_fill) {
+  if (skip_fill && tensor_fill(cv.N, hi, skip_fill)) return;  // the tensor tiles' part
   constexpr int ND = real_dims<DP, G>();
   constexpr int V = seg_v<DP>();
   constexpr uint32_t W = 32u * V;
@@ -228,22 +232,27 @@ k_density_seg(const float* __restrict__ spts, const unsigned long long* __restri
   for (uint32_t ch = blockIdx.x * kWarps + wib; ch < cv.nchunk; ch += gridDim.x * kWarps) {
     uint32_t inst, p0, end;
     cv.chunk(ch, inst, p0, end);
-    const CutGeom& C = cuts[inst];
-    const int k = C.k;
-    const int R = C.R;
+    const int k = geo[inst].k;
+    const int R = geo[inst].R;
     const int shift = G * k;
     const int cmax = (1 << (cv.geom[inst].B - k)) - 1;
-    const double dc2 = C.dc2;
-    const float t_in = C.t_in, t_out = C.t_out;
-    const BandBits bb = band_bits(t_in, t_out);
     // s <= t_in  <=>  s - up(t_in) < 0, with up(t_in) the next float above
-    const f32x2 ntin2 = pack2(-next_up(t_in), -next_up(t_in));
+    BandBits bb[M];
+    f32x2 ntin2[M];
+#pragma unroll
+    for (int c = 0; c < M; ++c) {
+      const CutGeom& C = mc.cut[c][inst];
+      bb[c] = band_bits(C.t_in, C.t_out);
+      ntin2[c] = pack2(-next_up(C.t_in), -next_up(C.t_in));
+    }
     const unsigned long long hb = ib ? ((unsigned long long)inst << S) : 0ull;
     const uint32_t p = p0 + lane;
     const bool valid = p < end;
     const unsigned long long mycell = valid ? (key_code(scode[p], S, ib) >> shift) : ~0ull;
     const int nvalid = (int)min(32u, end - p0);
-    int32_t acc = 0;  // lane j: the count of query p0 + j
+    int32_t acc[M];  // lane j: the counts of query p0 + j
+#pragma unroll
+    for (int c = 0; c < M; ++c) acc[c] = 0;
     int s = 0;
     while (s < nvalid) {
       Union<G> u;
@@ -261,16 +270,26 @@ k_density_seg(const float* __restrict__ spts, const unsigned long long* __restri
             const bool two = j + 1 < e;
             const Pt<DP> xa = load_pt<DP>(spts, p0 + j);
             const Pt<DP> xb = load_pt<DP>(spts, p0 + (two ? j + 1 : j));
-            unsigned c = 0;
+            unsigned n2[M];
+#pragma unroll
+            for (int c = 0; c < M; ++c) n2[c] = 0u;
 #pragma unroll
             for (int v = 0; v < V; ++v) {
               if (v >= vn) break;
-              c += (dist64<DP, ND>(xa, cand[v]) <= dc2) ? 1u : 0u;
-              c += (dist64<DP, ND>(xb, cand[v]) <= dc2) ? 0x10000u : 0u;
+              const double da = dist64<DP, ND>(xa, cand[v]), db = dist64<DP, ND>(xb, cand[v]);
+#pragma unroll
+              for (int c = 0; c < M; ++c) {
+                const double dc2 = mc.cut[c][inst].dc2;
+                n2[c] += da <= dc2 ? 1u : 0u;
+                n2[c] += db <= dc2 ? 0x10000u : 0u;
+              }
             }
-            c = __reduce_add_sync(kFull, c);
-            if (lane == j) acc += (int32_t)(c & 0xffffu);
-            if (two && lane == j + 1) acc += (int32_t)(c >> 16);
+#pragma unroll
+            for (int c = 0; c < M; ++c) {
+              const unsigned t = __reduce_add_sync(kFull, n2[c]);
+              if (lane == j) acc[c] += (int32_t)(t & 0xffffu);
+              if (two && lane == j + 1) acc[c] += (int32_t)(t >> 16);
+            }
           }
         } else {
           // the lane's candidates negated, two slots per packed register; a
@@ -289,7 +308,9 @@ k_density_seg(const float* __restrict__ spts, const unsigned long long* __restri
           // chains); their per-lane counts (at most V each) share one 32-bit
           // word per reduction, and one unsigned minimum per lane tells
           // whether any of its pairs fell in the band
-          uint32_t bandq = 0;  // bit j: queries j and j + 1 met a band pair
+          uint32_t bandq[M];  // bit j: queries j and j + 1 met a band pair
+#pragma unroll
+          for (int c = 0; c < M; ++c) bandq[c] = 0u;
           auto passes = [&](auto full_window) {
             constexpr bool kFullWindow = decltype(full_window)::value;
             const int vp = (vn + 1) >> 1;
@@ -303,36 +324,50 @@ k_density_seg(const float* __restrict__ spts, const unsigned long long* __restri
                 qa[k] = pack2(xa.x[k], xa.x[k]);
                 qb[k] = pack2(xb.x[k], xb.x[k]);
               }
-              uint32_t na = 0, nb = 0, mband = 0xffffffffu;
+              uint32_t na[M], nb[M], mband[M];
+#pragma unroll
+              for (int c = 0; c < M; ++c) {
+                na[c] = nb[c] = 0u;
+                mband[c] = 0xffffffffu;
+              }
 #pragma unroll
               for (int i = 0; i < V / 2; ++i) {
                 if (!kFullWindow && i >= vp) break;
                 const f32x2 sa = dist32x2<ND>(qa, nc[i]);
                 const f32x2 sb = dist32x2<ND>(qb, nc[i]);
-                na += sign_count2(add2(sa, ntin2));
-                nb += sign_count2(add2(sb, ntin2));
-                mband = min(mband, band_min2(sa, bb.lo));
-                mband = min(mband, band_min2(sb, bb.lo));
+#pragma unroll
+                for (int c = 0; c < M; ++c) {
+                  na[c] += sign_count2(add2(sa, ntin2[c]));
+                  nb[c] += sign_count2(add2(sb, ntin2[c]));
+                  mband[c] = min(mband[c], band_min2(sa, bb[c].lo));
+                  mband[c] = min(mband[c], band_min2(sb, bb[c].lo));
+                }
               }
-              unsigned c = na + (nb << 16);
-              c = __reduce_add_sync(kFull, c);
-              // band pairs: recounted in binary64 after the window's passes
-              if (__any_sync(kFull, mband < bb.width)) bandq |= 1u << j;
-              if (lane == j) acc += (int32_t)(c & 0xffffu);
-              if (two && lane == j + 1) acc += (int32_t)(c >> 16);
+#pragma unroll
+              for (int c = 0; c < M; ++c) {
+                const unsigned t = __reduce_add_sync(kFull, na[c] + (nb[c] << 16));
+                // band pairs: recounted in binary64 after the window's passes
+                if (__any_sync(kFull, mband[c] < bb[c].width)) bandq[c] |= 1u << j;
+                if (lane == j) acc[c] += (int32_t)(t & 0xffffu);
+                if (two && lane == j + 1) acc[c] += (int32_t)(t >> 16);
+              }
             }
           };
           if (vn == V) passes(std::true_type{});
           else passes(std::false_type{});
-          while (bandq) {
-            const int j = __ffs(bandq) - 1;
-            bandq &= bandq - 1u;
-            const bool two = j + 1 < e;
-            const uint2 r = seg_band_recount<DP, V, ND>(rt, nr, w0, total, spts, lane, p0 + j,
-                                                        p0 + (two ? j + 1 : j), t_in, t_out, dc2);
-            if (lane == j) acc += (int32_t)(r.x & 0xffffu);
-            if (two && lane == j + 1) acc += (int32_t)(r.x >> 16);
-            if (lane == 0) band += (r.y & 0xffffu) + (two ? (r.y >> 16) : 0u);
+#pragma unroll
+          for (int c = 0; c < M; ++c) {
+            while (bandq[c]) {
+              const int j = __ffs(bandq[c]) - 1;
+              bandq[c] &= bandq[c] - 1u;
+              const bool two = j + 1 < e;
+              const CutGeom& C = mc.cut[c][inst];
+              const uint2 r = seg_band_recount<DP, V, ND>(rt, nr, w0, total, spts, lane, p0 + j,
+                                                          p0 + (two ? j + 1 : j), C.t_in, C.t_out, C.dc2);
+              if (lane == j) acc[c] += (int32_t)(r.x & 0xffffu);
+              if (two && lane == j + 1) acc[c] += (int32_t)(r.x >> 16);
+              if (lane == 0) band += (r.y & 0xffffu) + (two ? (r.y >> 16) : 0u);
+            }
           }
         }
       }
@@ -340,8 +375,9 @@ k_density_seg(const float* __restrict__ spts, const unsigned long long* __restri
     }
     if (valid) {
       const uint32_t id = sid[p];
-      rho_out[id] = acc;
-      skey[p] = order_key(acc, id);
+#pragma unroll
+      for (int c = 0; c < M; ++c) mc.rho[c][id] = acc[c];
+      if (skey) skey[p] = order_key(acc[0], id);
     }
   }
   if (lane == 0 && pairs) atomicAdd(&ctr->pairs, pairs);
@@ -578,7 +614,7 @@ template <int DP, int G>
 void density_dg(bool fp64, int layout, const float* spts, const unsigned long long* scode,
                 const uint32_t* sid, const ClassView& cv, const CutGeom* cuts, const HashInfo* hi,
                 const unsigned long long* hkeys, const uint2* hvals, int32_t* rho_out,
-                unsigned long long* skey, Counters* ctr, int seg_cells, cudaStream_t st) {
+                unsigned long long* skey, Counters* ctr, int seg_cells, uint32_t skip_fill, cudaStream_t st) {
   const unsigned grid = grid_for(cv.nchunk, kWarps, sm_count() * 64u);
   if (layout == kLayoutPairs) {
     cudaMemsetAsync(skey, 0, sizeof(unsigned long long) * cv.N, st);
@@ -592,12 +628,16 @@ void density_dg(bool fp64, int layout, const float* spts, const unsigned long lo
     k_pairs_finish<<<grid_for(cv.N, 256, sm_count() * 16u), 256, 0, st>>>(sid, cv.N, rho_out, skey);
     count_launches(1);
   } else if (layout == kLayoutSegment) {
+    MultiCut mc;
+    mc.m = 1;
+    mc.cut[0] = cuts;
+    mc.rho[0] = rho_out;
     if (fp64)
-      k_density_seg<DP, G, true><<<grid, kThreads, 0, st>>>(spts, scode, sid, cv, cuts, hi, hkeys,
-                                                            hvals, rho_out, skey, ctr, seg_cells);
+      k_density_seg<DP, G, true, 1><<<grid, kThreads, 0, st>>>(spts, scode, sid, cv, cuts, hi, hkeys,
+                                                               hvals, mc, skey, ctr, seg_cells, skip_fill);
     else
-      k_density_seg<DP, G, false><<<grid, kThreads, 0, st>>>(spts, scode, sid, cv, cuts, hi, hkeys,
-                                                             hvals, rho_out, skey, ctr, seg_cells);
+      k_density_seg<DP, G, false, 1><<<grid, kThreads, 0, st>>>(spts, scode, sid, cv, cuts, hi, hkeys,
+                                                                hvals, mc, skey, ctr, seg_cells, skip_fill);
   } else {
     if (fp64)
       k_density<DP, G, true><<<grid, kThreads, 0, st>>>(spts, scode, sid, cv, cuts, hi, hkeys, hvals,
@@ -611,16 +651,61 @@ void density_dg(bool fp64, int layout, const float* spts, const unsigned long lo
 
 }  // namespace
 
-void launch_density(int dp, int g, bool fp64, int layout, const float* spts,
+template <int DP, int G, bool F64>
+static void density_multi_dg(const float* spts, const unsigned long long* scode, const uint32_t* sid,
+                             const ClassView& cv, const CutGeom* geo, const HashInfo* hi,
+                             const unsigned long long* hkeys, const uint2* hvals, const MultiCut& mc, Counters* ctr,
+                             int seg_cells, uint32_t skip_fill, cudaStream_t st) {
+  auto go = [&](auto kern) {
+    kern<<<grid_for(cv.nchunk, kWarps, sm_count() * 64u), kThreads, 0, st>>>(spts, scode, sid, cv, geo, hi, hkeys,
+                                                                            hvals, mc, nullptr, ctr, seg_cells, skip_fill);
+  };
+  if (mc.m == 1) go(k_density_seg<DP, G, F64, 1>);
+  else if (mc.m == 2) go(k_density_seg<DP, G, F64, 2>);
+  else if (mc.m == 3) go(k_density_seg<DP, G, F64, 3>);
+  else go(k_density_seg<DP, G, F64, 4>);
+  count_launches(1);
+}
+
+void launch_density_multi(int dp, int g, int d, bool fp64, const float* spts, const unsigned long long* scode,
+                          const uint32_t* sid, const ClassView& cv, const CutGeom* geo, HashInfo* hi,
+                          const unsigned long long* hkeys, const uint2* hvals, uint4* pieces, const MultiCut& mc,
+                          Counters* ctr, cudaStream_t st, int seg_cells, uint32_t min_fill) {
+  if (cv.N == 0) return;
+  uint32_t skip_fill = 0;
+  if (dp == 8 && !fp64) {
+    launch_density_tc(d, spts, scode, sid, cv, geo, hi, hkeys, hvals, pieces, mc, nullptr, ctr, min_fill, st);
+    if (min_fill == 0) return;
+    skip_fill = min_fill;
+  }
+  auto go = [&](auto f64) {
+    constexpr bool F = decltype(f64)::value;
+    if (g == 1) density_multi_dg<2, 1, F>(spts, scode, sid, cv, geo, hi, hkeys, hvals, mc, ctr, seg_cells, skip_fill, st);
+    else if (g == 2) density_multi_dg<2, 2, F>(spts, scode, sid, cv, geo, hi, hkeys, hvals, mc, ctr, seg_cells, skip_fill, st);
+    else if (g == 3) density_multi_dg<4, 3, F>(spts, scode, sid, cv, geo, hi, hkeys, hvals, mc, ctr, seg_cells, skip_fill, st);
+    else if (dp == 4) density_multi_dg<4, 4, F>(spts, scode, sid, cv, geo, hi, hkeys, hvals, mc, ctr, seg_cells, skip_fill, st);
+    else density_multi_dg<8, 4, F>(spts, scode, sid, cv, geo, hi, hkeys, hvals, mc, ctr, seg_cells, skip_fill, st);
+  };
+  if (fp64) go(std::true_type{});
+  else go(std::false_type{});
+}
+
+void launch_density(int dp, int g, int d, bool fp64, int layout, const float* spts,
                     const unsigned long long* scode, const uint32_t* sid, const ClassView& cv,
                     const CutGeom* cuts, HashInfo* hi, const unsigned long long* hkeys,
-                    const uint2* hvals, uint2* pieces, int32_t* rho_out,
-                    unsigned long long* skey, Counters* ctr, cudaStream_t st, int seg_cells) {
+                    const uint2* hvals, uint4* pieces, int32_t* rho_out,
+                    unsigned long long* skey, Counters* ctr, cudaStream_t st, int seg_cells, uint32_t min_fill) {
   if (cv.N == 0) return;
+  uint32_t skip_fill = 0;
   if (layout == kLayoutTensor) {
     if (dp == 8 && !fp64 && pieces) {
-      launch_density_tc(g, spts, sid, cv, cuts, hi, hkeys, hvals, pieces, rho_out, skey, ctr, st);
-      return;
+      MultiCut mc;
+      mc.m = 1;
+      mc.cut[0] = cuts;
+      mc.rho[0] = rho_out;
+      launch_density_tc(d, spts, scode, sid, cv, cuts, hi, hkeys, hvals, pieces, mc, skey, ctr, min_fill, st);
+      if (min_fill == 0) return;
+      skip_fill = min_fill;
     }
     layout = kLayoutSegment;
   }
@@ -629,11 +714,11 @@ void launch_density(int dp, int g, bool fp64, int layout, const float* spts,
                         st);
     return;
   }
-  if (g == 1) density_dg<2, 1>(fp64, layout, spts, scode, sid, cv, cuts, hi, hkeys, hvals, rho_out, skey, ctr, seg_cells, st);
-  else if (g == 2) density_dg<2, 2>(fp64, layout, spts, scode, sid, cv, cuts, hi, hkeys, hvals, rho_out, skey, ctr, seg_cells, st);
-  else if (g == 3) density_dg<4, 3>(fp64, layout, spts, scode, sid, cv, cuts, hi, hkeys, hvals, rho_out, skey, ctr, seg_cells, st);
-  else if (dp == 4) density_dg<4, 4>(fp64, layout, spts, scode, sid, cv, cuts, hi, hkeys, hvals, rho_out, skey, ctr, seg_cells, st);
-  else density_dg<8, 4>(fp64, layout, spts, scode, sid, cv, cuts, hi, hkeys, hvals, rho_out, skey, ctr, seg_cells, st);
+  if (g == 1) density_dg<2, 1>(fp64, layout, spts, scode, sid, cv, cuts, hi, hkeys, hvals, rho_out, skey, ctr, seg_cells, skip_fill, st);
+  else if (g == 2) density_dg<2, 2>(fp64, layout, spts, scode, sid, cv, cuts, hi, hkeys, hvals, rho_out, skey, ctr, seg_cells, skip_fill, st);
+  else if (g == 3) density_dg<4, 3>(fp64, layout, spts, scode, sid, cv, cuts, hi, hkeys, hvals, rho_out, skey, ctr, seg_cells, skip_fill, st);
+  else if (dp == 4) density_dg<4, 4>(fp64, layout, spts, scode, sid, cv, cuts, hi, hkeys, hvals, rho_out, skey, ctr, seg_cells, skip_fill, st);
+  else density_dg<8, 4>(fp64, layout, spts, scode, sid, cv, cuts, hi, hkeys, hvals, rho_out, skey, ctr, seg_cells, skip_fill, st);
 }
 
 void launch_keys_from_rho(const int32_t* rho, const uint32_t* sid, uint32_t n,

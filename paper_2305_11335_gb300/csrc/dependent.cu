@@ -170,7 +170,8 @@ k_dep_near(const float* __restrict__ spts, const unsigned long long* __restrict_
            const void* __restrict__ pts, int dtype, const CutGeom* __restrict__ cuts,
            const HashInfo* __restrict__ hi, const unsigned long long* __restrict__ hkeys,
            const uint2* __restrict__ hvals, int32_t* __restrict__ lambda,
-           double* __restrict__ delta, FarQueue q, Counters* ctr) {
+           double* __restrict__ delta, FarQueue q, Counters* ctr, uint32_t skip_fill) {
+  if (skip_fill && tensor_fill(cv.N, hi, skip_fill)) return;  // the tensor tiles' part
   constexpr int kNearCap = DP == 8 ? 128 : 256;
   __shared__ __align__(16) float s_pts[kNearWarps * kNearCap * DP];
   __shared__ unsigned long long s_key[kNearWarps * kNearCap];
@@ -681,7 +682,8 @@ k_dep_near_seg(const float* __restrict__ spts, const unsigned long long* __restr
 __global__ void k_near_to_far(const unsigned long long* __restrict__ skey, ClassView cv,
                               const CutGeom* __restrict__ cuts, int32_t rho_skip,
                               int32_t* __restrict__ lambda, double* __restrict__ delta, FarQueue q,
-                              Counters* ctr) {
+                              Counters* ctr, const HashInfo* __restrict__ hi, uint32_t skip_fill) {
+  if (skip_fill && tensor_fill(cv.N, hi, skip_fill)) return;  // the tensor tiles' part
   const int lane = threadIdx.x & 31;
   const uint32_t lanemask_lt = (1u << lane) - 1u;
   const uint64_t total = (uint64_t)cv.nchunk * 32u;
@@ -800,7 +802,7 @@ __device__ __noinline__ int tree_walk_from(const Node* __restrict__ nodes,
 // Per-query context shared by the two far kernels.
 template <int DP>
 struct FarQuery {
-  uint32_t p, id;
+  uint32_t p, id, inst;
   uint32_t base;   // output index of the instance's point 0 (ids - base = local ids)
   uint32_t root;   // the instance's subtree, kNoNode for a single point
   unsigned long long K;
@@ -814,12 +816,28 @@ struct FarQuery {
     K = skey[p];
     id = key_id(K);
     xq = load_pt<DP>(spts, p);
-    uint32_t inst = key_inst(scode[p], S, ib);
+    inst = key_inst(scode[p], S, ib);
     if (inst >= cv.ninst) inst = 0;
     base = (uint32_t)cv.instance(inst).out;
     root = roots[inst];
   }
 };
+
+// The dependent point of the same point under another cutoff of the sweep, if
+// it is higher here too: its distance bounds the search from the start (the
+// walk meets it again, so it needs no place among the candidates).
+template <int DP, bool F64>
+__device__ __forceinline__ double hint_bound(const FarHint& h, const ClassView& cv, const FarQuery<DP>& fq) {
+  if (!h.lambda) return INFINITY;
+  const int32_t l = h.lambda[fq.id];
+  const InstDev I = cv.instance(fq.inst);
+  if (l < 0 || (uint32_t)l >= I.n) return INFINITY;
+  const uint32_t o = fq.base + (uint32_t)l;
+  if (order_key(h.rho[o], o) <= fq.K) return INFINITY;
+  const Pt<DP> x = input_pt<DP>(h.pts, h.dtype, I.coord, I.d, (uint32_t)l);
+  if constexpr (F64) return dist64<DP>(fq.xq, x);
+  else return (double)dist32<DP>(fq.xq, x);
+}
 
 // Far queries, first round: one thread per query, a depth-first search with
 // an expansion budget.  Most queries finish within it (they expand a few dozen
@@ -830,7 +848,7 @@ __global__ void __launch_bounds__(kFarThreads)
 k_dep_far(const float* __restrict__ spts, const unsigned long long* __restrict__ scode,
           const unsigned long long* __restrict__ skey, ClassView cv,
           const CutGeom* __restrict__ cuts, const Node* __restrict__ nodes,
-          const float* __restrict__ nbox, const uint32_t* __restrict__ roots, FarQueue q,
+          const float* __restrict__ nbox, const uint32_t* __restrict__ roots, FarQueue q, FarHint hint,
           int32_t* __restrict__ lambda, double* __restrict__ delta, Counters* ctr) {
   const uint32_t qn = ctr->queue_n;
   const uint32_t n = cv.N;
@@ -855,7 +873,7 @@ k_dep_far(const float* __restrict__ spts, const unsigned long long* __restrict__
       } else if constexpr (F64) {
         Best<double> best;
         best.init();
-        const double s_init = q.s1d[e];
+        const double s_init = fmin(q.s1d[e], hint_bound<DP, true>(hint, cv, fq));
         const int r = tree_walk_from<DP>(
             nodes, nbox, n, skey, fq.K, fq.xq, fq.root, kFarBudget, expanded,
             [&](float lbs) { return (double)lbs > fmin(best.s1, s_init); },
@@ -876,7 +894,7 @@ k_dep_far(const float* __restrict__ spts, const unsigned long long* __restrict__
       } else {
         Best<float> best;
         best.init();
-        const float s_init = q.s1[e];
+        const float s_init = fminf(q.s1[e], (float)hint_bound<DP, false>(hint, cv, fq));
         const int r = tree_walk_from<DP>(
             nodes, nbox, n, skey, fq.K, fq.xq, fq.root, kFarBudget, expanded,
             [&](float lbs) { return beyond(lbs, band_of(fminf(best.s1, s_init), bmul, badd)); },
@@ -1144,7 +1162,7 @@ void near_dg(bool fp64, int layout, const float* spts, const unsigned long long*
              const unsigned long long* skey, const ClassView& cv, int32_t rho_skip,
              const void* pts, int dtype, const CutGeom* cuts, const HashInfo* hi,
              const unsigned long long* hkeys, const uint2* hvals, int32_t* lambda, double* delta,
-             FarQueue q, Counters* ctr, int seg_cells, cudaStream_t st) {
+             FarQueue q, Counters* ctr, int seg_cells, uint32_t skip_fill, cudaStream_t st) {
   const unsigned grid = grid_for(cv.nchunk, kNearWarps, sm_count() * 64u);
   if (layout == kLayoutSegment) {
     if (fp64)
@@ -1159,18 +1177,18 @@ void near_dg(bool fp64, int layout, const float* spts, const unsigned long long*
     if (fp64)
       k_dep_near<DP, G, true><<<grid, kNearThreads, 0, st>>>(spts, scode, skey, cv, rho_skip, pts,
                                                              dtype, cuts, hi, hkeys, hvals, lambda,
-                                                             delta, q, ctr);
+                                                             delta, q, ctr, skip_fill);
     else
       k_dep_near<DP, G, false><<<grid, kNearThreads, 0, st>>>(spts, scode, skey, cv, rho_skip, pts,
                                                               dtype, cuts, hi, hkeys, hvals, lambda,
-                                                              delta, q, ctr);
+                                                              delta, q, ctr, skip_fill);
   }
 }
 
 template <int DP>
 void far_dp(bool fp64, const float* spts, const unsigned long long* scode,
             const unsigned long long* skey, const ClassView& cv, const CutGeom* cuts,
-            const Node* nodes, const float* nbox, const uint32_t* root, FarQueue q,
+            const Node* nodes, const float* nbox, const uint32_t* root, FarQueue q, const FarHint& hint,
             int32_t* lambda, double* delta, Counters* ctr, cudaStream_t st) {
   // the queue length is known only on the device: launch enough threads for
   // a full SM load and let them stride over it
@@ -1178,12 +1196,12 @@ void far_dp(bool fp64, const float* spts, const unsigned long long* scode,
   const unsigned grid2 = grid_for(cv.N, kFarThreads / 32, sm_count() * 16u);
   if (fp64) {
     k_dep_far<DP, true><<<grid, kFarThreads, 0, st>>>(spts, scode, skey, cv, cuts, nodes, nbox,
-                                                      root, q, lambda, delta, ctr);
+                                                      root, q, hint, lambda, delta, ctr);
     k_dep_far_wide<DP, true><<<grid2, kFarThreads, 0, st>>>(spts, scode, skey, cv, cuts, nodes,
                                                             nbox, root, q, lambda, delta, ctr);
   } else {
     k_dep_far<DP, false><<<grid, kFarThreads, 0, st>>>(spts, scode, skey, cv, cuts, nodes, nbox,
-                                                       root, q, lambda, delta, ctr);
+                                                       root, q, hint, lambda, delta, ctr);
     k_dep_far_wide<DP, false><<<grid2, kFarThreads, 0, st>>>(spts, scode, skey, cv, cuts, nodes,
                                                              nbox, root, q, lambda, delta, ctr);
   }
@@ -1196,10 +1214,10 @@ void launch_dep_near(int dp, int g, bool fp64, int layout, const float* spts,
                      const ClassView& cv, int32_t rho_skip, const void* pts, int dtype,
                      const CutGeom* cuts, const HashInfo* hi, const unsigned long long* hkeys,
                      const uint2* hvals, int32_t* lambda, double* delta, FarQueue q, Counters* ctr,
-                     cudaStream_t st, int seg_cells) {
+                     cudaStream_t st, int seg_cells, uint32_t skip_fill) {
   if (cv.N == 0) return;
-  cudaMemsetAsync(&ctr->queue_n, 0, sizeof(unsigned int), st);
-  cudaMemsetAsync(&ctr->queue2_n, 0, sizeof(unsigned int), st);
+  // (beside the tensor form the queue is cleared and may be filled already)
+  if (!skip_fill) cudaMemsetAsync(&ctr->queue_n, 0, 2 * sizeof(unsigned int), st);  // queue_n and queue2_n
   if (layout == kLayoutCell) {
     launch_dep_near_cell(dp, g, fp64, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys,
                          hvals, lambda, delta, q, ctr, st);
@@ -1207,23 +1225,23 @@ void launch_dep_near(int dp, int g, bool fp64, int layout, const float* spts,
   }
   if (layout == kLayoutTree) {
     k_near_to_far<<<grid_for((uint64_t)cv.nchunk * 32u, 256, sm_count() * 16u), 256, 0, st>>>(
-        skey, cv, cuts, rho_skip, lambda, delta, q, ctr);
-  } else if (g == 1) near_dg<2, 1>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, st);
-  else if (g == 2) near_dg<2, 2>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, st);
-  else if (g == 3) near_dg<4, 3>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, st);
-  else if (dp == 4) near_dg<4, 4>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, st);
-  else near_dg<8, 4>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, st);
+        skey, cv, cuts, rho_skip, lambda, delta, q, ctr, hi, skip_fill);
+  } else if (g == 1) near_dg<2, 1>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, skip_fill, st);
+  else if (g == 2) near_dg<2, 2>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, skip_fill, st);
+  else if (g == 3) near_dg<4, 3>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, skip_fill, st);
+  else if (dp == 4) near_dg<4, 4>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, skip_fill, st);
+  else near_dg<8, 4>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, skip_fill, st);
   count_launches(1);
 }
 
 void launch_dep_far(int dp, bool fp64, const float* spts, const unsigned long long* scode,
                     const unsigned long long* skey, const ClassView& cv, const CutGeom* cuts,
                     const Node* nodes, const float* nbox, const uint32_t* root, FarQueue q,
-                    int32_t* lambda, double* delta, Counters* ctr, cudaStream_t st) {
+                    const FarHint& hint, int32_t* lambda, double* delta, Counters* ctr, cudaStream_t st) {
   if (cv.N == 0) return;
-  if (dp == 2) far_dp<2>(fp64, spts, scode, skey, cv, cuts, nodes, nbox, root, q, lambda, delta, ctr, st);
-  else if (dp == 4) far_dp<4>(fp64, spts, scode, skey, cv, cuts, nodes, nbox, root, q, lambda, delta, ctr, st);
-  else far_dp<8>(fp64, spts, scode, skey, cv, cuts, nodes, nbox, root, q, lambda, delta, ctr, st);
+  if (dp == 2) far_dp<2>(fp64, spts, scode, skey, cv, cuts, nodes, nbox, root, q, hint, lambda, delta, ctr, st);
+  else if (dp == 4) far_dp<4>(fp64, spts, scode, skey, cv, cuts, nodes, nbox, root, q, hint, lambda, delta, ctr, st);
+  else far_dp<8>(fp64, spts, scode, skey, cv, cuts, nodes, nbox, root, q, hint, lambda, delta, ctr, st);
   k_far_count<<<1, 1, 0, st>>>(ctr);
   count_launches(3);
 }

@@ -104,6 +104,14 @@ struct HashInfo {
   uint32_t npieces;    // entries of the piece list (tensor-core density)
 };
 
+// The rule between the tensor layouts and the CUDA-core ones, decided on the
+// device once the cells are counted: tensor tiles from min_fill points per
+// occupied cell on (0: always).  Both sides are launched; the one that is not
+// meant returns at once.
+__device__ __forceinline__ bool tensor_fill(uint32_t n, const HashInfo* hi, uint32_t min_fill) {
+  return (uint64_t)n >= (uint64_t)min_fill * hi->m;
+}
+
 // What a kernel needs to know about the class it works on.  A chunk is up to
 // 32 consecutive positions of one instance; chunk c of a single-instance
 // class holds positions 32c .. 32c+31, so it needs no tables.

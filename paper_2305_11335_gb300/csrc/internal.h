@@ -59,6 +59,13 @@ void launch_setup(const ClassView& cv, CutGeom* cuts, int ncut, const CutHost* h
 void launch_set_radius(const ClassView& cv, CutGeom* cuts, int rpref, cudaStream_t st);
 // near-dependent search `shift` grid levels finer than the density's (0: same)
 void launch_near_level(const ClassView& cv, CutGeom* cuts, int shift, cudaStream_t st);
+// The block geometry several cutoffs share: per instance that of the largest
+// of the cutoffs in `mask` (bit c: cutoff c of cuts [ncut][ninst]) into
+// geo [ninst]
+void launch_group_geometry(const ClassView& cv, const CutGeom* cuts, int ncut, unsigned long long mask,
+                           CutGeom* geo, cudaStream_t st);
+// cut ([ninst]) takes the level, radius and far bounds of geo ([ninst])
+void launch_adopt_geometry(const ClassView& cv, const CutGeom* geo, CutGeom* cut, cudaStream_t st);
 void launch_codes(const void* pts, int dtype, const ClassView& cv, int g, unsigned long long* codes,
                   uint32_t* ids, cudaStream_t st);
 void launch_gather(const void* pts, int dtype, const ClassView& cv, int dp,
@@ -127,20 +134,42 @@ enum { kLayoutUnion = 1, kLayoutSegment = 2, kLayoutTree = 3, kLayoutTensor = 4,
        kLayoutCell = 6 };
 
 // ---- density (density.cu) -------------------------------------------------------
+// Cutoffs evaluated in one density launch: they share the block geometry of
+// the largest of them; cut[j] is the [ninst] thresholds of cutoff j, rho[j]
+// its output row.
+constexpr int kMultiCuts = 4;
+struct MultiCut {
+  int m = 0;
+  const CutGeom* cut[kMultiCuts] = {};
+  int32_t* rho[kMultiCuts] = {};
+};
+// min_fill: points per occupied cell from which a tensor layout runs; below it
+// the CUDA-core layout launched beside it does (tensor_fill in dpc_device.cuh;
+// 0: always tensor).
 // rho of every point for one cutoff (cuts: [ninst]); rho_out is indexed by
-// output index (sid)
-void launch_density(int dp, int g, bool fp64, int layout, const float* spts,
+// output index (sid); d: the largest dimension of the class
+void launch_density(int dp, int g, int d, bool fp64, int layout, const float* spts,
                     const unsigned long long* scode, const uint32_t* sid, const ClassView& cv,
                     const CutGeom* cuts, HashInfo* hi, const unsigned long long* hkeys,
-                    const uint2* hvals, uint2* pieces, int32_t* rho_out,
+                    const uint2* hvals, uint4* pieces, int32_t* rho_out,
                     unsigned long long* skey, Counters* ctr, cudaStream_t st,
-                    int seg_cells = 0);
-// the tensor-core form of the density step (dp = 8, float32 filter only)
-// (pieces: scratch for the piece list, at least N / 128 + occupied cells entries)
-void launch_density_tc(int g, const float* spts, const uint32_t* sid, const ClassView& cv,
-                       const CutGeom* cuts, HashInfo* hi, const unsigned long long* hkeys,
-                       const uint2* hvals, uint2* pieces, int32_t* rho_out,
-                       unsigned long long* skey, Counters* ctr, cudaStream_t st);
+                    int seg_cells = 0, uint32_t min_fill = 0);
+// rho of the cutoffs of `mc` in one pass over the blocks of `geo` ([ninst]; the
+// hash holds its level's cells): tensor tiles for dp = 8 with the float32
+// filter, segments otherwise.  No order keys are written.
+void launch_density_multi(int dp, int g, int d, bool fp64, const float* spts, const unsigned long long* scode,
+                          const uint32_t* sid, const ClassView& cv, const CutGeom* geo, HashInfo* hi,
+                          const unsigned long long* hkeys, const uint2* hvals, uint4* pieces,
+                          const MultiCut& mc, Counters* ctr, cudaStream_t st, int seg_cells,
+                          uint32_t min_fill);
+// the tensor-core form of the density step (dp = 8, float32 filter only; d:
+// the largest dimension of the class; pieces: N entries of scratch; skey: the
+// order keys of cutoff 0, or null)
+void launch_density_tc(int d, const float* spts, const unsigned long long* scode, const uint32_t* sid,
+                       const ClassView& cv, const CutGeom* geo, HashInfo* hi,
+                       const unsigned long long* hkeys, const uint2* hvals, uint4* pieces,
+                       const MultiCut& mc, unsigned long long* skey, Counters* ctr, uint32_t min_fill,
+                       cudaStream_t st);
 // the cell layout of the density step (cell_tile.cu)
 void launch_density_cell(int dp, int g, bool fp64, const float* spts,
                          const unsigned long long* scode, const uint32_t* sid, const ClassView& cv,
@@ -160,6 +189,15 @@ struct FarQueue {
   float* s1_2;
   double* s1d2;
 };
+// Dependent points already found for another cutoff of the same call (null:
+// none), with this cutoff's densities and the caller's points: bounds for the
+// far search.
+struct FarHint {
+  const int32_t* lambda = nullptr;
+  const int32_t* rho = nullptr;
+  const void* pts = nullptr;
+  int dtype = 0;
+};
 // lambda and delta are indexed by output index; lambda values are
 // instance-local ids
 void launch_dep_near(int dp, int g, bool fp64, int layout, const float* spts,
@@ -168,7 +206,7 @@ void launch_dep_near(int dp, int g, bool fp64, int layout, const float* spts,
                      const CutGeom* cuts, const HashInfo* hi, const unsigned long long* hkeys,
                      const uint2* hvals, int32_t* lambda, double* delta, FarQueue q, Counters* ctr,
                      cudaStream_t st,
-                     int seg_cells = 0);
+                     int seg_cells = 0, uint32_t skip_fill = 0);
 // the cell layout of the near phase (cell_tile.cu)
 void launch_dep_near_cell(int dp, int g, bool fp64, const float* spts,
                           const unsigned long long* scode, const unsigned long long* skey,
@@ -176,18 +214,19 @@ void launch_dep_near_cell(int dp, int g, bool fp64, const float* spts,
                           const CutGeom* cuts, const HashInfo* hi,
                           const unsigned long long* hkeys, const uint2* hvals, int32_t* lambda,
                           double* delta, FarQueue q, Counters* ctr, cudaStream_t st);
-// the tensor-core form of the near phase (dp = 8, float32 filter only;
-// pieces: scratch as for launch_density_tc)
-void launch_dep_near_tc(int g, const float* spts, const uint32_t* sid,
+// the tensor-core form of the near phase (dp = 8, float32 filter only; d and
+// pieces as for launch_density_tc)
+void launch_dep_near_tc(int d, const float* spts, const unsigned long long* scode, const uint32_t* sid,
                         const unsigned long long* skey, const ClassView& cv, int32_t rho_skip,
                         const void* pts, int dtype, const CutGeom* cuts, HashInfo* hi,
-                        const unsigned long long* hkeys, const uint2* hvals, uint2* pieces,
-                        int32_t* lambda, double* delta, FarQueue q, Counters* ctr,
+                        const unsigned long long* hkeys, const uint2* hvals, uint4* pieces,
+                        int32_t* lambda, double* delta, FarQueue q, Counters* ctr, uint32_t min_fill,
                         cudaStream_t st);
 void launch_dep_far(int dp, bool fp64, const float* spts, const unsigned long long* scode,
                     const unsigned long long* skey, const ClassView& cv, const CutGeom* cuts,
                     const Node* nodes, const float* nbox, const uint32_t* root, FarQueue q,
-                    int32_t* lambda, double* delta, Counters* ctr, cudaStream_t st);
+                    const FarHint& hint, int32_t* lambda, double* delta, Counters* ctr,
+                    cudaStream_t st);
 
 // ---- decision graph (decision.cu) -------------------------------------------------
 // top-k by gamma = rho * delta and the (rho, delta) histogram of every instance

@@ -45,7 +45,8 @@ constexpr size_t kOffSid = kOffScode + al(8 * kStaticN);
 constexpr size_t kOffSkey = kOffSid + al(4 * kStaticN);
 constexpr size_t kOffHkeys = kOffSkey + al(8 * kStaticN);
 constexpr size_t kOffHvals = kOffHkeys + al(8 * (size_t)kStaticHash);
-constexpr size_t kStaticBytes = kOffHvals + al(8 * (size_t)kStaticHash);
+constexpr size_t kOffPieces = kOffHvals + al(8 * (size_t)kStaticHash);
+constexpr size_t kStaticBytes = kOffPieces + al(sizeof(uint4) * kStaticN);
 
 // The scratch area.  In host code this name is only a handle; its device
 // address comes from cudaGetSymbolAddress (once per device, below).
@@ -147,9 +148,10 @@ extern "C" int dpc_density_static(const void* pts, int dtype, int64_t n, int32_t
     launch_sort(codes_a, codes_b, ids_a, ids_b, nn, cls, hist, st);
     launch_gather(pts, dtype, cv, dp, codes_a, codes_b, ids_a, ids_b, spts, scode, sid, st);
     launch_cells(scode, cv, g, cut, hinfo, hkeys, hvals, kStaticHash, st);
-    launch_density(dp, g, prec == DPC_PREC_FP64, g >= 2 ? kLayoutSegment : kLayoutUnion, spts, scode,
-                   sid, cv, cut, hinfo, hkeys, hvals, nullptr, rho,
-                   skey, ctr, st);
+    const bool f64 = prec == DPC_PREC_FP64;
+    const int layout = dp == 8 && !f64 ? kLayoutTensor : (g >= 2 ? kLayoutSegment : kLayoutUnion);
+    launch_density(dp, g, d, f64, layout, spts, scode, sid, cv, cut, hinfo, hkeys, hvals,
+                   (uint4*)(base + kOffPieces), rho, skey, ctr, st, 0, 2);
   }
   if (cudaGetLastError() != cudaSuccess) return DPC_ERR_CUDA;
   if (flags & DPC_FLAG_SYNC_CHECK) {
