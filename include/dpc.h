@@ -115,21 +115,26 @@ enum {
 #define DPC_FLAG_RADIUS(r) ((uint32_t)(r) << 12)
 #define DPC_FLAG_RADIUS_MASK (0x7u << 12)
 /* Fixed work layout of the density and near-dependent kernels instead of the
- * default rule (density in segments for d >= 2; the near phase in segments for
- * d = 3, union otherwise) or the autotuned choice:
+ * default rule (density: tensor tiles in 5-8 dimensions with
+ * DPC_PREC_FP32_CERT from 2 points per occupied cell on, pairs in binary64,
+ * segments otherwise, union in 1-D; near phase: tensor tiles in 5-8 dimensions
+ * from 4 points per cell on, else the tree, union in 1-D above 1e6 points) or
+ * the autotuned choice:
  * 1 = union (a warp's 32 consecutive points, one query per lane, the union of
- * their blocks streamed as broadcast reads), 2 = segment (the block of one
- * cell spread over the lanes, the cell's queries one at a time), 3 = tree
- * (near phase only, density keeps its default: no block scan, every query goes
- * to the tree search of the far phase), 4 = tensor (density and near phase,
- * 5-8 dimensions with DPC_PREC_FP32_CERT: distance tiles on the tensor cores
- * with a certified error band; other cases use segment for the density and
- * union for the near phase), 5 = pairs (density only:
- * the segment layout evaluating every unordered pair once and counting it for
- * both points), 6 = cell (density and near phase: one warp per occupied cell,
- * the cell's block staged in shared memory, every lane one query -- or a share
- * of one query's candidates in cells of fewer than 32 points -- against all of
- * it).  Results do not depend on it. */
+ * their blocks streamed as broadcast reads), 2 = segment (the points around a
+ * few consecutive cells staged once, the cells' queries spread over the lanes),
+ * 3 = tree (near phase only, density keeps its default: no block scan, every
+ * query goes to the tree search of the far phase), 4 = tensor (density and near
+ * phase, 5-8 dimensions with DPC_PREC_FP32_CERT: distance tiles on the tensor
+ * cores with a certified error band; other cases use segment for the density
+ * and union for the near phase), 5 = pairs (density only: every unordered pair
+ * of a block once, counted for both points), 6 = cell (density and near phase:
+ * one warp per occupied cell, the cell's block staged in shared memory, every
+ * lane one query -- or a share of one query's candidates in cells of fewer than
+ * 32 points -- against all of it).  Without a fixed radius, layout or near
+ * shift small instances are compared in full (see dpc_stats.density_layout),
+ * and the cutoffs of a sweep share their passes: neither autotuning nor its
+ * choices apply to a call with several cutoffs.  Results do not depend on it. */
 #define DPC_FLAG_LAYOUT(v) ((uint32_t)(v) << 16)
 #define DPC_FLAG_LAYOUT_MASK (0x7u << 16)
 /* dpc_run only: capture the call's kernels into a CUDA graph the first time a

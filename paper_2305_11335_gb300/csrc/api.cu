@@ -211,7 +211,6 @@ struct Choice {
   int ns = 0;    // near-phase grid levels below the density's
   int sc = 0;    // segment layouts: cells a segment's union may hold (0: one cell)
   uint32_t dfill = 0, nfill = 0;  // points per cell from which a tensor layout runs (0: always)
-  int nsparse = kLayoutUnion;     // near layout below nfill
 };
 
 struct Workspace {
@@ -785,7 +784,7 @@ void density_step(Workspace* w, const ClassPlan& c, const ClassView& cv, const C
 void dependent_step(Workspace* w, const ClassPlan& c, const ClassView& cv, CutGeom* cuts,
                     const void* pts, int dtype, int32_t rho_skip, bool fp64, int layout, int nshift,
                     int seg_cells, int32_t* lambda, double* delta, uint32_t min_fill,
-                    int sparse_layout = kLayoutUnion, const FarHint& hint = FarHint()) {
+                    const FarHint& hint = FarHint()) {
   cudaStream_t st = w->stream;
   {
     Phase ph(w, DPC_PHASE_MAXKEY);
@@ -803,18 +802,18 @@ void dependent_step(Workspace* w, const ClassPlan& c, const ClassView& cv, CutGe
       launch_dep_near_tc(c.dmax, w->spts, w->scode, w->sid, w->skey, cv, rho_skip, pts, dtype, cuts, w->hinfo,
                          w->hkeys, w->hvals, w->pieces, lambda, delta, queue_of(w), w->ctr, min_fill, st);
       if (min_fill)  // sparse cells
-        launch_dep_near(c.dp, c.g, fp64, sparse_layout, w->spts, w->scode, w->skey, cv, rho_skip, pts, dtype, cuts,
-                        w->hinfo, w->hkeys, w->hvals, lambda, delta, queue_of(w), w->ctr, st, seg_cells, min_fill);
+        launch_dep_near(c.dp, c.g, fp64, kLayoutTree, w->spts, w->scode, w->skey, cv, rho_skip, pts, dtype, cuts,
+                        w->hinfo, w->hkeys, w->hvals, lambda, delta, queue_of(w), w->ctr, st, w->nbox, w->roots, seg_cells,
+                        min_fill);
     } else {
       // the tensor layout exists for 5-8 dimensions with the float32 filter
       if (layout == kLayoutTensor) layout = kLayoutUnion;
       launch_dep_near(c.dp, c.g, fp64, layout, w->spts, w->scode, w->skey, cv, rho_skip, pts, dtype,
                       cuts, w->hinfo, w->hkeys, w->hvals, lambda, delta, queue_of(w), w->ctr, st,
-                      seg_cells);
+                      w->nbox, w->roots, seg_cells);
     }
     w->last_choice.nlay = layout;
     w->last_choice.nfill = min_fill;
-    w->last_choice.nsparse = sparse_layout;
   }
   {
     Phase ph(w, DPC_PHASE_FAR);
@@ -925,18 +924,29 @@ struct NearTrial {
   double* delta;
 };
 
-// Default layouts (measured on the GB300): tensor tiles in 5-8 dimensions with
-// the float32 filter; else density in segments from 2 gridded dimensions up and
-// the near phase in segments in 3, union otherwise.
+// Default layouts (measured on the GB300).  Density: tensor tiles in 5-8
+// dimensions with the float32 filter, segments otherwise, pairs in binary64
+// (the binary64 pipe is the bound, so half the pairs: 1e5 points in 2-D 0.45 ms
+// against 1.34, in 3-D 3.7 against 5.7, in 7-D 12.2 against 20.5), union in 1-D.
+// Near phase: tensor tiles again; else the tree search (near phase + far search,
+// ms, blocks scanned -> tree: 1e6 points in 2-D 0.74 -> 0.34, blobs of 1e6 in 3-D
+// 2.21 -> 0.66, in 4-D 4.6 -> 1.9, binary64 1e5 in 5-D 62.9 -> 2.6; against it
+// only the 1e7-point 3-D walk, 4.84 -> 5.83, which the autotuner finds), in 1-D
+// up to 1e6 points (2e5: 0.14 -> 0.10; 2e6: 0.70 -> 1.02).
 inline bool tensor_class(const ClassPlan& c, bool fp64) { return c.dp == 8 && !fp64; }
 inline int default_dlayout(const ClassPlan& c, bool fp64) {
-  return tensor_class(c, fp64) ? kLayoutTensor : (c.g >= 2 ? kLayoutSegment : kLayoutUnion);
+  if (tensor_class(c, fp64)) return kLayoutTensor;
+  return c.g < 2 ? kLayoutUnion : (fp64 ? kLayoutPairs : kLayoutSegment);
 }
 inline int default_nlayout(const ClassPlan& c, bool fp64) {
-  return tensor_class(c, fp64) ? kLayoutTensor : (c.g == 3 ? kLayoutSegment : kLayoutUnion);
+  if (tensor_class(c, fp64)) return kLayoutTensor;
+  return c.g == 1 && c.N > 1000000u ? kLayoutUnion : kLayoutTree;
 }
 // segments of the segment layouts span cells while their union fits this
-inline int default_seg_cells(int g) { return g == 3 ? 48 : 0; }
+// (1e7 points in 3-D, density + near phase: 7.04 ms at 48 cells, 6.98 at 64,
+// 7.11 at 80, 7.41 at 128; 1e6 in 2-D, density: 0.43 ms one cell, 0.365 at 36,
+// 0.356 at 49, 0.545 at 81)
+inline int default_seg_cells(int g) { return g == 3 ? 56 : (g == 2 ? 36 : 0); }
 
 // The grid level and kernel layouts of one (class, cutoff): a fixed radius or
 // layout from the flags, else the autotuned choice (measured now when the
@@ -1017,7 +1027,7 @@ Choice choose(Workspace* w, const ClassPlan& c, const ClassView& cv, CutGeom* cu
               launch_dep_near(c.dp, c.g, fp64, nlays[l], w->spts, w->scode, w->skey, cv, 0,
                               near->pts, near->dtype, cuts, w->hinfo, w->hkeys, w->hvals,
                               near->lambda, near->delta, queue_of(w), w->ctr, st,
-                              default_seg_cells(c.g));
+                              w->nbox, w->roots, default_seg_cells(c.g));
             launch_dep_far(c.dp, fp64, w->spts, w->scode, w->skey, cv, cuts, w->nodes, w->nbox,
                            w->roots, queue_of(w), FarHint(), near->lambda, near->delta, w->ctr, st);
           }
@@ -1178,6 +1188,14 @@ void group_density_step(Workspace* w, const ClassPlan& c, const ClassView& cv, i
   w->last_choice = Choice();
   w->last_choice.dlay = tensor_class(c, fp64) ? kLayoutTensor : kLayoutSegment;
   w->last_choice.dfill = kTensorDensityFill;
+  if (g.cuts.size() == 1 && !tensor_class(c, fp64)) {  // one cutoff: the single-cutoff default
+    const int j = g.cuts[0];
+    w->last_choice.dlay = default_dlayout(c, fp64);
+    launch_density(c.dp, c.g, c.dmax, fp64, w->last_choice.dlay, w->spts, w->scode, w->sid, cv,
+                   w->cuts + (size_t)j * cv.ninst, w->hinfo, w->hkeys, w->hvals, w->pieces, rho + (size_t)j * N,
+                   w->skey, w->ctr, w->stream, default_seg_cells(c.g));
+    return;
+  }
   for (size_t i = 0; i < g.cuts.size(); i += kMultiCuts) {
     MultiCut mc;
     for (size_t j = i; j < g.cuts.size() && j < i + kMultiCuts; ++j) {
@@ -1392,11 +1410,8 @@ static void run_classes(Workspace* w, const CallPlan& P, const void* pts, int dt
             hint.dtype = dtype;
           }
           prev = k;
-          // with a bound to start from, the tree search alone beats a scan of
-          // the blocks except where tensor tiles run
-          const int nlay = hint.lambda && !tensor_class(c, fp64) ? kLayoutTree : default_nlayout(c, fp64);
-          dependent_step(w, c, cv, cuts, pts, dtype, 0, fp64, nlay, 0, default_seg_cells(c.g), lambda + o, delta + o,
-                         kTensorNearFill, hint.lambda ? kLayoutTree : kLayoutUnion, hint);
+          dependent_step(w, c, cv, cuts, pts, dtype, 0, fp64, default_nlayout(c, fp64), 0, default_seg_cells(c.g),
+                         lambda + o, delta + o, kTensorNearFill, hint);
           if (last && done) (*done)(1, k);
           labels_step(w, c, cv, k, one_params(params, c, P.ncut_all, k), rho + o, lambda + o, delta + o, label + o);
           if (last && done) (*done)(2, k);
@@ -1786,7 +1801,7 @@ int dpc_get_stats(void* stream, dpc_stats* out) {
     const Choice& ch = w->last_choice;
     auto sparse = [&](uint32_t fill) { return (uint64_t)w->last_points < (uint64_t)fill * hi.m; };
     out->density_layout = ch.dlay == kLayoutTensor && sparse(ch.dfill) ? kLayoutSegment : ch.dlay;
-    out->near_layout = ch.nlay == kLayoutTensor && sparse(ch.nfill) ? ch.nsparse : ch.nlay;
+    out->near_layout = ch.nlay == kLayoutTensor && sparse(ch.nfill) ? kLayoutTree : ch.nlay;
     out->near_shift = w->last_choice.ns;
     out->bits_per_axis = g.B;
   }

@@ -124,95 +124,6 @@ __device__ __forceinline__ int union_runs(const Union<G>& u,
   return nr;
 }
 
-// Run table of a union of at most 64 cells around the queries of one
-// segment, ordered by offset class for a multi-pass search over blocks of
-// radius 1.  A cell's class is the least number of axes on which it differs
-// from the cell of a segment query whose 3^G block contains it (0: a query's
-// own cell, 1: a face neighbour, 2: an edge neighbour, ...); cells in no
-// query's block get class G + 1 and are left out (no hash lookup either).
-// segc holds the segment's nseg distinct query cells.  cend[k] is one past
-// the last run of class <= k; returns the number of runs.
-template <int G>
-__device__ __forceinline__ int union_runs_classed(const Union<G>& u,
-                                                  const unsigned long long* __restrict__ hkeys,
-                                                  const uint2* __restrict__ hvals, uint32_t hmask,
-                                                  unsigned long long hb, uint32_t n, int lane,
-                                                  RunTable& rt, const uint32_t (*segc)[G], int nseg,
-                                                  int* cend) {
-  const uint32_t lanemask_lt = (1u << lane) - 1u;
-  uint32_t st[2], len[2], rel[2];
-  int cl[2];
-#pragma unroll
-  for (int b = 0; b < 2; ++b) {
-    const int o = 32 * b + lane;
-    st[b] = len[b] = rel[b] = 0u;
-    cl[b] = G + 1;
-    if (o < u.ncell) {
-      int rem = o;
-      uint32_t c[G];
-#pragma unroll
-      for (int a = 0; a < G; ++a) {
-        const int q = div_small(rem, u.inv[a]);
-        const uint32_t r = (uint32_t)(rem - q * u.w[a]);
-        c[a] = (uint32_t)u.lo[a] + r;
-        rel[b] |= r << (7 * a);
-        rem = q;
-      }
-      for (int t = 0; t < nseg; ++t) {
-        int nnz = 0;
-        bool inb = true;
-#pragma unroll
-        for (int a = 0; a < G; ++a) {
-          const int dl = (int)c[a] - (int)segc[t][a];
-          inb &= dl >= -1 && dl <= 1;
-          nnz += dl != 0;
-        }
-        if (inb) cl[b] = min(cl[b], nnz);
-      }
-      if (cl[b] <= G) {
-        const uint2 run = clip_run(hash_find(hkeys, hvals, hmask, hb | morton<G>(c)), n);
-        st[b] = run.x;
-        len[b] = run.y - run.x;
-      }
-    }
-  }
-  // slots: by class, then by round and lane; lengths first, offsets below
-  int nr = 0;
-#pragma unroll
-  for (int k = 0; k <= G; ++k) {
-#pragma unroll
-    for (int b = 0; b < 2; ++b) {
-      const bool mine = len[b] > 0 && cl[b] == k;
-      const unsigned m = __ballot_sync(kFull, mine);
-      if (mine) {
-        const int slot = nr + __popc(m & lanemask_lt);
-        rt.start[slot] = st[b];
-        rt.cell[slot] = rel[b];
-        rt.pre[slot] = len[b];
-      }
-      nr += __popc(m);
-    }
-    cend[k] = nr;
-  }
-  __syncwarp();
-  uint32_t carry = 0;
-  for (int base = 0; base < nr; base += 32) {
-    const int sl = base + lane;
-    const uint32_t v = sl < nr ? rt.pre[sl] : 0u;
-    uint32_t incl = v;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const uint32_t t = __shfl_up_sync(kFull, incl, d);
-      if (lane >= d) incl += t;
-    }
-    if (sl < nr) rt.pre[sl] = carry + incl - v;
-    carry += __shfl_sync(kFull, incl, 31);
-  }
-  if (lane == 0) rt.pre[nr] = carry;
-  __syncwarp();
-  return nr;
-}
-
 // Copy candidates [w0, w1) of the concatenated list into the window: lane l
 // copies candidates w0 + l, w0 + l + 32, ...; all loads of a window are
 // independent, so the warp keeps many of them in flight.
@@ -389,6 +300,84 @@ __device__ __forceinline__ void load_window_pos(const RunTable& rt, int nr, uint
       for (int a = 0; a < DP; ++a) cand[v].x[a] = __int_as_float(0x7fffffff);
     }
   }
+}
+
+// A warp's tile of candidates in shared memory, one array per coordinate,
+// negated (t = q + (-c) in the packed distances), with their order keys where
+// the kernel compares them; padded to a multiple of 4 * 32 with +inf
+// coordinates (distance +inf) and key 0.  Segment layouts: lane l answers query
+// l % nqp of the segment (nqp: its queries rounded up to a power of two) on the
+// candidates of part l / nqp, four at a time, so every read is a broadcast of
+// 16 bytes and no reduction is needed before the end.
+template <int ND, int CAP, bool KEYS>
+struct __align__(16) CandTile {
+  float x[ND][CAP];
+  unsigned long long key[KEYS ? CAP : 1];
+};
+
+// Stages candidates [w0, w1) of the run table (w1 - w0 <= CAP): the run of a
+// candidate is the number of run starts at or before it, counted with one
+// ballot per 32 candidates over byte flags kept in the table's cell words
+// (overwritten: CAP <= 4 kMaxUnion).
+template <int DP, int ND, int CAP, bool KEYS>
+__device__ __forceinline__ void stage_tile(RunTable& rt, int nr, uint32_t w0, uint32_t w1,
+                                           const float* __restrict__ spts,
+                                           const unsigned long long* __restrict__ skey,
+                                           CandTile<ND, CAP, KEYS>& t, int lane) {
+  const uint32_t n = w1 - w0;
+  const uint32_t npad = (n + 127u) & ~127u;
+  static_assert(CAP <= 4 * kMaxUnion, "flags fit the cell words");
+  for (uint32_t i = lane; i < npad / 4; i += 32) rt.cell[i] = 0u;
+  __syncwarp();
+  uint8_t* const flag = reinterpret_cast<uint8_t*>(rt.cell);
+  uint32_t before = 0;
+  for (int r = lane; r < nr; r += 32) {
+    const uint32_t p = rt.pre[r];
+    if (p <= w0) ++before;
+    else if (p < w1) flag[p - w0] = 1u;
+  }
+  uint32_t run = __reduce_add_sync(kFull, before) - 1u;  // the run holding w0
+  __syncwarp();
+  const uint32_t le = 0xffffffffu >> (31 - lane);
+  for (uint32_t e = lane; e < npad; e += 32) {
+    const unsigned m = __ballot_sync(kFull, flag[e] != 0);
+    const uint32_t r = run + __popc(m & le);
+    run += __popc(m);
+    Pt<DP> c;
+    unsigned long long k = 0ull;
+    if (e < n) {
+      const uint32_t src = rt.start[r] + (w0 + e - rt.pre[r]);
+      c = load_pt<DP>(spts, src);
+      if constexpr (KEYS) k = __ldg(skey + src);
+    } else {
+#pragma unroll
+      for (int a = 0; a < DP; ++a) c.x[a] = -INFINITY;
+    }
+#pragma unroll
+    for (int a = 0; a < ND; ++a) t.x[a][e] = -c.x[a];
+    if constexpr (KEYS) t.key[e] = k;
+  }
+  __syncwarp();
+}
+
+// Candidates e .. e + 3 of the tile as two packed pairs per coordinate.
+template <int ND, int CAP, bool KEYS>
+__device__ __forceinline__ void tile_quad(const CandTile<ND, CAP, KEYS>& t, uint32_t e, f32x2 (*c)[ND]) {
+#pragma unroll
+  for (int a = 0; a < ND; ++a) {
+    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(&t.x[a][e]);
+    c[0][a] = v.x;
+    c[1][a] = v.y;
+  }
+}
+
+// Candidate e's point (the padding coordinates 0).
+template <int DP, int ND, int CAP, bool KEYS>
+__device__ __forceinline__ Pt<DP> tile_pt(const CandTile<ND, CAP, KEYS>& t, uint32_t e) {
+  Pt<DP> p;
+#pragma unroll
+  for (int a = 0; a < DP; ++a) p.x[a] = a < ND ? -t.x[a < ND ? a : 0][e] : 0.f;
+  return p;
 }
 
 // Does the block of radius R around cell c0 contain cell c?

@@ -150,67 +150,31 @@ k_density(const float* __restrict__ spts, const unsigned long long* __restrict__
 }
 
 // ---------------------------------------------------------------------------
-// Segment form: the 32 points of a chunk are split into segments of equal
-// level-k cell; for each segment the warp looks up that cell's (2R+1)^g block
-// and spreads the block's candidates over the lanes (V per lane, held in
-// registers), then walks the segment's queries one by one: every lane
-// compares its V candidates with the query (read as a broadcast) and one warp
-// reduction gives the query's count.  No lane evaluates a candidate outside
-// the query's block, so the work is exactly the block's pairs.
-// In float32 the lane holds its candidates negated, two per packed register,
-// and evaluates dist32 for both at once (packed add / mul / fma: the same
-// rounding as the scalar sequence, so the certified band is unchanged); a
-// pair counts when s - up(t_in) is negative (its sign bit), and one unsigned
-// minimum per lane over the bit patterns of s finds band pairs, which are
-// recounted in binary64 after the window.  Small V (4 slots in 3-D) keeps the
-// kernel at 80 registers, 6 blocks per SM: the loop is latency-bound, and more
-// resident warps pay more than longer windows.
-
-// Exact count of the band pairs of queries qa and qb (sorted positions) among
-// this lane's candidates of window w0 (rare path: a warp takes it only for the
-// query pairs of a window that met a band pair, after the window's passes).
-// The candidates are loaded again one slot at a time, so neither the hot loop
-// nor this pass holds a window's copy.  Returns (binary64 counts of a | b << 16,
-// band pairs seen of a | b << 16), summed over the warp.
-template <int DP, int V, int ND>
-__device__ __forceinline__ uint2 seg_band_recount(const RunTable& rt, int nr, uint32_t w0,
-                                                  uint32_t total, const float* __restrict__ spts,
-                                                  int lane, uint32_t qa, uint32_t qb, float t_in,
-                                                  float t_out, double dc2) {
-  const Pt<DP> xa = load_pt<DP>(spts, qa);
-  const Pt<DP> xb = load_pt<DP>(spts, qb);
-  unsigned in = 0, seen = 0;
-#pragma unroll 1
-  for (uint32_t e = w0 + lane; e < total && e < w0 + 32u * V; e += 32u) {
-    int lo = 0, hi = nr - 1;  // the run holding candidate e
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (rt.pre[mid] <= e) lo = mid;
-      else hi = mid - 1;
-    }
-    const Pt<DP> x = load_pt<DP>(spts, rt.start[lo] + (e - rt.pre[lo]));
-    const float sa = dist32<DP, ND>(xa, x);
-    const float sb = dist32<DP, ND>(xb, x);
-    if (sa > t_in && sa <= t_out) {
-      ++seen;
-      in += dist64<DP, ND>(xa, x) <= dc2 ? 1u : 0u;
-    }
-    if (sb > t_in && sb <= t_out) {
-      seen += 0x10000u;
-      in += dist64<DP, ND>(xb, x) <= dc2 ? 0x10000u : 0u;
-    }
-  }
-  return make_uint2(__reduce_add_sync(kFull, in), __reduce_add_sync(kFull, seen));
-}
-
-template <int DP>
-constexpr int seg_v() { return DP == 2 ? 8 : (DP == 4 ? 4 : 2); }
-
+// Segment form: the 32 points of a chunk are split into segments of
+// consecutive cells (super_segment: one cell, or several while the box around
+// their blocks stays small); the warp looks the box's cells up once, stages
+// their points in shared memory and every lane counts for one query of the
+// segment: lane l answers query l % nqp on part l / nqp of the candidates, four
+// at a time as broadcast reads (CandTile).  The box contains every query's
+// block, so counting over all of it is exact.
+// In float32 two candidates are evaluated at once with packed add / mul / fma
+// (the same rounding as the scalar sequence, so the certified band is
+// unchanged); u = s - up(t_in) is negative (its sign bit) for a pair that
+// counts, and as an unsigned word at most (t_out - up(t_in)) rounded for one in
+// the band: one unsigned minimum per pair finds those, and a query that met one
+// recounts its band pairs of the tile in binary64.
+// What bounds it: issue slots; about half of them are the segment's set-up
+// (cell lookups, staging).  1e7 points in 3-D: 3.60 ms with the candidates in
+// registers across the lanes and one warp reduction per query pair and window
+// of 128 candidates, 2.65 with queries across the lanes.
 // M cutoffs of a sweep that share the block geometry `geo` (M = 1: one cutoff)
-// are counted in one pass: the distances, lookups and window loads are paid
-// once, every cutoff adds its own compare and count.
+// are counted in one pass: the distances, lookups and staging are paid once,
+// every cutoff adds its own compare and count.
+template <int DP>
+constexpr int seg_cap() { return DP == 8 ? 256 : 512; }
+
 template <int DP, int G, bool F64, int M>
-__global__ void __launch_bounds__(kThreads, (F64 || G >= 4 || M > 2) ? 5 : 6)
+__global__ void __launch_bounds__(kThreads, (DP == 8 || F64) ? 5 : 7)
 k_density_seg(const float* __restrict__ spts, const unsigned long long* __restrict__ scode,
               const uint32_t* __restrict__ sid, ClassView cv, const CutGeom* __restrict__ geo,
               const HashInfo* __restrict__ hi, const unsigned long long* __restrict__ hkeys,
@@ -218,12 +182,13 @@ k_density_seg(const float* __restrict__ spts, const unsigned long long* __restri
               Counters* ctr, int seg_cells, uint32_t skip_fill) {
   if (skip_fill && tensor_fill(cv.N, hi, skip_fill)) return;  // the tensor tiles' part
   constexpr int ND = real_dims<DP, G>();
-  constexpr int V = seg_v<DP>();
-  constexpr uint32_t W = 32u * V;
+  constexpr int kCap = seg_cap<DP>();
   __shared__ RunTable s_rt[kWarps];
+  __shared__ CandTile<ND, kCap, false> s_tile[kWarps];
   const int lane = threadIdx.x & 31;
   const int wib = threadIdx.x >> 5;
   RunTable& rt = s_rt[wib];
+  CandTile<ND, kCap, false>& tile = s_tile[wib];
   const int S = cv.cls->S, ib = cv.cls->ib;
   const uint32_t hmask = hi->hmask;
   const uint32_t n = cv.N;
@@ -236,152 +201,117 @@ k_density_seg(const float* __restrict__ spts, const unsigned long long* __restri
     const int R = geo[inst].R;
     const int shift = G * k;
     const int cmax = (1 << (cv.geom[inst].B - k)) - 1;
-    // s <= t_in  <=>  s - up(t_in) < 0, with up(t_in) the next float above
-    BandBits bb[M];
     f32x2 ntin2[M];
+    uint32_t width[M];  // band: bits(u) <= width
+    double dc2s[M];
 #pragma unroll
     for (int c = 0; c < M; ++c) {
       const CutGeom& C = mc.cut[c][inst];
-      bb[c] = band_bits(C.t_in, C.t_out);
-      ntin2[c] = pack2(-next_up(C.t_in), -next_up(C.t_in));
+      const float up = next_up(C.t_in);
+      dc2s[c] = C.dc2;
+      ntin2[c] = pack2(-up, -up);
+      // s <= t_out implies fl(s - up) <= fl(t_out - up)
+      width[c] = __float_as_uint(fmaxf(C.t_out - up, 0.f));
     }
     const unsigned long long hb = ib ? ((unsigned long long)inst << S) : 0ull;
     const uint32_t p = p0 + lane;
     const bool valid = p < end;
     const unsigned long long mycell = valid ? (key_code(scode[p], S, ib) >> shift) : ~0ull;
     const int nvalid = (int)min(32u, end - p0);
-    int32_t acc[M];  // lane j: the counts of query p0 + j
-#pragma unroll
-    for (int c = 0; c < M; ++c) acc[c] = 0;
     int s = 0;
     while (s < nvalid) {
       Union<G> u;
       const int e = super_segment<G>(mycell, valid, s, nvalid, R, cmax, seg_cells, lane, u);  // queries s .. e-1
       const int nr = union_runs<G>(u, hkeys, hvals, hmask, hb, n, lane, rt);
       const uint32_t total = rt.pre[nr];
-      pairs += (unsigned long long)(e - s) * total;
-      for (uint32_t w0 = 0; w0 < total; w0 += W) {
-        Pt<DP> cand[V];
-        load_window<DP, V>(rt, nr, w0, total, spts, lane, cand);
-        // slots of this window that hold candidates (warp-uniform)
-        const int vn = (int)min((uint32_t)V, (total - w0 + 31u) / 32u);
+      const int nq = e - s;
+      pairs += (unsigned long long)nq * total;
+      const int lg = nq > 1 ? 32 - __clz(nq - 1) : 0;  // nqp = 1 << lg
+      const int nqp = 1 << lg;
+      const uint32_t part = (uint32_t)lane >> lg, step = 4u * (32u >> lg);
+      const int mine = lane & (nqp - 1);
+      const uint32_t pq = p0 + (uint32_t)(s + min(mine, nq - 1));
+      const Pt<DP> me = load_pt<DP>(spts, pq);
+      int32_t cnt[M];
+#pragma unroll
+      for (int c = 0; c < M; ++c) cnt[c] = 0;
+      f32x2 q2[ND];
+#pragma unroll
+      for (int a = 0; a < ND; ++a) q2[a] = pack2(me.x[a], me.x[a]);
+      for (uint32_t w0 = 0; w0 < total; w0 += kCap) {
+        const uint32_t w1 = min(total, w0 + (uint32_t)kCap);
+        __syncwarp();
+        stage_tile<DP, ND, kCap, false>(rt, nr, w0, w1, spts, nullptr, tile, lane);
+        const uint32_t tn = w1 - w0;
         if constexpr (F64) {
-          for (int j = s; j < e; j += 2) {
-            const bool two = j + 1 < e;
-            const Pt<DP> xa = load_pt<DP>(spts, p0 + j);
-            const Pt<DP> xb = load_pt<DP>(spts, p0 + (two ? j + 1 : j));
-            unsigned n2[M];
+          for (uint32_t i = 4u * part; i < tn; i += step) {
 #pragma unroll
-            for (int c = 0; c < M; ++c) n2[c] = 0u;
+            for (int v = 0; v < 4; ++v) {
+              const double d = dist64<DP, ND>(me, tile_pt<DP>(tile, i + v));
 #pragma unroll
-            for (int v = 0; v < V; ++v) {
-              if (v >= vn) break;
-              const double da = dist64<DP, ND>(xa, cand[v]), db = dist64<DP, ND>(xb, cand[v]);
-#pragma unroll
-              for (int c = 0; c < M; ++c) {
-                const double dc2 = mc.cut[c][inst].dc2;
-                n2[c] += da <= dc2 ? 1u : 0u;
-                n2[c] += db <= dc2 ? 0x10000u : 0u;
-              }
-            }
-#pragma unroll
-            for (int c = 0; c < M; ++c) {
-              const unsigned t = __reduce_add_sync(kFull, n2[c]);
-              if (lane == j) acc[c] += (int32_t)(t & 0xffffu);
-              if (two && lane == j + 1) acc[c] += (int32_t)(t >> 16);
+              for (int c = 0; c < M; ++c) cnt[c] += d <= dc2s[c] ? 1 : 0;
             }
           }
         } else {
-          // the lane's candidates negated, two slots per packed register; a
-          // slot past the window's end holds +inf (distance +inf: never
-          // counted, never in the band)
-          f32x2 nc[V / 2][ND];
+          uint32_t lowest[M];
 #pragma unroll
-          for (int i = 0; i < V / 2; ++i) {
-            const bool ok0 = w0 + (uint32_t)lane + 64u * i < total;
-            const bool ok1 = w0 + (uint32_t)lane + 64u * i + 32u < total;
+          for (int c = 0; c < M; ++c) lowest[c] = 0xffffffffu;
+#pragma unroll 2
+          for (uint32_t i = 4u * part; i < tn; i += step) {
+            f32x2 cc[2][ND];
+            tile_quad(tile, i, cc);
 #pragma unroll
-            for (int k = 0; k < ND; ++k)
-              nc[i][k] = pack2(ok0 ? -cand[2 * i].x[k] : INFINITY, ok1 ? -cand[2 * i + 1].x[k] : INFINITY);
-          }
-          // two queries per pass over the lane's candidate pairs (independent
-          // chains); their per-lane counts (at most V each) share one 32-bit
-          // word per reduction, and one unsigned minimum per lane tells
-          // whether any of its pairs fell in the band
-          uint32_t bandq[M];  // bit j: queries j and j + 1 met a band pair
-#pragma unroll
-          for (int c = 0; c < M; ++c) bandq[c] = 0u;
-          auto passes = [&](auto full_window) {
-            constexpr bool kFullWindow = decltype(full_window)::value;
-            const int vp = (vn + 1) >> 1;
-            for (int j = s; j < e; j += 2) {
-              const bool two = j + 1 < e;
-              const Pt<DP> xa = load_pt<DP>(spts, p0 + j);
-              const Pt<DP> xb = load_pt<DP>(spts, p0 + (two ? j + 1 : j));
-              f32x2 qa[ND], qb[ND];
-#pragma unroll
-              for (int k = 0; k < ND; ++k) {
-                qa[k] = pack2(xa.x[k], xa.x[k]);
-                qb[k] = pack2(xb.x[k], xb.x[k]);
-              }
-              uint32_t na[M], nb[M], mband[M];
+            for (int h = 0; h < 2; ++h) {
+              const f32x2 sq = dist32x2<ND>(q2, cc[h]);
 #pragma unroll
               for (int c = 0; c < M; ++c) {
-                na[c] = nb[c] = 0u;
-                mband[c] = 0xffffffffu;
-              }
-#pragma unroll
-              for (int i = 0; i < V / 2; ++i) {
-                if (!kFullWindow && i >= vp) break;
-                const f32x2 sa = dist32x2<ND>(qa, nc[i]);
-                const f32x2 sb = dist32x2<ND>(qb, nc[i]);
-#pragma unroll
-                for (int c = 0; c < M; ++c) {
-                  na[c] += sign_count2(add2(sa, ntin2[c]));
-                  nb[c] += sign_count2(add2(sb, ntin2[c]));
-                  mband[c] = min(mband[c], band_min2(sa, bb[c].lo));
-                  mband[c] = min(mband[c], band_min2(sb, bb[c].lo));
-                }
-              }
-#pragma unroll
-              for (int c = 0; c < M; ++c) {
-                const unsigned t = __reduce_add_sync(kFull, na[c] + (nb[c] << 16));
-                // band pairs: recounted in binary64 after the window's passes
-                if (__any_sync(kFull, mband[c] < bb[c].width)) bandq[c] |= 1u << j;
-                if (lane == j) acc[c] += (int32_t)(t & 0xffffu);
-                if (two && lane == j + 1) acc[c] += (int32_t)(t >> 16);
+                const f32x2 x = add2(sq, ntin2[c]);
+                const uint32_t x0 = __float_as_uint(lo2(x)), x1 = __float_as_uint(hi2(x));
+                cnt[c] += (int32_t)((x0 >> 31) + (x1 >> 31));
+                lowest[c] = min(lowest[c], min(x0, x1));
               }
             }
-          };
-          if (vn == V) passes(std::true_type{});
-          else passes(std::false_type{});
+          }
 #pragma unroll
           for (int c = 0; c < M; ++c) {
-            while (bandq[c]) {
-              const int j = __ffs(bandq[c]) - 1;
-              bandq[c] &= bandq[c] - 1u;
-              const bool two = j + 1 < e;
+            if (__any_sync(kFull, lowest[c] <= width[c])) {  // rare: band pairs of this tile
               const CutGeom& C = mc.cut[c][inst];
-              const uint2 r = seg_band_recount<DP, V, ND>(rt, nr, w0, total, spts, lane, p0 + j,
-                                                          p0 + (two ? j + 1 : j), C.t_in, C.t_out, C.dc2);
-              if (lane == j) acc[c] += (int32_t)(r.x & 0xffffu);
-              if (two && lane == j + 1) acc[c] += (int32_t)(r.x >> 16);
-              if (lane == 0) band += (r.y & 0xffffu) + (two ? (r.y >> 16) : 0u);
+              const float t_in = C.t_in, t_out = C.t_out;
+              const double dc2 = C.dc2;
+              if (lowest[c] <= width[c]) {
+#pragma unroll 1
+                for (uint32_t i = 4u * part; i < tn; i += step) {
+#pragma unroll 1
+                  for (uint32_t v = i; v < i + 4u; ++v) {
+                    const Pt<DP> x = tile_pt<DP>(tile, v);
+                    const float s32 = dist32<DP, ND>(me, x);
+                    if (s32 > t_in && s32 <= t_out && mine < nq) {
+                      ++band;
+                      cnt[c] += dist64<DP, ND>(me, x) <= dc2 ? 1 : 0;
+                    }
+                  }
+                }
+              }
             }
           }
         }
       }
-      s = e;
-    }
-    if (valid) {
-      const uint32_t id = sid[p];
+      // the parts of each query
 #pragma unroll
-      for (int c = 0; c < M; ++c) mc.rho[c][id] = acc[c];
-      if (skey) skey[p] = order_key(acc[0], id);
+      for (int c = 0; c < M; ++c)
+        for (int o = nqp; o < 32; o <<= 1) cnt[c] += __shfl_xor_sync(kFull, cnt[c], o);
+      if (lane < nq) {
+        const uint32_t id = sid[pq];
+#pragma unroll
+        for (int c = 0; c < M; ++c) mc.rho[c][id] = cnt[c];
+        if (skey) skey[pq] = order_key(cnt[0], id);
+      }
+      s = e;
     }
   }
   if (lane == 0 && pairs) atomicAdd(&ctr->pairs, pairs);
   if constexpr (!F64) {
+    for (int o = 16; o > 0; o >>= 1) band += __shfl_xor_sync(kFull, band, o);
     if (lane == 0 && band) atomicAdd(&ctr->band_pairs, band);
   }
 }

@@ -343,34 +343,23 @@ k_dep_near(const float* __restrict__ spts, const unsigned long long* __restrict_
 }
 
 // Segment form of the near phase (the work layout of k_density_seg): the
-// chunk's points are split into segments of equal cell; for each segment the
-// block's candidates (and their order keys) are spread over the lanes, and for
-// every query of the segment each lane keeps the two smallest float32
-// distances among its higher candidates, merged over the warp with three
-// reductions.  Lane j collects the running best of the chunk's query j, then
-// settles it or queues it for the far phase exactly as k_dep_near does.
-// With radius-1 blocks in 2 or 3 gridded dimensions (float32) the block's
-// cells are taken in order of the number of axes on which they differ from a
-// query's own cell, and between windows a query whose winner is already
-// certified against every cell left leaves the sweep (on c3 73% of the
-// queries are certified before the cells that differ on all three axes).
-// 4 candidate slots per lane at 5 blocks per SM: the kernel is latency-bound,
-// and resident warps pay more than longer windows.
-
-template <int DP>
-constexpr int near_seg_v() { return DP == 8 ? 4 : (DP == 4 ? 4 : 8); }
-
-// Merges the candidate summary (a1 smallest, a2 second smallest, ao an id at
-// a1) into a running one; equal smallest distances leave s2 == s1.
-__device__ __forceinline__ void min2_merge(Min2& m, float a1, float a2, uint32_t ao) {
-  const float hi1 = fmaxf(m.s1, a1);
-  m.s2 = fminf(fminf(m.s2, a2), hi1);
-  m.o1 = a1 < m.s1 ? ao : m.o1;
-  m.s1 = fminf(m.s1, a1);
-}
+// chunk's points are split into segments of consecutive cells; the warp looks
+// the cells around a segment up once, stages their points and order keys in
+// shared memory, and lane l keeps the smallest and second smallest float32
+// distance among the higher candidates of query l % nqp in part l / nqp of the
+// tile, four candidates at a time as broadcast reads.  The parts are merged with
+// shuffles at the end; lane j then settles the chunk's query j or queues it
+// for the far phase exactly as k_dep_near does.
+// What bounds it: issue slots (about 13 instructions per candidate and lane,
+// and the segment's set-up).  1e7 points in 3-D: 6.09 ms with the candidates in
+// registers across the lanes and a warp reduction per query and window, 5.6 with
+// those reductions only where a window could still matter, 4.4 with queries
+// across the lanes.
+template <int DP, int G>
+constexpr int near_cap() { return DP == 2 ? 512 : (DP == 4 && G < 4 ? 384 : (DP == 4 ? 256 : 128)); }
 
 template <int DP, int G, bool F64>
-__global__ void __launch_bounds__(kNearThreads, 5)
+__global__ void __launch_bounds__(kNearThreads, DP == 8 ? 4 : 5)
 k_dep_near_seg(const float* __restrict__ spts, const unsigned long long* __restrict__ scode,
                const unsigned long long* __restrict__ skey, ClassView cv, int32_t rho_skip,
                const void* __restrict__ pts, int dtype, const CutGeom* __restrict__ cuts,
@@ -378,15 +367,15 @@ k_dep_near_seg(const float* __restrict__ spts, const unsigned long long* __restr
                const uint2* __restrict__ hvals, int32_t* __restrict__ lambda,
                double* __restrict__ delta, FarQueue q, Counters* ctr, int seg_cells) {
   constexpr int ND = real_dims<DP, G>();  // coordinates that can be nonzero
-  constexpr int V = near_seg_v<DP>();
-  constexpr uint32_t W = 32u * V;
+  constexpr int kCap = near_cap<DP, G>();
   __shared__ RunTable s_rt[kNearWarps];
   __shared__ RunTable s_rt2[kNearWarps];
-  __shared__ uint32_t s_segc[kNearWarps][32][G];  // distinct query cells of a segment
+  __shared__ CandTile<ND, kCap, true> s_tile[kNearWarps];
   const int lane = threadIdx.x & 31;
   const int wib = threadIdx.x >> 5;
   RunTable& rt = s_rt[wib];
   RunTable& rt2 = s_rt2[wib];
+  CandTile<ND, kCap, true>& tile = s_tile[wib];
   const int S = cv.cls->S, ib = cv.cls->ib;
   const uint32_t hmask = hi->hmask;
   const uint32_t n = cv.N;
@@ -395,15 +384,11 @@ k_dep_near_seg(const float* __restrict__ spts, const unsigned long long* __restr
   for (uint32_t ch = blockIdx.x * kNearWarps + wib; ch < cv.nchunk; ch += gridDim.x * kNearWarps) {
     uint32_t inst, p0, end;
     cv.chunk(ch, inst, p0, end);
-    const InstDev I = cv.instance(inst);
     const CutGeom& C = cuts[inst];
     const int k = C.k;
     const int R = C.R;
     const int shift = G * k;
     const int cmax = (1 << (cv.geom[inst].B - k)) - 1;
-    const float bmul = C.band_mul, badd = C.band_add;
-    const float far32 = C.far32;
-    const double far64 = C.far64;
     const unsigned long long hb = ib ? ((unsigned long long)inst << S) : 0ull;
     const uint32_t p = p0 + lane;
     const bool valid = p < end;
@@ -412,42 +397,6 @@ k_dep_near_seg(const float* __restrict__ spts, const unsigned long long* __restr
     const unsigned long long mycell = valid ? (key_code(scode[p], S, ib) >> shift) : ~0ull;
     const bool skip = valid && (int32_t)(K >> 32) < max(rho_skip, C.skip);
     const int nvalid = (int)min(32u, end - p0);
-    // this lane's query in fine units, for the cell lower bounds of pass 2
-    const GridGeom* geom = cv.geom + inst;
-    const float f2lo = geom->f2 * (1.f - 1e-5f);
-    const float cell_fine = (float)(1u << k);
-    float uq[G];
-    {
-      const Pt<DP> me = valid ? load_pt<DP>(spts, p) : Pt<DP>{};
-#pragma unroll
-      for (int a = 0; a < G; ++a)
-        uq[a] = valid ? (float)(((double)me.x[a] - geom->org[a]) * geom->inv_f) : 0.f;
-    }
-    // multi-pass search (float32, radius-1 blocks of 2 or 3 gridded axes):
-    // this lane's cell, and squared lower bounds of the distance from its
-    // query to any cell differing from its own on at least 2 (lbc[0]) or 3
-    // (lbc[1]) axes: the sums of the smallest squared gaps to the cell's faces
-    constexpr bool kClassed = !F64 && (G == 2 || G == 3);
-    float lbc[2] = {0.f, 0.f};
-    if constexpr (kClassed) {
-      uint32_t cown[G];
-      unmorton<G>(valid ? mycell : 0ull, cown);
-      float g2[G];
-#pragma unroll
-      for (int a = 0; a < G; ++a) {
-        const float lo = (float)cown[a] * cell_fine;
-        const float gp = fmaxf(fminf(uq[a] - lo - 1.f, lo + cell_fine - 1.f - uq[a]), 0.f);
-        g2[a] = gp * gp;
-      }
-      if constexpr (G == 2) {
-        lbc[0] = (g2[0] + g2[1]) * f2lo;
-      } else {
-        const float mx = fmaxf(fmaxf(g2[0], g2[1]), g2[2]);
-        const float sum = g2[0] + g2[1] + g2[2];
-        lbc[0] = (sum - mx) * f2lo;
-        lbc[1] = sum * f2lo;
-      }
-    }
     Min2 best;  // lane j: query p0 + j
     best.init();
     Exact best64;
@@ -458,180 +407,153 @@ k_dep_near_seg(const float* __restrict__ spts, const unsigned long long* __restr
       Union<G> u;
       const int e = super_segment<G>(mycell, valid, s, nvalid, R, cmax, seg_cells, lane, u);
       const unsigned seg = (e >= 32 ? 0xffffffffu : ((1u << e) - 1u)) & ~((1u << s) - 1u);  // lanes s .. e-1
-      // one cell only: the own-cell-first passes below apply
-      const bool single = (__ballot_sync(kFull, valid && mycell == cell) & seg) == seg;
       if (__ballot_sync(kFull, valid && !skip) & seg) {
-        uint32_t c0[G];
-        unmorton<G>(cell, c0);
-        // the segment's queries to answer
-        const unsigned qall = seg & __ballot_sync(kFull, valid && !skip);
-        // class-ordered run table (see below): runs [0, ce1) hold the cells
-        // differing from some query's own cell on at most one axis, [ce1,
-        // ce2) those differing on two
-        bool classed = false;
-        int ce1 = 0, ce2 = 0;
-        // candidates [P0, total) of a run table, window by window, for the
-        // queries of mask qm
-        auto scan = [&](const RunTable& tab, int ntab, uint32_t P0, uint32_t total, unsigned qm) {
-        for (uint32_t w0 = P0; w0 < total; w0 += W) {
-          Pt<DP> cand[V];
-          unsigned long long ck[V];
-          load_window<DP, V, true>(tab, ntab, w0, total, spts, lane, cand, skey, ck);
-          const int vn = (int)min((uint32_t)V, (total - w0 + 31u) / 32u);
-          // two queries per pass over the lane's candidates (independent chains)
-          for (unsigned m = qm; m;) {
-            const int j = __ffs(m) - 1;
-            m &= m - 1u;
-            const bool two = m != 0u;
-            const int jb = two ? __ffs(m) - 1 : j;
-            if (two) m &= m - 1u;
-            const unsigned long long Ka = __shfl_sync(kFull, K, j);
-            const unsigned long long Kb = __shfl_sync(kFull, K, jb);
-            constexpr bool act_a = true;
-            const bool act_b = two;
-            const Pt<DP> xa = load_pt<DP>(spts, p0 + j);
-            const Pt<DP> xb = load_pt<DP>(spts, p0 + jb);
+        // one cell only: the own-cell-first passes below apply
+        const bool single = (__ballot_sync(kFull, valid && mycell == cell) & seg) == seg;
+        const int nq = e - s;
+        const int lg = nq > 1 ? 32 - __clz(nq - 1) : 0;  // nqp = 1 << lg
+        const int nqp = 1 << lg;
+        const uint32_t part = (uint32_t)lane >> lg, step = 4u * (32u >> lg);
+        const int mine = lane & (nqp - 1);
+        const bool active = mine < nq;
+        const uint32_t pq = p0 + (uint32_t)(s + (active ? mine : 0));
+        const Pt<DP> me = load_pt<DP>(spts, pq);
+        // a lane without a query (or with a skipped one) takes no candidate
+        const int src = s + (active ? mine : 0);
+        unsigned long long Kq = __shfl_sync(kFull, K, src);
+        const int skipped = __shfl_sync(kFull, (int)skip, src);  // (every lane takes part)
+        if (!active || skipped) Kq = ~0ull;
+        f32x2 q2[ND];
+#pragma unroll
+        for (int a = 0; a < ND; ++a) q2[a] = pack2(me.x[a], me.x[a]);
+        float s1 = INFINITY, s2 = INFINITY;
+        uint32_t w1 = 0;  // low key word of the candidate at s1
+        Exact ex;
+        ex.init();
+        // every candidate of a run table, tile by tile
+        auto scan = [&](RunTable& tab, int ntab) {
+          const uint32_t total = tab.pre[ntab];
+          for (uint32_t t0 = 0; t0 < total; t0 += kCap) {
+            const uint32_t t1 = min(total, t0 + (uint32_t)kCap);
+            __syncwarp();
+            stage_tile<DP, ND, kCap, true>(tab, ntab, t0, t1, spts, skey, tile, lane);
+            const uint32_t tn = t1 - t0;
+            for (uint32_t i = 4u * part; i < tn; i += step) {
+              unsigned long long ck[4];
+              const ulonglong2 k0 = *reinterpret_cast<const ulonglong2*>(&tile.key[i]);
+              const ulonglong2 k1 = *reinterpret_cast<const ulonglong2*>(&tile.key[i + 2]);
+              ck[0] = k0.x;
+              ck[1] = k0.y;
+              ck[2] = k1.x;
+              ck[3] = k1.y;
+              if constexpr (F64) {
+#pragma unroll
+                for (int v = 0; v < 4; ++v)
+                  if (ck[v] > Kq) ex.add(dist64<DP, ND>(me, tile_pt<DP>(tile, i + v)), key_id(ck[v]));
+              } else {
+                f32x2 cc[2][ND];
+                tile_quad(tile, i, cc);
+                float dd[4];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                  const f32x2 sq = dist32x2<ND>(q2, cc[h]);
+                  dd[2 * h] = lo2(sq);
+                  dd[2 * h + 1] = hi2(sq);
+                }
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                  const float x = ck[v] > Kq ? dd[v] : INFINITY;
+                  s2 = fminf(s2, fmaxf(s1, x));
+                  w1 = x < s1 ? (uint32_t)ck[v] : w1;
+                  s1 = fminf(s1, x);
+                }
+              }
+            }
+          }
+          // the parts of each query (every lane of a query ends with the same)
+          for (int o = nqp; o < 32; o <<= 1) {
             if constexpr (F64) {
-              Exact ea, eb;
-              ea.init();
-              eb.init();
-#pragma unroll
-              for (int v = 0; v < V; ++v) {
-                if (v >= vn) break;
-                if (ck[v] > Ka) ea.add(dist64<DP, ND>(xa, cand[v]), key_id(ck[v]));
-                if (ck[v] > Kb) eb.add(dist64<DP, ND>(xb, cand[v]), key_id(ck[v]));
-              }
-              ea.merge_warp();
-              eb.merge_warp();
-              if (act_a && lane == j) best64.add(ea.s, ea.o);
-              if (act_b && lane == jb) best64.add(eb.s, eb.o);
+              ex.add(__shfl_xor_sync(kFull, ex.s, o), __shfl_xor_sync(kFull, ex.o, o));
             } else {
-              Min2 ma, mb;
-              ma.init();
-              mb.init();
-#pragma unroll
-              for (int v = 0; v < V; ++v) {
-                if (v >= vn) break;
-                const float da = dist32<DP, ND>(xa, cand[v]);
-                const float db = dist32<DP, ND>(xb, cand[v]);
-                const uint32_t id = key_id(ck[v]);
-                ma.add(ck[v] > Ka ? da : INFINITY, id);
-                mb.add(ck[v] > Kb ? db : INFINITY, id);
-              }
-              // per query: the warp's two smallest and an id at the smallest
-              auto warp_min2 = [&](const Min2& m, float& g1, float& g2, uint32_t& go) {
-                g1 = __uint_as_float(__reduce_min_sync(kFull, __float_as_uint(m.s1)));
-                const unsigned at = __ballot_sync(kFull, m.s1 == g1);
-                go = __reduce_min_sync(kFull, m.s1 == g1 ? m.o1 : 0xffffffffu);
-                g2 = __popc(at) > 1
-                         ? g1
-                         : __uint_as_float(
-                               __reduce_min_sync(kFull, __float_as_uint(m.s1 == g1 ? m.s2 : m.s1)));
-                if (!(g1 < INFINITY)) go = 0xffffffffu;
-              };
-              float a1, a2, b1, b2;
-              uint32_t ao, bo;
-              warp_min2(ma, a1, a2, ao);
-              warp_min2(mb, b1, b2, bo);
-              if (act_a && lane == j) min2_merge(best, a1, a2, ao);
-              if (act_b && lane == jb) min2_merge(best, b1, b2, bo);
+              const float o1 = __shfl_xor_sync(kFull, s1, o), o2 = __shfl_xor_sync(kFull, s2, o);
+              const uint32_t ow = __shfl_xor_sync(kFull, w1, o);
+              s2 = fminf(fminf(s2, o2), fmaxf(s1, o1));
+              w1 = o1 < s1 ? ow : w1;
+              s1 = fminf(s1, o1);
             }
           }
-          if constexpr (kClassed) {
-            // class-ordered table: the candidates left all lie in cells that
-            // differ from each query's own cell on at least two (three) axes;
-            // a query whose winner is certified and closer than every such
-            // cell takes no part in the windows left
-            const uint32_t nxt = w0 + W;
-            if (classed && nxt < total && nxt >= tab.pre[ce1]) {
-              const float lb = nxt >= tab.pre[ce2] ? lbc[1] : lbc[0];
-              bool done = false;
-              if ((qm >> lane) & 1u) {
-                if (best.o1 != 0xffffffffu) {
-                  const float bnd = band_of(best.s1, bmul, badd);
-                  done = bnd < far32 && best.s2 > bnd && beyond(lb, bnd);
-                }
-              }
-              qm &= ~__ballot_sync(kFull, done);
-              if (!qm) break;
-            }
-          }
-        }
         };
-        if constexpr (kClassed) classed = R == 1 && u.ncell <= 64;
-        // Classed (float32, radius-1 blocks of 2 or 3 gridded axes): the
-        // union's cells ordered by the least number of axes on which they
-        // differ from some query's own cell, one sweep of windows over them,
-        // and queries certified early leave it (above).  Cells in no query's
-        // block are left out: they lie beyond the far bound of every query.
-        // Otherwise dense blocks (more than 8 windows) of one cell: pass 1
-        // scans the segment's own cell, pass 2 only the other cells that can
-        // still hold a point closer than some query's best (a conservative
-        // lower bound decides); any other block: one pass over everything.
-        int nr, np;
-        if (classed) {
-          // the first lane of each cell of the segment (all lanes shuffle)
-          const unsigned long long prev = __shfl_up_sync(kFull, mycell, 1);
-          const bool head = ((seg >> lane) & 1u) && valid && (lane == s || prev != mycell);
-          const unsigned heads = __ballot_sync(kFull, head);
-          if (head) {
-            uint32_t cc[G];
-            unmorton<G>(mycell, cc);
-            const int r = __popc(heads & lanemask_lt);
-#pragma unroll
-            for (int a = 0; a < G; ++a) s_segc[wib][r][a] = cc[a];
-          }
-          __syncwarp();
-          int cend[G + 1];
-          nr = union_runs_classed<G>(u, hkeys, hvals, hmask, hb, n, lane, rt, s_segc[wib],
-                                     __popc(heads), cend);
-          ce1 = cend[1];
-          ce2 = cend[2];
-          np = 1;
+        const int nr = union_runs<G>(u, hkeys, hvals, hmask, hb, n, lane, rt);
+        // Dense blocks of one cell: first the cell itself, then only the other
+        // cells that can still hold a point closer than some query's best (a
+        // conservative lower bound decides); any other block: one pass.
+        if (!single || rt.pre[nr] <= 1024u) {
+          scan(rt, nr);
         } else {
-          nr = union_runs<G>(u, hkeys, hvals, hmask, hb, n, lane, rt);
-          np = (!single || rt.pre[nr] <= 8u * W) ? 1 : 2;
-        }
-        auto own = [&](const uint32_t* cc) {
-          bool same = true;
+          uint32_t c0[G];
+          unmorton<G>(cell, c0);
+          auto own = [&](const uint32_t* cc) {
+            bool same = true;
 #pragma unroll
-          for (int a = 0; a < G; ++a) same &= cc[a] == c0[a];
-          return same;
-        };
-        const bool mine = ((seg >> lane) & 1u) && !skip;
-        for (int pass = 0; pass < np; ++pass) {
-          int ntab = nr;
-          const RunTable* tab = &rt;
-          if (np == 2) {
-            tab = &rt2;
-            if (pass == 0) {
-              ntab = filter_runs<G>(rt, nr, u, rt2, lane, own);
-            } else {
-              ntab = filter_runs<G>(rt, nr, u, rt2, lane, [&](const uint32_t* cc) {
-                if (own(cc)) return false;
-                bool need = mine;
-                if (need) {
-                  float lb2 = 0.f;
+            for (int a = 0; a < G; ++a) same &= cc[a] == c0[a];
+            return same;
+          };
+          scan(rt2, filter_runs<G>(rt, nr, u, rt2, lane, own));
+          const GridGeom* geom = cv.geom + inst;
+          const float f2lo = geom->f2 * (1.f - 1e-5f);
+          const float cell_fine = (float)(1u << k);
+          float uq[G];  // the query in fine units
 #pragma unroll
-                  for (int a = 0; a < G; ++a) {
-                    const float lo = (float)cc[a] * cell_fine;
-                    const float l = lb_axis(lo, lo + cell_fine - 1.f, uq[a]);
-                    lb2 = fmaf(l, l, lb2);
-                  }
-                  const float lbs = lb2 * f2lo;
-                  if constexpr (F64) need = (double)lbs <= best64.s;
-                  else need = !beyond(lbs, band_of(best.s1, bmul, badd));
-                }
-                return __any_sync(kFull, need) != 0;
-              });
+          for (int a = 0; a < G; ++a) uq[a] = (float)(((double)me.x[a] - geom->org[a]) * geom->inv_f);
+          const float bnd = band_of(s1, C.band_mul, C.band_add);
+          const int n2 = filter_runs<G>(rt, nr, u, rt2, lane, [&](const uint32_t* cc) {
+            if (own(cc)) return false;
+            bool need = Kq != ~0ull;
+            if (need) {
+              float lb2 = 0.f;
+#pragma unroll
+              for (int a = 0; a < G; ++a) {
+                const float lo = (float)cc[a] * cell_fine;
+                const float l = lb_axis(lo, lo + cell_fine - 1.f, uq[a]);
+                lb2 = fmaf(l, l, lb2);
+              }
+              const float lbs = lb2 * f2lo;
+              if constexpr (F64) need = (double)lbs <= ex.s;
+              else need = !beyond(lbs, bnd);
             }
+            return __any_sync(kFull, need) != 0;
+          });
+          if constexpr (!F64) {  // the parts hold the merged best: keep it in one of them
+            if (part) s1 = s2 = INFINITY;
           }
-          scan(*tab, ntab, 0u, tab->pre[ntab], qall);
+          scan(rt2, n2);
+        }
+        // lane j takes query j's result
+        const int from = (lane - s) & 31;
+        if constexpr (F64) {
+          const double es = __shfl_sync(kFull, ex.s, from);
+          const uint32_t eo = __shfl_sync(kFull, ex.o, from);
+          if ((seg >> lane) & 1u) {
+            best64.s = es;
+            best64.o = eo;
+          }
+        } else {
+          const float b1 = __shfl_sync(kFull, s1, from), b2 = __shfl_sync(kFull, s2, from);
+          const uint32_t bw = __shfl_sync(kFull, w1, from);
+          if ((seg >> lane) & 1u) {
+            best.s1 = b1;
+            best.s2 = b2;
+            best.o1 = b1 < INFINITY ? 0xffffffffu - bw : 0xffffffffu;  // key_id of the low word
+          }
         }
       }
       s = e;
     }
 
+    const InstDev I = cv.instance(inst);
+    const float bmul = C.band_mul, badd = C.band_add;
+    const float far32 = C.far32;
+    const double far64 = C.far64;
     bool settled = false;
     float s1 = INFINITY;
     if (valid && !skip) {
@@ -674,33 +596,91 @@ k_dep_near_seg(const float* __restrict__ spts, const unsigned long long* __restr
 }
 
 // Tree layout of the near phase: no block scan; every query (but the skipped
-// ones) goes to the tree search with no bound.  Pays off where blocks are
-// dense enough that a best-first search of the tree, pruned by maximum key and
-// by box distance, visits far fewer points than the block holds.
-// One warp per 32-point chunk (the chunk gives the instance, hence its skip
-// threshold).
-__global__ void k_near_to_far(const unsigned long long* __restrict__ skey, ClassView cv,
-                              const CutGeom* __restrict__ cuts, int32_t rho_skip,
-                              int32_t* __restrict__ lambda, double* __restrict__ delta, FarQueue q,
-                              Counters* ctr, const HashInfo* __restrict__ hi, uint32_t skip_fill) {
+// ones) goes to the tree search, bounded by its nearest higher point among the
+// 96 sorted points around its chunk (Morton neighbours are mostly spatial
+// neighbours, so the bound is near the answer and the search mostly verifies
+// it).  One warp per 32-point chunk: the points of the chunk and of its two
+// neighbours staged once, every lane over all of them.
+// 1e6 points in 2-D: near phase and far search 0.53 + 0.21 ms with the blocks
+// scanned, 0.03 + 0.54 with the tree searched unbounded, 0.04 + 0.46 with this
+// bound, 0.04 + 0.29 with the walk of far_walk.
+template <int DP, int ND>
+__global__ void __launch_bounds__(kNearThreads)
+k_near_to_far(const float* __restrict__ spts, const unsigned long long* __restrict__ skey, ClassView cv,
+              const CutGeom* __restrict__ cuts, int32_t rho_skip, int32_t* __restrict__ lambda,
+              double* __restrict__ delta, FarQueue q, Counters* ctr, const HashInfo* __restrict__ hi,
+              const float* __restrict__ nbox, const uint32_t* __restrict__ roots, uint32_t skip_fill) {
   if (skip_fill && tensor_fill(cv.N, hi, skip_fill)) return;  // the tensor tiles' part
+  constexpr int kAround = 128;  // 96 used
+  __shared__ CandTile<ND, kAround, true> s_tile[kNearWarps];
   const int lane = threadIdx.x & 31;
+  CandTile<ND, kAround, true>& tile = s_tile[threadIdx.x >> 5];
   const uint32_t lanemask_lt = (1u << lane) - 1u;
-  const uint64_t total = (uint64_t)cv.nchunk * 32u;
-  for (uint64_t e = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; e < total;
-       e += (uint64_t)gridDim.x * blockDim.x) {
+  for (uint32_t c = blockIdx.x * kNearWarps + (threadIdx.x >> 5); c < cv.nchunk; c += gridDim.x * kNearWarps) {
     uint32_t inst, p0, end;
-    cv.chunk((uint32_t)(e >> 5), inst, p0, end);
+    cv.chunk(c, inst, p0, end);
+    const uint32_t start = cv.instance(inst).start;
+    const uint32_t a0 = p0 >= start + 32u ? p0 - 32u : start;
+    const uint32_t an = min(end, p0 + 64u) - a0;  // at most 96
+    const uint32_t npad = (an + 3u) & ~3u;
+    __syncwarp();
+    for (uint32_t e = lane; e < npad; e += 32) {
+      Pt<DP> x;
+#pragma unroll
+      for (int k = 0; k < DP; ++k) x.x[k] = -INFINITY;
+      unsigned long long kc = 0ull;
+      if (e < an) {
+        x = load_pt<DP>(spts, a0 + e);
+        kc = skey[a0 + e];
+      }
+#pragma unroll
+      for (int k = 0; k < ND; ++k) tile.x[k][e] = -x.x[k];
+      tile.key[e] = kc;
+    }
+    __syncwarp();
     const uint32_t p = p0 + lane;
     const bool valid = p < end;
-    const unsigned long long K = valid ? skey[p] : 0ull;
-    const bool skip = valid && (int32_t)(K >> 32) < max(rho_skip, cuts[inst].skip);
+    const uint32_t own = (valid ? p : p0) - a0;
+    const unsigned long long K = tile.key[own];
+    const Pt<DP> me = tile_pt<DP>(tile, own);
+    f32x2 q2[ND];
+#pragma unroll
+    for (int k = 0; k < ND; ++k) q2[k] = pack2(me.x[k], me.x[k]);
+    float s1 = INFINITY;
+#pragma unroll 2
+    for (uint32_t i = 0; i < npad; i += 4) {
+      const ulonglong2 k0 = *reinterpret_cast<const ulonglong2*>(&tile.key[i]);
+      const ulonglong2 k1 = *reinterpret_cast<const ulonglong2*>(&tile.key[i + 2]);
+      f32x2 cc[2][ND];
+      tile_quad(tile, i, cc);
+      const f32x2 sa = dist32x2<ND>(q2, cc[0]), sb = dist32x2<ND>(q2, cc[1]);
+      s1 = fminf(s1, k0.x > K ? lo2(sa) : INFINITY);
+      s1 = fminf(s1, k0.y > K ? hi2(sa) : INFINITY);
+      s1 = fminf(s1, k1.x > K ? lo2(sb) : INFINITY);
+      s1 = fminf(s1, k1.y > K ? hi2(sb) : INFINITY);
+    }
+    const CutGeom& C = cuts[inst];
+    const bool skip = valid && (int32_t)(K >> 32) < max(rho_skip, C.skip);
     if (skip) {
       const uint32_t id = key_id(K);
       lambda[id] = -1;
       delta[id] = __longlong_as_double(0x7ff8000000000000ll);  // NaN: skipped
     }
-    const bool push = valid && !skip;
+    // the instance's highest point has no dependent point: its key is the
+    // largest of the root's record
+    const uint32_t root = roots[inst];
+    bool top = false;
+    if (valid && !skip && root < cv.N - 1u) {  // (kNoNode: an instance of one point)
+      const unsigned long long* rk =
+          reinterpret_cast<const unsigned long long*>(nbox + (size_t)root * rec_words<DP>() + 4);
+      top = rk[0] <= K && rk[1] <= K;
+    }
+    if (top) {
+      const uint32_t id = key_id(K);
+      lambda[id] = -1;
+      delta[id] = INFINITY;
+    }
+    const bool push = valid && !skip && !top;
     const unsigned pm = __ballot_sync(kFull, push);
     uint32_t base = 0;
     if (lane == 0 && pm) base = atomicAdd(&ctr->queue_n, (unsigned)__popc(pm));
@@ -708,8 +688,10 @@ __global__ void k_near_to_far(const unsigned long long* __restrict__ skey, Class
     if (push) {
       const uint32_t slot = base + __popc(pm & lanemask_lt);
       q.pos[slot] = p;
-      q.s1[slot] = INFINITY;
-      q.s1d[slot] = INFINITY;
+      q.s1[slot] = s1;
+      // the binary64 search prunes with distances of its own: the bound is
+      // widened by the float32 error
+      q.s1d[slot] = s1 < INFINITY ? (double)band_of(s1, C.band_mul, C.band_add) : (double)INFINITY;
     }
   }
 }
@@ -799,6 +781,71 @@ __device__ __noinline__ int tree_walk_from(const Node* __restrict__ nodes,
   return kWalkDone;
 }
 
+// The walk of the far phase's first round: as tree_walk_from, with the nearer
+// child kept in a register (only the farther one is pushed) and the stack in
+// shared memory, [entry][thread]: lanes of a warp stand at different depths, so
+// entries in local memory cost a sector per lane and access.  Entries past
+// kFastStack (deep trees) go to a local array.
+constexpr int kFastStack = 24;
+struct FastStack {
+  uint32_t node[kFastStack][kFarThreads];
+  float lb[kFastStack][kFarThreads];
+};
+
+template <int DP, typename Prune, typename Visit>
+__device__ __forceinline__ int far_walk(FastStack& fs, const float* __restrict__ nbox, uint32_t n,
+                                        unsigned long long K, const Pt<DP>& xq, uint32_t start, uint32_t budget,
+                                        uint32_t& expanded, Prune prune, Visit visit) {
+  const int tid = threadIdx.x;
+  uint32_t more[kStack - kFastStack];
+  float morel[kStack - kFastStack];
+  int sp = 0;
+  uint32_t ni = start;
+  for (;;) {
+    if (ni + 1 >= n) return kWalkBad;
+    if (expanded >= budget) return kWalkBudget;
+    ++expanded;
+    const ChildRec<DP> r = load_rec<DP>(nbox, ni);
+    const bool h0 = r.key[0] > K, h1 = r.key[1] > K;  // something of higher key below
+    const bool leaf0 = r.child[0] & kLeafBit, leaf1 = r.child[1] & kLeafBit;
+    if (h0 && leaf0) visit(r.child[0] & ~kLeafBit, r.key[0], rec_point<DP>(r, 0));
+    if (h1 && leaf1) visit(r.child[1] & ~kLeafBit, r.key[1], rec_point<DP>(r, 1));
+    const float l0 = rec_lb2<DP>(r, 0, xq), l1 = rec_lb2<DP>(r, 1, xq);
+    const bool g0 = h0 && !leaf0 && !prune(l0), g1 = h1 && !leaf1 && !prune(l1);
+    if (g0 && g1) {
+      const bool first = l0 < l1;
+      const uint32_t far_c = first ? r.child[1] : r.child[0];
+      const float far_l = first ? l1 : l0;
+      if (sp < kFastStack) {
+        fs.node[sp][tid] = far_c;
+        fs.lb[sp][tid] = far_l;
+      } else if (sp < kStack) {
+        more[sp - kFastStack] = far_c;
+        morel[sp - kFastStack] = far_l;
+      } else {
+        return kWalkBad;
+      }
+      ++sp;
+      ni = first ? r.child[0] : r.child[1];
+    } else if (g0 || g1) {
+      ni = g0 ? r.child[0] : r.child[1];
+    } else {
+      float l;
+      do {
+        if (sp == 0) return kWalkDone;
+        --sp;
+        if (sp < kFastStack) {
+          ni = fs.node[sp][tid];
+          l = fs.lb[sp][tid];
+        } else {
+          ni = more[sp - kFastStack];
+          l = morel[sp - kFastStack];
+        }
+      } while (prune(l));
+    }
+  }
+}
+
 // Per-query context shared by the two far kernels.
 template <int DP>
 struct FarQuery {
@@ -850,6 +897,7 @@ k_dep_far(const float* __restrict__ spts, const unsigned long long* __restrict__
           const CutGeom* __restrict__ cuts, const Node* __restrict__ nodes,
           const float* __restrict__ nbox, const uint32_t* __restrict__ roots, FarQueue q, FarHint hint,
           int32_t* __restrict__ lambda, double* __restrict__ delta, Counters* ctr) {
+  __shared__ FastStack fs;
   const uint32_t qn = ctr->queue_n;
   const uint32_t n = cv.N;
   const int S = cv.cls->S, ib = cv.cls->ib;
@@ -874,8 +922,8 @@ k_dep_far(const float* __restrict__ spts, const unsigned long long* __restrict__
         Best<double> best;
         best.init();
         const double s_init = fmin(q.s1d[e], hint_bound<DP, true>(hint, cv, fq));
-        const int r = tree_walk_from<DP>(
-            nodes, nbox, n, skey, fq.K, fq.xq, fq.root, kFarBudget, expanded,
+        const int r = far_walk<DP>(
+            fs, nbox, n, fq.K, fq.xq, fq.root, kFarBudget, expanded,
             [&](float lbs) { return (double)lbs > fmin(best.s1, s_init); },
             [&](uint32_t t, unsigned long long kt, const Pt<DP>& x) {
               best.add(dist64<DP>(fq.xq, x), key_id(kt), t);
@@ -895,8 +943,8 @@ k_dep_far(const float* __restrict__ spts, const unsigned long long* __restrict__
         Best<float> best;
         best.init();
         const float s_init = fminf(q.s1[e], (float)hint_bound<DP, false>(hint, cv, fq));
-        const int r = tree_walk_from<DP>(
-            nodes, nbox, n, skey, fq.K, fq.xq, fq.root, kFarBudget, expanded,
+        const int r = far_walk<DP>(
+            fs, nbox, n, fq.K, fq.xq, fq.root, kFarBudget, expanded,
             [&](float lbs) { return beyond(lbs, band_of(fminf(best.s1, s_init), bmul, badd)); },
             [&](uint32_t t, unsigned long long kt, const Pt<DP>& x) {
               best.add(dist32<DP>(fq.xq, x), key_id(kt), t);
@@ -1214,7 +1262,8 @@ void launch_dep_near(int dp, int g, bool fp64, int layout, const float* spts,
                      const ClassView& cv, int32_t rho_skip, const void* pts, int dtype,
                      const CutGeom* cuts, const HashInfo* hi, const unsigned long long* hkeys,
                      const uint2* hvals, int32_t* lambda, double* delta, FarQueue q, Counters* ctr,
-                     cudaStream_t st, int seg_cells, uint32_t skip_fill) {
+                     cudaStream_t st, const float* nbox, const uint32_t* roots, int seg_cells,
+                     uint32_t skip_fill) {
   if (cv.N == 0) return;
   // (beside the tensor form the queue is cleared and may be filled already)
   if (!skip_fill) cudaMemsetAsync(&ctr->queue_n, 0, 2 * sizeof(unsigned int), st);  // queue_n and queue2_n
@@ -1224,8 +1273,16 @@ void launch_dep_near(int dp, int g, bool fp64, int layout, const float* spts,
     return;  // counted there
   }
   if (layout == kLayoutTree) {
-    k_near_to_far<<<grid_for((uint64_t)cv.nchunk * 32u, 256, sm_count() * 16u), 256, 0, st>>>(
-        skey, cv, cuts, rho_skip, lambda, delta, q, ctr, hi, skip_fill);
+    const unsigned grid = grid_for(cv.nchunk, kNearWarps, sm_count() * 64u);
+    auto go = [&](auto kern) {
+      kern<<<grid, kNearThreads, 0, st>>>(spts, skey, cv, cuts, rho_skip, lambda, delta, q, ctr, hi, nbox, roots,
+                                          skip_fill);
+    };
+    if (g == 1) go(k_near_to_far<2, 1>);
+    else if (g == 2) go(k_near_to_far<2, 2>);
+    else if (g == 3) go(k_near_to_far<4, 3>);
+    else if (dp == 4) go(k_near_to_far<4, 4>);
+    else go(k_near_to_far<8, 8>);
   } else if (g == 1) near_dg<2, 1>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, skip_fill, st);
   else if (g == 2) near_dg<2, 2>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, skip_fill, st);
   else if (g == 3) near_dg<4, 3>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, skip_fill, st);

@@ -205,8 +205,8 @@ void launch_dep_near(int dp, int g, bool fp64, int layout, const float* spts,
                      const ClassView& cv, int32_t rho_skip, const void* pts, int dtype,
                      const CutGeom* cuts, const HashInfo* hi, const unsigned long long* hkeys,
                      const uint2* hvals, int32_t* lambda, double* delta, FarQueue q, Counters* ctr,
-                     cudaStream_t st,
-                     int seg_cells = 0, uint32_t skip_fill = 0);
+                     cudaStream_t st, const float* nbox, const uint32_t* roots, int seg_cells = 0,
+                     uint32_t skip_fill = 0);
 // the cell layout of the near phase (cell_tile.cu)
 void launch_dep_near_cell(int dp, int g, bool fp64, const float* spts,
                           const unsigned long long* scode, const unsigned long long* skey,
