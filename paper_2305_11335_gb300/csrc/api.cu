@@ -727,8 +727,10 @@ void bin_class(Workspace* w, const void* pts, int dtype, const CallPlan& P, cons
   launch_chunks(cv, w->chunk_inst, w->chunk_pos, st);
   launch_bbox(pts, dtype, cv, c.g, st);
   launch_setup(cv, w->cuts, P.ncut, cut_table(w, c), host_cuts(P, b, c).data(), st);
-  launch_codes(pts, dtype, cv, c.g, w->codes_a, w->ids_a, st);
-  launch_sort(w->codes_a, w->codes_b, w->ids_a, w->ids_b, cv.N, w->cls, w->hist, st);
+  const bool counted = cv.N <= kSortMiddle;
+  uint32_t* count = counted ? launch_sort_clear(cv.N, w->hist, st) : nullptr;
+  launch_codes(pts, dtype, cv, c.g, w->codes_a, w->ids_a, count, st);
+  launch_sort(w->codes_a, w->codes_b, w->ids_a, w->ids_b, cv.N, w->cls, w->hist, counted, st);
   launch_gather(pts, dtype, cv, c.dp, w->codes_a, w->codes_b, w->ids_a, w->ids_b, w->spts,
                 w->scode, w->sid, st);
   (void)insts;
@@ -770,14 +772,14 @@ void cells_step(Workspace* w, const ClassPlan& c, const ClassView& cv, const Cut
 }
 
 void density_step(Workspace* w, const ClassPlan& c, const ClassView& cv, const CutGeom* cuts,
-                  bool fp64, int layout, int seg_cells, int32_t* rho, uint32_t min_fill) {
+                  int prec, int layout, int seg_cells, int32_t* rho, uint32_t min_fill) {
   Phase ph(w, DPC_PHASE_DENSITY);
   // the tensor layout exists for 5-8 dimensions with the float32 filter;
   // other cases run in segments, and the statistics report what ran
-  if (layout == kLayoutTensor && !(c.dp == 8 && !fp64)) layout = kLayoutSegment;
+  if (layout == kLayoutTensor && !(c.dp == 8 && prec == 0)) layout = kLayoutSegment;
   w->last_choice.dlay = layout;
   w->last_choice.dfill = min_fill;
-  launch_density(c.dp, c.g, c.dmax, fp64, layout, w->spts, w->scode, w->sid, cv, cuts, w->hinfo, w->hkeys,
+  launch_density(c.dp, c.g, c.dmax, prec, layout, w->spts, w->scode, w->sid, cv, cuts, w->hinfo, w->hkeys,
                  w->hvals, w->pieces, rho, w->skey, w->ctr, w->stream, seg_cells, min_fill);
 }
 
@@ -848,6 +850,16 @@ LabelParams one_params(const dpc_params* params, const ClassPlan& c, int ncut_al
   return L;
 }
 
+// Names one (class shape, cutoff) among the autotuned choices.
+std::string tune_key(const ClassPlan& c, const dpc_batch* b, int cut) {
+  char buf[160];
+  const double dc = b->d_cut[(size_t)c.members[0] * b->n_dcut + cut];
+  unsigned long long bits;
+  std::memcpy(&bits, &dc, sizeof(bits));
+  std::snprintf(buf, sizeof(buf), "%d/%d/%zu/%u/%d/%llx", c.dp, c.g, c.members.size(), c.N, cut, bits);
+  return buf;
+}
+
 // ---- small instances -----------------------------------------------------------
 
 // Whether a class runs from all pairs (small.cu) instead of the grid: one
@@ -861,11 +873,14 @@ LabelParams one_params(const dpc_params* params, const ClassPlan& c, int ncut_al
 // 1,336 at 4,096.  A captured call (DPC_FLAG_GRAPH) takes this path up to
 // 4,096 points only: tests/test_gpu_parity.py counts the kernels of a captured
 // grid pipeline at 6,000.
-bool small_class(const Workspace* w, const ClassPlan& c, const std::vector<Inst>& insts, uint32_t flags,
-                 bool density_only) {
+bool small_class(const Workspace* w, const dpc_batch* b, const CallPlan& P, const ClassPlan& c,
+                 const std::vector<Inst>& insts, uint32_t flags, bool density_only) {
   if (flags & (DPC_FLAG_RADIUS_MASK | DPC_FLAG_LAYOUT_MASK | DPC_FLAG_NEAR_SHIFT_MASK | DPC_FLAG_AUTOTUNE))
     return false;
-  if (!w->tuned.empty()) return false;  // choices of earlier calls stay in force
+  // an earlier call's choice for this shape stays in force
+  for (int k = 0; k < P.ncut && !w->tuned.empty(); ++k)
+    for (const char* kind : {"R/", "D/"})
+      if (w->tuned.count(kind + tune_key(c, b, P.cut_first + k))) return false;
   const bool fp64 = (flags & DPC_PREC_MASK) == DPC_PREC_FP64;
   const int d = insts[c.members[0]].d;
   const uint32_t nmax = small_limit(d, fp64, density_only);
@@ -907,15 +922,6 @@ void small_dependent_step(Workspace* w, const void* pts, int dtype, const CallPl
 // 3; 4 gridded dims allow only R = 1) and keeps the fastest for later calls of
 // the same shape.
 
-std::string tune_key(const ClassPlan& c, const dpc_batch* b, int cut) {
-  char buf[160];
-  const double dc = b->d_cut[(size_t)c.members[0] * b->n_dcut + cut];
-  unsigned long long bits;
-  std::memcpy(&bits, &dc, sizeof(bits));
-  std::snprintf(buf, sizeof(buf), "%d/%d/%zu/%u/%d/%llx", c.dp, c.g, c.members.size(), c.N, cut, bits);
-  return buf;
-}
-
 // What a tuning trial of the dependent step needs (null: density only).
 struct NearTrial {
   const void* pts;
@@ -934,9 +940,10 @@ struct NearTrial {
 // only the 1e7-point 3-D walk, 4.84 -> 5.83, which the autotuner finds), in 1-D
 // up to 1e6 points (2e5: 0.14 -> 0.10; 2e6: 0.70 -> 1.02).
 inline bool tensor_class(const ClassPlan& c, bool fp64) { return c.dp == 8 && !fp64; }
-inline int default_dlayout(const ClassPlan& c, bool fp64) {
-  if (tensor_class(c, fp64)) return kLayoutTensor;
-  return c.g < 2 ? kLayoutUnion : (fp64 ? kLayoutPairs : kLayoutSegment);
+inline int default_dlayout(const ClassPlan& c, int prec) {
+  if (tensor_class(c, prec != 0)) return kLayoutTensor;
+  if (prec == 2) return kLayoutSegment;  // 64-bit integers
+  return c.g < 2 ? kLayoutUnion : (prec == 1 ? kLayoutPairs : kLayoutSegment);
 }
 inline int default_nlayout(const ClassPlan& c, bool fp64) {
   if (tensor_class(c, fp64)) return kLayoutTensor;
@@ -958,13 +965,14 @@ inline int default_seg_cells(int g) { return g == 3 ? 56 : (g == 2 ? 36 : 0); }
 // with its best layouts.  The counters are saved around the trials;
 // rho_scratch (and the NearTrial outputs) receive the trials' results.
 Choice choose(Workspace* w, const ClassPlan& c, const ClassView& cv, CutGeom* cuts,
-              const dpc_batch* b, int cut, bool fp64, int32_t* rho_scratch, uint32_t flags,
+              const dpc_batch* b, int cut, int prec, int32_t* rho_scratch, uint32_t flags,
               const NearTrial* near = nullptr) {
+  const bool fp64 = prec != 0;
   Choice ch;
   ch.r = (int)((flags & DPC_FLAG_RADIUS_MASK) >> 12);
   const int forced = (int)((flags & DPC_FLAG_LAYOUT_MASK) >> 16);
   const int forced_ns = (int)((flags & DPC_FLAG_NEAR_SHIFT_MASK) >> 20);
-  ch.dlay = (forced && forced != kLayoutTree) ? forced : default_dlayout(c, fp64);
+  ch.dlay = (forced && forced != kLayoutTree) ? forced : default_dlayout(c, prec);
   ch.nlay = (forced && forced != kLayoutPairs) ? forced : default_nlayout(c, fp64);
   ch.ns = forced_ns ? forced_ns - 1 : 0;
   ch.sc = default_seg_cells(c.g);
@@ -1000,7 +1008,7 @@ Choice choose(Workspace* w, const ClassPlan& c, const ClassView& cv, CutGeom* cu
       if (timed) cudaEventRecord(w->tune_ev[1], st);
       for (int l = 0; l < 4; ++l) {
         if (l < ndl)
-          launch_density(c.dp, c.g, c.dmax, fp64, dlays[l], w->spts, w->scode, w->sid, cv, cuts, w->hinfo,
+          launch_density(c.dp, c.g, c.dmax, prec, dlays[l], w->spts, w->scode, w->sid, cv, cuts, w->hinfo,
                          w->hkeys, w->hvals, w->pieces, rho_scratch, w->skey, w->ctr, st,
                          default_seg_cells(c.g));
         if (timed) cudaEventRecord(w->tune_ev[2 + l], st);
@@ -1086,7 +1094,7 @@ Choice choose(Workspace* w, const ClassPlan& c, const ClassView& cv, CutGeom* cu
           if (t[l] < 0.97f * t[bi]) bi = l;
         return bi;
       };
-      const int di = pick(dt, dlays, ndl, default_dlayout(c, fp64));
+      const int di = pick(dt, dlays, ndl, default_dlayout(c, prec));
       int nsi = 0, ni = -1;
       float nms = 0.f;
       if (near) {
@@ -1179,19 +1187,19 @@ std::vector<CutGroup> group_cuts(const CallPlan& P, const dpc_batch* b, const Cl
 
 // The densities of one group (cells of its geometry into the hash first).
 void group_density_step(Workspace* w, const ClassPlan& c, const ClassView& cv, int ncut, const CutGroup& g,
-                        bool fp64, int32_t* rho, uint64_t N) {
+                        int prec, int32_t* rho, uint64_t N) {
   unsigned long long mask = 0;
   for (int j : g.cuts) mask |= 1ull << j;
   launch_group_geometry(cv, w->cuts, ncut, mask, w->geo, w->stream);
   cells_step(w, c, cv, w->geo);
   Phase ph(w, DPC_PHASE_DENSITY);
   w->last_choice = Choice();
-  w->last_choice.dlay = tensor_class(c, fp64) ? kLayoutTensor : kLayoutSegment;
+  w->last_choice.dlay = tensor_class(c, prec != 0) ? kLayoutTensor : kLayoutSegment;
   w->last_choice.dfill = kTensorDensityFill;
-  if (g.cuts.size() == 1 && !tensor_class(c, fp64)) {  // one cutoff: the single-cutoff default
+  if (g.cuts.size() == 1 && !tensor_class(c, prec != 0)) {  // one cutoff: the single-cutoff default
     const int j = g.cuts[0];
-    w->last_choice.dlay = default_dlayout(c, fp64);
-    launch_density(c.dp, c.g, c.dmax, fp64, w->last_choice.dlay, w->spts, w->scode, w->sid, cv,
+    w->last_choice.dlay = default_dlayout(c, prec);
+    launch_density(c.dp, c.g, c.dmax, prec, w->last_choice.dlay, w->spts, w->scode, w->sid, cv,
                    w->cuts + (size_t)j * cv.ninst, w->hinfo, w->hkeys, w->hvals, w->pieces, rho + (size_t)j * N,
                    w->skey, w->ctr, w->stream, default_seg_cells(c.g));
     return;
@@ -1202,7 +1210,7 @@ void group_density_step(Workspace* w, const ClassPlan& c, const ClassView& cv, i
       mc.cut[mc.m] = w->cuts + (size_t)g.cuts[j] * cv.ninst;
       mc.rho[mc.m++] = rho + (size_t)g.cuts[j] * N;
     }
-    launch_density_multi(c.dp, c.g, c.dmax, fp64, w->spts, w->scode, w->sid, cv, w->geo, w->hinfo, w->hkeys,
+    launch_density_multi(c.dp, c.g, c.dmax, prec, w->spts, w->scode, w->sid, cv, w->geo, w->hinfo, w->hkeys,
                          w->hvals, w->pieces, mc, w->ctr, w->stream, default_seg_cells(c.g), kTensorDensityFill);
   }
 }
@@ -1274,22 +1282,24 @@ int dpc_density(const void* pts, int dtype, const dpc_batch* b, int32_t* rho, ui
   CallPlan P = make_plan(b, insts, 0, b->n_dcut, false);
   if ((rc = prepare(w, P, b, insts, nullptr, flags))) return rc;
   const bool fp64 = (flags & DPC_PREC_MASK) == DPC_PREC_FP64;
+  // binary64 densities of int32 points: the same values in 64-bit integers
+  const int prec = fp64 ? (dtype == DPC_I32 ? 2 : 1) : 0;
   for (const ClassPlan& c : P.classes) {
     const ClassView cv = view_of(w, c, insts);
-    if (small_class(w, c, insts, flags, true)) {
+    if (small_class(w, b, P, c, insts, flags, true)) {
       small_density_step(w, pts, dtype, P, c, cv, b, insts, fp64, rho, N);
       continue;
     }
     bin_class(w, pts, dtype, P, c, cv, b, insts);
     if (sweep_call(P, flags)) {
-      for (const CutGroup& g : group_cuts(P, b, c)) group_density_step(w, c, cv, P.ncut, g, fp64, rho, N);
+      for (const CutGroup& g : group_cuts(P, b, c)) group_density_step(w, c, cv, P.ncut, g, prec, rho, N);
       continue;
     }
     for (int k = 0; k < P.ncut; ++k) {
       CutGeom* cuts = w->cuts + (size_t)k * cv.ninst;
-      const Choice ch = choose(w, c, cv, cuts, b, k, fp64, rho + (size_t)k * N, flags);
+      const Choice ch = choose(w, c, cv, cuts, b, k, prec, rho + (size_t)k * N, flags);
       cells_step(w, c, cv, cuts);
-      density_step(w, c, cv, cuts, fp64, ch.dlay, ch.sc, rho + (size_t)k * N, ch.dfill);
+      density_step(w, c, cv, cuts, prec, ch.dlay, ch.sc, rho + (size_t)k * N, ch.dfill);
     }
   }
   return finish(w, flags);
@@ -1313,9 +1323,11 @@ int dpc_dependent(const void* pts, int dtype, const dpc_batch* b, int32_t dcut_i
   CallPlan P = make_plan(b, insts, dcut_index, 1, false);
   if ((rc = prepare(w, P, b, insts, nullptr, flags))) return rc;
   const bool fp64 = (flags & DPC_PREC_MASK) == DPC_PREC_FP64;
+  // binary64 densities of int32 points: the same values in 64-bit integers
+  const int prec = fp64 ? (dtype == DPC_I32 ? 2 : 1) : 0;
   for (const ClassPlan& c : P.classes) {
     const ClassView cv = view_of(w, c, insts);
-    if (small_class(w, c, insts, flags, false)) {
+    if (small_class(w, b, P, c, insts, flags, false)) {
       launch_chunks(cv, w->chunk_inst, w->chunk_pos, w->stream);
       w->have_last = false;
       small_dependent_step(w, pts, dtype, P, c, cv, b, insts, fp64, 0, rho_skip, rho, lambda, delta);
@@ -1323,7 +1335,7 @@ int dpc_dependent(const void* pts, int dtype, const dpc_batch* b, int32_t dcut_i
     }
     bin_class(w, pts, dtype, P, c, cv, b, insts);
     tree_step(w, cv);
-    const Choice ch = choose(w, c, cv, w->cuts, b, dcut_index, fp64, nullptr,
+    const Choice ch = choose(w, c, cv, w->cuts, b, dcut_index, prec, nullptr,
                              flags & ~DPC_FLAG_AUTOTUNE, nullptr);
     cells_step(w, c, cv, w->cuts);
     launch_keys_from_rho(rho, w->sid, cv.N, w->skey, w->stream);
@@ -1372,12 +1384,14 @@ static void run_classes(Workspace* w, const CallPlan& P, const void* pts, int dt
                         const dpc_params* params, int32_t* rho, int32_t* lambda, double* delta,
                         int32_t* label, uint32_t flags, const StageDone* done = nullptr) {
   const bool fp64 = (flags & DPC_PREC_MASK) == DPC_PREC_FP64;
+  // binary64 densities of int32 points: the same values in 64-bit integers
+  const int prec = fp64 ? (dtype == DPC_I32 ? 2 : 1) : 0;
   for (const ClassPlan& c : P.classes) {
     // classes run one after another on the stream, so a phase of the last
     // class finishes that phase's output of every class
     const bool last = &c == &P.classes.back();
     const ClassView cv = view_of(w, c, insts);
-    if (small_class(w, c, insts, flags, false)) {
+    if (small_class(w, b, P, c, insts, flags, false)) {
       small_density_step(w, pts, dtype, P, c, cv, b, insts, fp64, rho, N);
       for (int k = 0; k < P.ncut; ++k) {
         const size_t o = (size_t)k * N;
@@ -1394,7 +1408,7 @@ static void run_classes(Workspace* w, const CallPlan& P, const void* pts, int dt
     if (sweep_call(P, flags)) {
       int prev = -1;  // the cutoff whose dependent points were found last
       for (const CutGroup& g : group_cuts(P, b, c)) {
-        group_density_step(w, c, cv, P.ncut, g, fp64, rho, N);
+        group_density_step(w, c, cv, P.ncut, g, prec, rho, N);
         if (last && done)
           for (int k : g.cuts) (*done)(0, k);
         for (int k : g.near) {
@@ -1423,9 +1437,9 @@ static void run_classes(Workspace* w, const CallPlan& P, const void* pts, int dt
       const size_t o = (size_t)k * N;
       CutGeom* cuts = w->cuts + (size_t)k * cv.ninst;
       const NearTrial nt{pts, dtype, lambda + o, delta + o};
-      const Choice ch = choose(w, c, cv, cuts, b, k, fp64, rho + o, flags, &nt);
+      const Choice ch = choose(w, c, cv, cuts, b, k, prec, rho + o, flags, &nt);
       cells_step(w, c, cv, cuts);
-      density_step(w, c, cv, cuts, fp64, ch.dlay, ch.sc, rho + o, ch.dfill);
+      density_step(w, c, cv, cuts, prec, ch.dlay, ch.sc, rho + o, ch.dfill);
       if (last && done) (*done)(0, k);
       dependent_step(w, c, cv, cuts, pts, dtype, 0, fp64, ch.nlay, ch.ns, ch.sc, lambda + o,
                      delta + o, ch.nfill);
@@ -1577,7 +1591,7 @@ int dpc_priority_range(const void* pts, int dtype, const dpc_batch* b, const int
     g.status = w->status;
     cudaMemcpyAsync(w->cls, &g, sizeof(g), cudaMemcpyHostToDevice, st);
     launch_sort(keys_a, keys_b, (uint32_t*)(s2 + v_a), (uint32_t*)(s2 + v_b), tn, w->cls,
-                (uint32_t*)(s2 + h_o), st);
+                (uint32_t*)(s2 + h_o), false, st);
     const int passes = sort_passes(31, ib);
     launch_prange_scatter((passes & 1) ? keys_b : keys_a, total, off, nq, max_out, ids, w->status, st);
   }

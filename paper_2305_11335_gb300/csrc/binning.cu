@@ -174,9 +174,8 @@ __global__ void k_bbox(const T* __restrict__ pts, ClassView cv, int g) {
 // c = floor((x - org) * inv_f) is within 1e-9 cells of the exact real value,
 // so its real position lies in [c - 0.5, c + 1.5) fine units; every bound
 // below is derived from that interval.
-__global__ void k_setup_geom(ClassView cv, int ncut, const CutHost* __restrict__ hc, CutArgs args) {
-  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= cv.ninst) return;
+__device__ void setup_geom(const ClassView& cv, int ncut, const CutHost* __restrict__ hc, const CutArgs& args,
+                           uint32_t t) {
   GridGeom* geom = cv.geom + t;
   double dcmin = INFINITY;
   for (int c = 0; c < ncut; ++c) dcmin = fmin(dcmin, hc ? hc[(size_t)t * ncut + c].dc : args.h[c].dc);
@@ -215,6 +214,12 @@ __global__ void k_setup_geom(ClassView cv, int ncut, const CutHost* __restrict__
   geom->f2 = __double2float_rd(f * f);
   geom->nbits = g * B;
   atomicMax(&cv.cls->S, g * B);
+}
+
+__global__ void k_setup_geom(ClassView cv, int ncut, const CutHost* __restrict__ hc,
+                             const __grid_constant__ CutArgs args) {
+  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < cv.ninst) setup_geom(cv, ncut, hc, args, t);
 }
 
 // Grid level k and block radius R of one (instance, cutoff), and the bounds
@@ -308,14 +313,9 @@ __global__ void k_adopt_geometry(ClassView cv, const CutGeom* __restrict__ geo, 
   cut[i].far64 = geo[i].far64;
 }
 
-// Per (instance, cutoff) search parameters, one thread each.  cuts is
-// [ncut][ninst].
-__global__ void k_setup_cuts(ClassView cv, CutGeom* cuts, int ncut, const CutHost* __restrict__ hc,
-                             CutArgs args) {
-  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= cv.ninst * (uint32_t)ncut) return;
-  const uint32_t i = t / ncut;
-  const int c = (int)(t - i * ncut);
+// Per (instance, cutoff) search parameters.  cuts is [ncut][ninst].
+__device__ void setup_cut(const ClassView& cv, CutGeom* cuts, int ncut, const CutHost* __restrict__ hc,
+                          const CutArgs& args, uint32_t i, int c) {
   const CutHost H = hc ? hc[(size_t)i * ncut + c] : args.h[c];
   CutGeom& C = cuts[(size_t)c * cv.ninst + i];
   C.dc = H.dc;
@@ -328,6 +328,21 @@ __global__ void k_setup_cuts(ClassView cv, CutGeom* cuts, int ncut, const CutHos
   choose_level(C, cv.geom + i, 0);
 }
 
+__global__ void k_setup_cuts(ClassView cv, CutGeom* cuts, int ncut, const CutHost* __restrict__ hc,
+                             const __grid_constant__ CutArgs args) {
+  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= cv.ninst * (uint32_t)ncut) return;
+  setup_cut(cv, cuts, ncut, hc, args, t / ncut, (int)(t % ncut));
+}
+
+// A single instance: geometry and cutoffs in one launch (thread c: cutoff c).
+__global__ void k_setup_one(ClassView cv, CutGeom* cuts, int ncut, const CutHost* __restrict__ hc,
+                            const __grid_constant__ CutArgs args) {
+  if (threadIdx.x == 0) setup_geom(cv, ncut, hc, args, 0u);
+  __syncthreads();
+  for (int c = threadIdx.x; c < ncut; c += blockDim.x) setup_cut(cv, cuts, ncut, hc, args, 0u, c);
+}
+
 // The level and radius of one cutoff of every instance again, with a
 // preferred block radius.
 __global__ void k_set_radius(ClassView cv, CutGeom* cuts, int rpref) {
@@ -338,10 +353,14 @@ __global__ void k_set_radius(ClassView cv, CutGeom* cuts, int rpref) {
 
 // Sort key of every point: (instance << S) | fine-grid Morton code; the
 // payload is the point's class position.
-template <typename T, int G>
+template <typename T, int G, bool COUNT>
 __global__ void k_codes(const T* __restrict__ pts, ClassView cv,
-                        unsigned long long* __restrict__ codes, uint32_t* __restrict__ ids) {
+                        unsigned long long* __restrict__ codes, uint32_t* __restrict__ ids,
+                        uint32_t* __restrict__ count) {
+  __shared__ uint32_t s_cnt[COUNT ? kSortMaxPasses : 1][256];
   const int S = cv.cls->S, ib = cv.cls->ib;
+  const int npass = sort_passes(S, ib);
+  if constexpr (COUNT) rs_clear_digits(s_cnt);
   const uint64_t total = (uint64_t)cv.nchunk * 32u;
   for (uint64_t e = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; e < total;
        e += (uint64_t)gridDim.x * blockDim.x) {
@@ -365,9 +384,12 @@ __global__ void k_codes(const T* __restrict__ pts, ClassView cv,
       const uint32_t ci = __double2uint_rz(v);
       c[a] = ci < cmax ? ci : cmax;
     }
-    codes[p] = (ib ? ((unsigned long long)i << S) : 0ull) | morton<G>(c);
+    const unsigned long long key = (ib ? ((unsigned long long)i << S) : 0ull) | morton<G>(c);
+    codes[p] = key;
     ids[p] = p;
+    if constexpr (COUNT) rs_count_digits(s_cnt, key, npass);  // the sort's digit counts on the way
   }
+  if constexpr (COUNT) rs_flush_digits(s_cnt, count, npass);
 }
 
 // Points into key order, converted to float and zero padded to DP; sid gets
@@ -445,16 +467,18 @@ __global__ void k_cells_count(const unsigned long long* __restrict__ scode, Clas
   if ((threadIdx.x & 31) == 0 && local) atomicAdd(&hi->m, local);
 }
 
-__global__ void k_hash_size(HashInfo* hi, uint32_t hcap) {
-  uint32_t want = 2u * hi->m;
+// Table size for m occupied cells (load at most 1/2).
+__device__ __forceinline__ uint32_t hash_mask(uint32_t m, uint32_t hcap) {
+  const uint32_t want = 2u * m;
   uint32_t t = 16;
   while (t < want && t < hcap) t <<= 1;
-  hi->hmask = t - 1;
+  return t - 1;
 }
 
-__global__ void k_hash_clear(unsigned long long* __restrict__ hkeys, const HashInfo* __restrict__ hi) {
-  const uint32_t T = hi->hmask + 1;
-  for (uint32_t h = blockIdx.x * blockDim.x + threadIdx.x; h < T; h += gridDim.x * blockDim.x)
+__global__ void k_hash_clear(unsigned long long* __restrict__ hkeys, HashInfo* hi, uint32_t hcap) {
+  const uint32_t mask = hash_mask(hi->m, hcap);
+  if (blockIdx.x == 0 && threadIdx.x == 0) hi->hmask = mask;
+  for (uint32_t h = blockIdx.x * blockDim.x + threadIdx.x; h <= mask; h += gridDim.x * blockDim.x)
     hkeys[h] = kEmpty;
 }
 
@@ -593,6 +617,11 @@ void launch_setup(const ClassView& cv, CutGeom* cuts, int ncut, const CutHost* h
   CutArgs a;
   if (!hc_dev)
     for (int c = 0; c < ncut && c < kCutChunk; ++c) a.h[c] = hc_host[c];
+  if (cv.ninst == 1) {
+    k_setup_one<<<1, 64, 0, st>>>(cv, cuts, ncut, hc_dev, a);
+    count_launches(1);
+    return;
+  }
   k_setup_geom<<<grid_for(cv.ninst), kThreads, 0, st>>>(cv, ncut, hc_dev, a);
   k_setup_cuts<<<grid_for((uint64_t)cv.ninst * ncut), kThreads, 0, st>>>(cv, cuts, ncut, hc_dev, a);
   count_launches(2);
@@ -600,20 +629,24 @@ void launch_setup(const ClassView& cv, CutGeom* cuts, int ncut, const CutHost* h
 
 template <typename T>
 static void codes_t(const T* pts, const ClassView& cv, int g, unsigned long long* codes,
-                    uint32_t* ids, cudaStream_t st) {
-  const unsigned grid = grid_for((uint64_t)cv.nchunk * 32u);
-  if (g == 1) k_codes<T, 1><<<grid, kThreads, 0, st>>>(pts, cv, codes, ids);
-  else if (g == 2) k_codes<T, 2><<<grid, kThreads, 0, st>>>(pts, cv, codes, ids);
-  else if (g == 3) k_codes<T, 3><<<grid, kThreads, 0, st>>>(pts, cv, codes, ids);
-  else k_codes<T, 4><<<grid, kThreads, 0, st>>>(pts, cv, codes, ids);
+                    uint32_t* ids, uint32_t* count, cudaStream_t st) {
+  const unsigned grid = grid_for((uint64_t)cv.nchunk * 32u, kThreads, sm_count() * (count ? 8u : 16u));
+  auto go = [&](auto yes, auto no) {
+    if (count) yes<<<grid, kThreads, 0, st>>>(pts, cv, codes, ids, count);
+    else no<<<grid, kThreads, 0, st>>>(pts, cv, codes, ids, nullptr);
+  };
+  if (g == 1) go(k_codes<T, 1, true>, k_codes<T, 1, false>);
+  else if (g == 2) go(k_codes<T, 2, true>, k_codes<T, 2, false>);
+  else if (g == 3) go(k_codes<T, 3, true>, k_codes<T, 3, false>);
+  else go(k_codes<T, 4, true>, k_codes<T, 4, false>);
   count_launches(1);
 }
 
 void launch_codes(const void* pts, int dtype, const ClassView& cv, int g, unsigned long long* codes,
-                  uint32_t* ids, cudaStream_t st) {
+                  uint32_t* ids, uint32_t* count, cudaStream_t st) {
   if (cv.N == 0) return;
-  if (dtype == 0) codes_t((const int32_t*)pts, cv, g, codes, ids, st);
-  else codes_t((const float*)pts, cv, g, codes, ids, st);
+  if (dtype == 0) codes_t((const int32_t*)pts, cv, g, codes, ids, count, st);
+  else codes_t((const float*)pts, cv, g, codes, ids, count, st);
 }
 
 template <typename T>
@@ -645,10 +678,9 @@ void launch_cells(const unsigned long long* scode, const ClassView& cv, int g, c
   const unsigned grid = grid_for(cv.N);
   cudaMemsetAsync(hi, 0, sizeof(HashInfo), st);
   k_cells_count<<<grid, kThreads, 0, st>>>(scode, cv, g, cuts, hi);
-  k_hash_size<<<1, 1, 0, st>>>(hi, hcap);
-  k_hash_clear<<<grid_for(hcap), kThreads, 0, st>>>(hkeys, hi);
+  k_hash_clear<<<grid_for(hcap), kThreads, 0, st>>>(hkeys, hi, hcap);
   k_hash_insert<<<grid, kThreads, 0, st>>>(scode, cv, g, cuts, hi, hkeys, hvals);
-  count_launches(4);
+  count_launches(3);
 }
 
 }  // namespace dpc

@@ -157,12 +157,19 @@ k_density(const float* __restrict__ spts, const unsigned long long* __restrict__
 // segment: lane l answers query l % nqp on part l / nqp of the candidates, four
 // at a time as broadcast reads (CandTile).  The box contains every query's
 // block, so counting over all of it is exact.
-// In float32 two candidates are evaluated at once with packed add / mul / fma
+// PREC 0 (float32 filter): two candidates are evaluated at once with packed add / mul / fma
 // (the same rounding as the scalar sequence, so the certified band is
 // unchanged); u = s - up(t_in) is negative (its sign bit) for a pair that
 // counts, and as an unsigned word at most (t_out - up(t_in)) rounded for one in
 // the band: one unsigned minimum per pair finds those, and a query that met one
-// recounts its band pairs of the tile in binary64.
+// recounts its band pairs of the tile in binary64.  PREC 1: every pair in
+// binary64.  PREC 2 (binary64 mode, int32 input): the same squared distance in
+// 64-bit integers, exact as binary64 is there (below 2^53), off the binary64
+// pipe, which issues one result per 16 clocks and warp.
+// A set of few chunks is cut finer: `sub` warps share a chunk's queries, so that
+// the chip has enough warps to hide the lookups (1e4 points in 2-D: 83 us with
+// one warp per chunk; a replayed run 101 -> 70 us with this, the sort's small
+// tiles and the merged set-up launches).
 // What bounds it: issue slots; about half of them are the segment's set-up
 // (cell lookups, staging).  1e7 points in 3-D: 3.60 ms with the candidates in
 // registers across the lanes and one warp reduction per query pair and window
@@ -173,13 +180,13 @@ k_density(const float* __restrict__ spts, const unsigned long long* __restrict__
 template <int DP>
 constexpr int seg_cap() { return DP == 8 ? 256 : 512; }
 
-template <int DP, int G, bool F64, int M>
-__global__ void __launch_bounds__(kThreads, (DP == 8 || F64) ? 5 : 7)
+template <int DP, int G, int PREC, int M>
+__global__ void __launch_bounds__(kThreads, (DP == 8 || PREC == 1) ? 5 : 7)
 k_density_seg(const float* __restrict__ spts, const unsigned long long* __restrict__ scode,
               const uint32_t* __restrict__ sid, ClassView cv, const CutGeom* __restrict__ geo,
               const HashInfo* __restrict__ hi, const unsigned long long* __restrict__ hkeys,
               const uint2* __restrict__ hvals, MultiCut mc, unsigned long long* __restrict__ skey,
-              Counters* ctr, int seg_cells, uint32_t skip_fill) {
+              Counters* ctr, int seg_cells, uint32_t skip_fill, uint32_t sub) {
   if (skip_fill && tensor_fill(cv.N, hi, skip_fill)) return;  // the tensor tiles' part
   constexpr int ND = real_dims<DP, G>();
   constexpr int kCap = seg_cap<DP>();
@@ -194,9 +201,13 @@ k_density_seg(const float* __restrict__ spts, const unsigned long long* __restri
   const uint32_t n = cv.N;
 
   unsigned long long band = 0, pairs = 0;
-  for (uint32_t ch = blockIdx.x * kWarps + wib; ch < cv.nchunk; ch += gridDim.x * kWarps) {
+  const uint64_t work = (uint64_t)cv.nchunk * sub;
+  for (uint64_t it = blockIdx.x * kWarps + wib; it < work; it += gridDim.x * kWarps) {
     uint32_t inst, p0, end;
-    cv.chunk(ch, inst, p0, end);
+    cv.chunk((uint32_t)(it / sub), inst, p0, end);
+    p0 += (uint32_t)(it % sub) * (32u / sub);
+    if (p0 >= end) continue;  // warp-uniform
+    end = min(end, p0 + 32u / sub);
     const int k = geo[inst].k;
     const int R = geo[inst].R;
     const int shift = G * k;
@@ -204,11 +215,13 @@ k_density_seg(const float* __restrict__ spts, const unsigned long long* __restri
     f32x2 ntin2[M];
     uint32_t width[M];  // band: bits(u) <= width
     double dc2s[M];
+    long long thr[M];  // PREC 2: s <= thr; real distances are at most 2^53, the padding's at least 2^57
 #pragma unroll
     for (int c = 0; c < M; ++c) {
       const CutGeom& C = mc.cut[c][inst];
       const float up = next_up(C.t_in);
       dc2s[c] = C.dc2;
+      thr[c] = PREC == 2 ? (long long)fmin(floor(C.dc2), 0x1p54) : 0ll;
       ntin2[c] = pack2(-up, -up);
       // s <= t_out implies fl(s - up) <= fl(t_out - up)
       width[c] = __float_as_uint(fmaxf(C.t_out - up, 0.f));
@@ -243,7 +256,34 @@ k_density_seg(const float* __restrict__ spts, const unsigned long long* __restri
         __syncwarp();
         stage_tile<DP, ND, kCap, false>(rt, nr, w0, w1, spts, nullptr, tile, lane);
         const uint32_t tn = w1 - w0;
-        if constexpr (F64) {
+        if constexpr (PREC == 2) {
+          // coordinates as integers (exact: |x| <= 2^24), not negated
+          const uint32_t npad = (tn + 127u) & ~127u;
+          for (uint32_t i = lane; i < npad; i += 32) {
+#pragma unroll
+            for (int a = 0; a < ND; ++a) tile.x[a][i] = __int_as_float(i < tn ? (int)-tile.x[a][i] : 1 << 29);
+          }
+          __syncwarp();
+          int iq[ND];
+#pragma unroll
+          for (int a = 0; a < ND; ++a) iq[a] = (int)me.x[a];
+          for (uint32_t i = 4u * part; i < tn; i += step) {
+            long long d[4] = {0, 0, 0, 0};
+#pragma unroll
+            for (int a = 0; a < ND; ++a) {
+              const int4 c4 = *reinterpret_cast<const int4*>(&tile.x[a][i]);
+              const int t0 = iq[a] - c4.x, t1 = iq[a] - c4.y, t2 = iq[a] - c4.z, t3 = iq[a] - c4.w;
+              d[0] += (long long)t0 * t0;
+              d[1] += (long long)t1 * t1;
+              d[2] += (long long)t2 * t2;
+              d[3] += (long long)t3 * t3;
+            }
+#pragma unroll
+            for (int v = 0; v < 4; ++v)
+#pragma unroll
+              for (int c = 0; c < M; ++c) cnt[c] += d[v] <= thr[c] ? 1 : 0;
+          }
+        } else if constexpr (PREC == 1) {
           for (uint32_t i = 4u * part; i < tn; i += step) {
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
@@ -310,7 +350,7 @@ k_density_seg(const float* __restrict__ spts, const unsigned long long* __restri
     }
   }
   if (lane == 0 && pairs) atomicAdd(&ctr->pairs, pairs);
-  if constexpr (!F64) {
+  if constexpr (PREC == 0) {
     for (int o = 16; o > 0; o >>= 1) band += __shfl_xor_sync(kFull, band, o);
     if (lane == 0 && band) atomicAdd(&ctr->band_pairs, band);
   }
@@ -540,12 +580,41 @@ inline unsigned grid_for(uint64_t items, int per_block, unsigned cap) {
   return (unsigned)b;
 }
 
+// Segment densities of the cutoffs of mc (prec: 0 float32 filter, 1 binary64,
+// 2 64-bit integers).
 template <int DP, int G>
-void density_dg(bool fp64, int layout, const float* spts, const unsigned long long* scode,
+void density_multi_dg(int prec, const float* spts, const unsigned long long* scode, const uint32_t* sid,
+                      const ClassView& cv, const CutGeom* geo, const HashInfo* hi, const unsigned long long* hkeys,
+                      const uint2* hvals, const MultiCut& mc, unsigned long long* skey, Counters* ctr, int seg_cells,
+                      uint32_t skip_fill, cudaStream_t st) {
+  // at least 8 warps per SM's scheduler, down to 4 queries a warp
+  uint32_t sub = 1;
+  while (sub < 8u && (uint64_t)cv.nchunk * sub < (uint64_t)sm_count() * 32u) sub *= 2;
+  const unsigned grid = grid_for((uint64_t)cv.nchunk * sub, kWarps, sm_count() * 64u);
+  auto go = [&](auto kern) {
+    kern<<<grid, kThreads, 0, st>>>(spts, scode, sid, cv, geo, hi, hkeys, hvals, mc, skey, ctr, seg_cells, skip_fill,
+                                    sub);
+  };
+  auto cuts = [&](auto p) {
+    constexpr int P = decltype(p)::value;
+    if (mc.m == 1) go(k_density_seg<DP, G, P, 1>);
+    else if (mc.m == 2) go(k_density_seg<DP, G, P, 2>);
+    else if (mc.m == 3) go(k_density_seg<DP, G, P, 3>);
+    else go(k_density_seg<DP, G, P, 4>);
+  };
+  if (prec == 0) cuts(std::integral_constant<int, 0>{});
+  else if (prec == 1) cuts(std::integral_constant<int, 1>{});
+  else cuts(std::integral_constant<int, 2>{});
+  count_launches(1);
+}
+
+template <int DP, int G>
+void density_dg(int prec, int layout, const float* spts, const unsigned long long* scode,
                 const uint32_t* sid, const ClassView& cv, const CutGeom* cuts, const HashInfo* hi,
                 const unsigned long long* hkeys, const uint2* hvals, int32_t* rho_out,
                 unsigned long long* skey, Counters* ctr, int seg_cells, uint32_t skip_fill, cudaStream_t st) {
   const unsigned grid = grid_for(cv.nchunk, kWarps, sm_count() * 64u);
+  const bool fp64 = prec != 0;
   if (layout == kLayoutPairs) {
     cudaMemsetAsync(skey, 0, sizeof(unsigned long long) * cv.N, st);
     uint32_t* cnt2 = reinterpret_cast<uint32_t*>(skey);
@@ -562,12 +631,9 @@ void density_dg(bool fp64, int layout, const float* spts, const unsigned long lo
     mc.m = 1;
     mc.cut[0] = cuts;
     mc.rho[0] = rho_out;
-    if (fp64)
-      k_density_seg<DP, G, true, 1><<<grid, kThreads, 0, st>>>(spts, scode, sid, cv, cuts, hi, hkeys,
-                                                               hvals, mc, skey, ctr, seg_cells, skip_fill);
-    else
-      k_density_seg<DP, G, false, 1><<<grid, kThreads, 0, st>>>(spts, scode, sid, cv, cuts, hi, hkeys,
-                                                                hvals, mc, skey, ctr, seg_cells, skip_fill);
+    density_multi_dg<DP, G>(prec, spts, scode, sid, cv, cuts, hi, hkeys, hvals, mc, skey, ctr, seg_cells, skip_fill,
+                            st);
+    return;
   } else {
     if (fp64)
       k_density<DP, G, true><<<grid, kThreads, 0, st>>>(spts, scode, sid, cv, cuts, hi, hkeys, hvals,
@@ -581,46 +647,26 @@ void density_dg(bool fp64, int layout, const float* spts, const unsigned long lo
 
 }  // namespace
 
-template <int DP, int G, bool F64>
-static void density_multi_dg(const float* spts, const unsigned long long* scode, const uint32_t* sid,
-                             const ClassView& cv, const CutGeom* geo, const HashInfo* hi,
-                             const unsigned long long* hkeys, const uint2* hvals, const MultiCut& mc, Counters* ctr,
-                             int seg_cells, uint32_t skip_fill, cudaStream_t st) {
-  auto go = [&](auto kern) {
-    kern<<<grid_for(cv.nchunk, kWarps, sm_count() * 64u), kThreads, 0, st>>>(spts, scode, sid, cv, geo, hi, hkeys,
-                                                                            hvals, mc, nullptr, ctr, seg_cells, skip_fill);
-  };
-  if (mc.m == 1) go(k_density_seg<DP, G, F64, 1>);
-  else if (mc.m == 2) go(k_density_seg<DP, G, F64, 2>);
-  else if (mc.m == 3) go(k_density_seg<DP, G, F64, 3>);
-  else go(k_density_seg<DP, G, F64, 4>);
-  count_launches(1);
-}
-
-void launch_density_multi(int dp, int g, int d, bool fp64, const float* spts, const unsigned long long* scode,
+void launch_density_multi(int dp, int g, int d, int prec, const float* spts, const unsigned long long* scode,
                           const uint32_t* sid, const ClassView& cv, const CutGeom* geo, HashInfo* hi,
                           const unsigned long long* hkeys, const uint2* hvals, uint4* pieces, const MultiCut& mc,
                           Counters* ctr, cudaStream_t st, int seg_cells, uint32_t min_fill) {
   if (cv.N == 0) return;
   uint32_t skip_fill = 0;
-  if (dp == 8 && !fp64) {
+  if (dp == 8 && prec == 0) {
     launch_density_tc(d, spts, scode, sid, cv, geo, hi, hkeys, hvals, pieces, mc, nullptr, ctr, min_fill, st);
     if (min_fill == 0) return;
     skip_fill = min_fill;
   }
-  auto go = [&](auto f64) {
-    constexpr bool F = decltype(f64)::value;
-    if (g == 1) density_multi_dg<2, 1, F>(spts, scode, sid, cv, geo, hi, hkeys, hvals, mc, ctr, seg_cells, skip_fill, st);
-    else if (g == 2) density_multi_dg<2, 2, F>(spts, scode, sid, cv, geo, hi, hkeys, hvals, mc, ctr, seg_cells, skip_fill, st);
-    else if (g == 3) density_multi_dg<4, 3, F>(spts, scode, sid, cv, geo, hi, hkeys, hvals, mc, ctr, seg_cells, skip_fill, st);
-    else if (dp == 4) density_multi_dg<4, 4, F>(spts, scode, sid, cv, geo, hi, hkeys, hvals, mc, ctr, seg_cells, skip_fill, st);
-    else density_multi_dg<8, 4, F>(spts, scode, sid, cv, geo, hi, hkeys, hvals, mc, ctr, seg_cells, skip_fill, st);
-  };
-  if (fp64) go(std::true_type{});
-  else go(std::false_type{});
+  auto go = [&](auto run) { run(prec, spts, scode, sid, cv, geo, hi, hkeys, hvals, mc, nullptr, ctr, seg_cells, skip_fill, st); };
+  if (g == 1) go(density_multi_dg<2, 1>);
+  else if (g == 2) go(density_multi_dg<2, 2>);
+  else if (g == 3) go(density_multi_dg<4, 3>);
+  else if (dp == 4) go(density_multi_dg<4, 4>);
+  else go(density_multi_dg<8, 4>);
 }
 
-void launch_density(int dp, int g, int d, bool fp64, int layout, const float* spts,
+void launch_density(int dp, int g, int d, int prec, int layout, const float* spts,
                     const unsigned long long* scode, const uint32_t* sid, const ClassView& cv,
                     const CutGeom* cuts, HashInfo* hi, const unsigned long long* hkeys,
                     const uint2* hvals, uint4* pieces, int32_t* rho_out,
@@ -628,7 +674,7 @@ void launch_density(int dp, int g, int d, bool fp64, int layout, const float* sp
   if (cv.N == 0) return;
   uint32_t skip_fill = 0;
   if (layout == kLayoutTensor) {
-    if (dp == 8 && !fp64 && pieces) {
+    if (dp == 8 && prec == 0 && pieces) {
       MultiCut mc;
       mc.m = 1;
       mc.cut[0] = cuts;
@@ -640,15 +686,15 @@ void launch_density(int dp, int g, int d, bool fp64, int layout, const float* sp
     layout = kLayoutSegment;
   }
   if (layout == kLayoutCell) {
-    launch_density_cell(dp, g, fp64, spts, scode, sid, cv, cuts, hi, hkeys, hvals, rho_out, skey, ctr,
+    launch_density_cell(dp, g, prec != 0, spts, scode, sid, cv, cuts, hi, hkeys, hvals, rho_out, skey, ctr,
                         st);
     return;
   }
-  if (g == 1) density_dg<2, 1>(fp64, layout, spts, scode, sid, cv, cuts, hi, hkeys, hvals, rho_out, skey, ctr, seg_cells, skip_fill, st);
-  else if (g == 2) density_dg<2, 2>(fp64, layout, spts, scode, sid, cv, cuts, hi, hkeys, hvals, rho_out, skey, ctr, seg_cells, skip_fill, st);
-  else if (g == 3) density_dg<4, 3>(fp64, layout, spts, scode, sid, cv, cuts, hi, hkeys, hvals, rho_out, skey, ctr, seg_cells, skip_fill, st);
-  else if (dp == 4) density_dg<4, 4>(fp64, layout, spts, scode, sid, cv, cuts, hi, hkeys, hvals, rho_out, skey, ctr, seg_cells, skip_fill, st);
-  else density_dg<8, 4>(fp64, layout, spts, scode, sid, cv, cuts, hi, hkeys, hvals, rho_out, skey, ctr, seg_cells, skip_fill, st);
+  if (g == 1) density_dg<2, 1>(prec, layout, spts, scode, sid, cv, cuts, hi, hkeys, hvals, rho_out, skey, ctr, seg_cells, skip_fill, st);
+  else if (g == 2) density_dg<2, 2>(prec, layout, spts, scode, sid, cv, cuts, hi, hkeys, hvals, rho_out, skey, ctr, seg_cells, skip_fill, st);
+  else if (g == 3) density_dg<4, 3>(prec, layout, spts, scode, sid, cv, cuts, hi, hkeys, hvals, rho_out, skey, ctr, seg_cells, skip_fill, st);
+  else if (dp == 4) density_dg<4, 4>(prec, layout, spts, scode, sid, cv, cuts, hi, hkeys, hvals, rho_out, skey, ctr, seg_cells, skip_fill, st);
+  else density_dg<8, 4>(prec, layout, spts, scode, sid, cv, cuts, hi, hkeys, hvals, rho_out, skey, ctr, seg_cells, skip_fill, st);
 }
 
 void launch_keys_from_rho(const int32_t* rho, const uint32_t* sid, uint32_t n,

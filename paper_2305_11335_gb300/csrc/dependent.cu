@@ -1026,6 +1026,10 @@ k_dep_far_wide(const float* __restrict__ spts, const unsigned long long* __restr
   uint32_t* stk = s_stk[wib];
   float* stl = s_lb[wib];
   const uint32_t qn = ctr->queue2_n;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {  // statistics of the round
+    ctr->far_queries += ctr->queue_n;
+    ctr->far_wide_queries += qn;
+  }
   const uint32_t n = cv.N;
   const int S = cv.cls->S, ib = cv.cls->ib;
   const float bmul = cuts[0].band_mul, badd = cuts[0].band_add;
@@ -1192,12 +1196,6 @@ k_dep_far_wide(const float* __restrict__ spts, const unsigned long long* __restr
   }
 }
 
-__global__ void k_far_count(Counters* ctr) {
-  ctr->far_queries += ctr->queue_n;
-  ctr->far_wide_queries += ctr->queue2_n;
-}
-
-
 inline unsigned grid_for(uint64_t items, int per_block, unsigned cap) {
   uint64_t b = (items + per_block - 1) / per_block;
   if (b < 1) b = 1;
@@ -1299,8 +1297,7 @@ void launch_dep_far(int dp, bool fp64, const float* spts, const unsigned long lo
   if (dp == 2) far_dp<2>(fp64, spts, scode, skey, cv, cuts, nodes, nbox, root, q, hint, lambda, delta, ctr, st);
   else if (dp == 4) far_dp<4>(fp64, spts, scode, skey, cv, cuts, nodes, nbox, root, q, hint, lambda, delta, ctr, st);
   else far_dp<8>(fp64, spts, scode, skey, cv, cuts, nodes, nbox, root, q, hint, lambda, delta, ctr, st);
-  k_far_count<<<1, 1, 0, st>>>(ctr);
-  count_launches(3);
+  count_launches(2);
 }
 
 }  // namespace dpc

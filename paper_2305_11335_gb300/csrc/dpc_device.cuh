@@ -152,6 +152,24 @@ __device__ __forceinline__ unsigned long long key_code(unsigned long long key, i
 // 8-bit radix passes that sort keys of S + ib bits.
 __host__ __device__ __forceinline__ int sort_passes(int S, int ib) { return (S + ib + 7) / 8; }
 
+// Digit counts of every radix pass, in shared memory [8][256] (CTA-wide calls).
+__device__ __forceinline__ void rs_clear_digits(uint32_t (*cnt)[256]) {
+  for (int i = threadIdx.x; i < 8 * 256; i += blockDim.x) (&cnt[0][0])[i] = 0u;
+  __syncthreads();
+}
+__device__ __forceinline__ void rs_count_digits(uint32_t (*cnt)[256], unsigned long long key, int npass) {
+#pragma unroll
+  for (int p = 0; p < 8; ++p)
+    if (p < npass) atomicAdd(&cnt[p][(key >> (8 * p)) & 255u], 1u);
+}
+__device__ __forceinline__ void rs_flush_digits(uint32_t (*cnt)[256], uint32_t* __restrict__ count, int npass) {
+  __syncthreads();
+  for (int i = threadIdx.x; i < npass * 256 && i < 8 * 256; i += blockDim.x) {
+    const uint32_t v = (&cnt[0][0])[i];
+    if (v) atomicAdd(&count[i], v);
+  }
+}
+
 // Per (instance, cutoff) parameters.  Fields marked [host] are filled before
 // the launch; the others by the setup kernels.
 struct CutGeom {

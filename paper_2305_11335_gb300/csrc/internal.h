@@ -66,8 +66,9 @@ void launch_group_geometry(const ClassView& cv, const CutGeom* cuts, int ncut, u
                            CutGeom* geo, cudaStream_t st);
 // cut ([ninst]) takes the level, radius and far bounds of geo ([ninst])
 void launch_adopt_geometry(const ClassView& cv, const CutGeom* geo, CutGeom* cut, cudaStream_t st);
+// (count: the digit counts of launch_sort_clear, or null)
 void launch_codes(const void* pts, int dtype, const ClassView& cv, int g, unsigned long long* codes,
-                  uint32_t* ids, cudaStream_t st);
+                  uint32_t* ids, uint32_t* count, cudaStream_t st);
 void launch_gather(const void* pts, int dtype, const ClassView& cv, int dp,
                    const unsigned long long* codes_a, const unsigned long long* codes_b,
                    const uint32_t* ids_a, const uint32_t* ids_b, float* spts,
@@ -78,23 +79,33 @@ void launch_cells(const unsigned long long* scode, const ClassView& cv, int g, c
                   cudaStream_t st);
 
 // ---- radix sort (sort.cu) ------------------------------------------------------
-constexpr uint32_t kSortTile = 4096;    // items per tile of one pass
-constexpr uint32_t kSortMaxPasses = 8;  // 8-bit digits of a 64-bit key
-// 32-bit words of sort scratch for n items: per tile and digit a published
-// 64-bit count, the digit counts and starts of every pass, a tile counter per
-// pass (and slack)
+constexpr uint32_t kSortMaxPasses = 8;   // 8-bit digits of a 64-bit key
+constexpr uint32_t kSortSmall = 1u << 17, kSortMiddle = 1u << 21;  // tiles of 1024, 2048 items up to here
+// 32-bit words of sort scratch that serve every size up to n: per tile and
+// digit a published 64-bit count, the digit counts of every pass, a tile
+// counter per pass (and slack)
 constexpr size_t sort_hist_words_for(uint64_t n) {
-  return (size_t)(n ? (n + kSortTile - 1) / kSortTile : 1) * 256u * 2u +
-         2u * kSortMaxPasses * 256u + kSortMaxPasses + 8u;
+  const uint64_t a = ((n < kSortSmall ? n : kSortSmall) + 1023) / 1024;
+  const uint64_t b = ((n < kSortMiddle ? n : kSortMiddle) + 2047) / 2048;
+  const uint64_t c = (n + 4095) / 4096;
+  const uint64_t ab = a > b ? a : b, t = ab > c ? ab : c;
+  return (size_t)(t ? t : 1) * 256u * 2u + kSortMaxPasses * 256u + kSortMaxPasses + 8u;
 }
 size_t sort_hist_words(uint32_t n);
 // one-time kernel attribute setup (called before any stream capture)
 void sort_init();
+// Clears the scratch for a sort of n items and returns the digit counts
+// [kSortMaxPasses][256] for a kernel that fills them (rs_count_digits in
+// dpc_device.cuh) ahead of launch_sort(counted = true).  Worth it up to
+// kSortMiddle points; beyond, the shared-memory atomics cost the code kernel more
+// than one more read of the keys (1e7 points in 3-D: binning 1.36 ms counted, 1.32
+// not).
+uint32_t* launch_sort_clear(uint32_t n, uint32_t* hist, cudaStream_t st);
 // Sorts (codes_a, ids_a) by code, LSD over the device-side pass count
 // sort_passes(cls->S, cls->ib); the result lands in the _a buffers if that
 // count is even, else in _b.
 void launch_sort(unsigned long long* codes_a, unsigned long long* codes_b, uint32_t* ids_a,
-                 uint32_t* ids_b, uint32_t n, const ClassGeom* cls, uint32_t* hist,
+                 uint32_t* ids_b, uint32_t n, const ClassGeom* cls, uint32_t* hist, bool counted,
                  cudaStream_t st);
 
 // ---- radix tree (tree.cu) ------------------------------------------------------
@@ -148,7 +159,8 @@ struct MultiCut {
 // 0: always tensor).
 // rho of every point for one cutoff (cuts: [ninst]); rho_out is indexed by
 // output index (sid); d: the largest dimension of the class
-void launch_density(int dp, int g, int d, bool fp64, int layout, const float* spts,
+// (prec: 0 float32 filter, 1 binary64, 2 binary64 mode on int32 points)
+void launch_density(int dp, int g, int d, int prec, int layout, const float* spts,
                     const unsigned long long* scode, const uint32_t* sid, const ClassView& cv,
                     const CutGeom* cuts, HashInfo* hi, const unsigned long long* hkeys,
                     const uint2* hvals, uint4* pieces, int32_t* rho_out,
@@ -157,7 +169,7 @@ void launch_density(int dp, int g, int d, bool fp64, int layout, const float* sp
 // rho of the cutoffs of `mc` in one pass over the blocks of `geo` ([ninst]; the
 // hash holds its level's cells): tensor tiles for dp = 8 with the float32
 // filter, segments otherwise.  No order keys are written.
-void launch_density_multi(int dp, int g, int d, bool fp64, const float* spts, const unsigned long long* scode,
+void launch_density_multi(int dp, int g, int d, int prec, const float* spts, const unsigned long long* scode,
                           const uint32_t* sid, const ClassView& cv, const CutGeom* geo, HashInfo* hi,
                           const unsigned long long* hkeys, const uint2* hvals, uint4* pieces,
                           const MultiCut& mc, Counters* ctr, cudaStream_t st, int seg_cells,

@@ -425,11 +425,13 @@ k_small_labels(const int32_t* __restrict__ rho, const int32_t* __restrict__ lamb
     const InstDev I = cv.instance(inst);
     const LabelParams P = params ? params[inst] : one;
     const int32_t n = (int32_t)I.n;
+#pragma unroll 4
     for (int32_t i = threadIdx.x; i < n; i += kLabelThreads) {
-      const int32_t r = rho[I.out + i], l = lambda[I.out + i];
+      const int32_t r = __ldg(rho + I.out + i), l = __ldg(lambda + I.out + i);
+      const double dl = __ldg(delta + I.out + i);
       int32_t v;
       if (r < P.rho_noise) v = -1;                                                 // Definition 4
-      else if (l < 0 || (r >= P.rho_min && delta[I.out + i] >= P.delta_min)) v = i;  // Definition 5
+      else if (l < 0 || (r >= P.rho_min && dl >= P.delta_min)) v = i;  // Definition 5
       else v = l < n ? l : -1;
       s_par[i] = v;
     }

@@ -144,13 +144,13 @@ extern "C" int dpc_density_static(const void* pts, int dtype, int64_t n, int32_t
     launch_class_init(cv, g, 0, std::min(kMaxBits, 63 / g), status, st);
     launch_bbox(pts, dtype, cv, g, st);
     launch_setup(cv, cut, 1, nullptr, &ch, st);
-    launch_codes(pts, dtype, cv, g, codes_a, ids_a, st);
-    launch_sort(codes_a, codes_b, ids_a, ids_b, nn, cls, hist, st);
+    launch_codes(pts, dtype, cv, g, codes_a, ids_a, launch_sort_clear(nn, hist, st), st);
+    launch_sort(codes_a, codes_b, ids_a, ids_b, nn, cls, hist, true, st);
     launch_gather(pts, dtype, cv, dp, codes_a, codes_b, ids_a, ids_b, spts, scode, sid, st);
     launch_cells(scode, cv, g, cut, hinfo, hkeys, hvals, kStaticHash, st);
     const bool f64 = prec == DPC_PREC_FP64;
     const int layout = dp == 8 && !f64 ? kLayoutTensor : (g >= 2 ? kLayoutSegment : kLayoutUnion);
-    launch_density(dp, g, d, f64, layout, spts, scode, sid, cv, cut, hinfo, hkeys, hvals,
+    launch_density(dp, g, d, f64 ? (dtype == DPC_I32 ? 2 : 1) : 0, layout, spts, scode, sid, cv, cut, hinfo, hkeys, hvals,
                    (uint4*)(base + kOffPieces), rho, skey, ctr, st, 0, 2);
   }
   if (cudaGetLastError() != cudaSuccess) return DPC_ERR_CUDA;

@@ -36,6 +36,7 @@ __global__ void k_tree_build(const unsigned long long* __restrict__ code, ClassV
   const int S = cv.cls->S, ib = cv.cls->ib;
   for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t + 1 < n; t += gridDim.x * blockDim.x) {
     const int i = (int)t;
+    if (t == 0u) nodes[0].parent = 0u;  // (the class's root: no other thread writes it)
     const int dir = (prefix_len(code, n, i, i + 1) - prefix_len(code, n, i, i - 1)) >= 0 ? 1 : -1;
     const int dmin = prefix_len(code, n, i, i - dir);
     int lmax = 2;
@@ -83,8 +84,6 @@ __global__ void k_tree_build(const unsigned long long* __restrict__ code, ClassV
     }
   }
 }
-
-__global__ void k_root_parent(Node* nodes) { nodes[0].parent = 0u; }
 
 // Bottom-up pass: the second child to arrive at a node computes its largest
 // key and, on the first pass after a binning, its bounding box over all DP
@@ -310,8 +309,7 @@ void launch_tree_build(const unsigned long long* scode, const ClassView& cv, Nod
   cudaMemsetAsync(root, 0xff, sizeof(uint32_t) * cv.ninst, st);
   if (cv.N < 2) return;
   k_tree_build<<<grid_for(cv.N - 1), kThreads, 0, st>>>(scode, cv, nodes, leaf_parent, root);
-  k_root_parent<<<1, 1, 0, st>>>(nodes);
-  count_launches(2);
+  count_launches(1);
 }
 
 template <int DP>
