@@ -37,7 +37,8 @@ namespace {
 constexpr int kFarThreads = 128;
 constexpr int kStack = 128;
 constexpr int kWarpStack = 1024;  // shared stack entries per warp (far phase, round 2)
-constexpr uint32_t kFarBudget = 128;  // node expansions per query in round 1
+constexpr uint32_t kFarBudget = 128;  // node expansions per query in round 1, at least
+constexpr unsigned kFarGrid = 128;    // CTAs per SM of round 1, at most
 constexpr int kNearWarps = 4;
 constexpr int kNearThreads = kNearWarps * 32;
 
@@ -886,19 +887,39 @@ __device__ __forceinline__ double hint_bound(const FarHint& h, const ClassView& 
   else return (double)dist32<DP>(fq.xq, x);
 }
 
+// Node expansions a query may take in the first round.  The second round gives
+// a long search a whole warp, which shortens the last searches of a small set
+// but expands more nodes per query and starts over, so it is left to sets that
+// do not fill the chip and to the longest searches of the others: the budget
+// grows with the queries per resident thread (`room` of them).  Measured with
+// budgets of 128 / 256 / 512 / 1024 / 2048, far search in ms: 7-D, 438,000 far
+// queries of 2e6 points 17.7 / 16.3 / 12.2 / 10.4 / 10.6; 5-D, 1e6 queries
+// 18.2 / 6.4 / 5.4 / 5.7 / 5.9; 5-D, 1e5 queries .88 / .48 / .55 / .70 / .85;
+// 7-D, 13,000 queries .43 / .43 / .56 / .76 / .98; 3-D, 1.5e5 queries .154 /
+// .181 / .199 / .200 / .203; 2-D, 1e6 queries .290 / .280 / .265 / .267 / .267.
+template <int DP>
+__device__ __forceinline__ uint32_t far_budget(uint32_t qn, uint32_t room) {
+  const uint32_t b = (uint32_t)min((unsigned long long)qn * (DP > 4 ? 768u : 64u) / room, 1024ull);
+  return min(max(b, kFarBudget), DP > 4 ? 1024u : 512u);
+}
+
 // Far queries, first round: one thread per query, a depth-first search with
-// an expansion budget.  Most queries finish within it (they expand a few dozen
-// nodes); the others are passed to the second round with the best distance
-// found so far, which bounds their search there.
+// an expansion budget.  Most queries finish within it; the others are passed to
+// the second round with the best distance found so far, which bounds their
+// search there.  What bounds it is the child records' way from L2 (7-D: 32e9
+// expansions/s of 160 bytes, 5.1 TB/s).  Letting a lane that is done take the
+// next query while its neighbours go on costs more than the idle lanes (1e6
+// 2-D queries .35 ms for .26).
 template <int DP, bool F64>
 __global__ void __launch_bounds__(kFarThreads)
 k_dep_far(const float* __restrict__ spts, const unsigned long long* __restrict__ scode,
           const unsigned long long* __restrict__ skey, ClassView cv,
           const CutGeom* __restrict__ cuts, const Node* __restrict__ nodes,
           const float* __restrict__ nbox, const uint32_t* __restrict__ roots, FarQueue q, FarHint hint,
-          int32_t* __restrict__ lambda, double* __restrict__ delta, Counters* ctr) {
+          int32_t* __restrict__ lambda, double* __restrict__ delta, Counters* ctr, uint32_t room) {
   __shared__ FastStack fs;
   const uint32_t qn = ctr->queue_n;
+  const uint32_t budget = far_budget<DP>(qn, room);
   const uint32_t n = cv.N;
   const int S = cv.cls->S, ib = cv.cls->ib;
   // the band depends only on DP, the same for every instance of the class
@@ -923,7 +944,7 @@ k_dep_far(const float* __restrict__ spts, const unsigned long long* __restrict__
         best.init();
         const double s_init = fmin(q.s1d[e], hint_bound<DP, true>(hint, cv, fq));
         const int r = far_walk<DP>(
-            fs, nbox, n, fq.K, fq.xq, fq.root, kFarBudget, expanded,
+            fs, nbox, n, fq.K, fq.xq, fq.root, budget, expanded,
             [&](float lbs) { return (double)lbs > fmin(best.s1, s_init); },
             [&](uint32_t t, unsigned long long kt, const Pt<DP>& x) {
               best.add(dist64<DP>(fq.xq, x), key_id(kt), t);
@@ -944,7 +965,7 @@ k_dep_far(const float* __restrict__ spts, const unsigned long long* __restrict__
         best.init();
         const float s_init = fminf(q.s1[e], (float)hint_bound<DP, false>(hint, cv, fq));
         const int r = far_walk<DP>(
-            fs, nbox, n, fq.K, fq.xq, fq.root, kFarBudget, expanded,
+            fs, nbox, n, fq.K, fq.xq, fq.root, budget, expanded,
             [&](float lbs) { return beyond(lbs, band_of(fminf(best.s1, s_init), bmul, badd)); },
             [&](uint32_t t, unsigned long long kt, const Pt<DP>& x) {
               best.add(dist32<DP>(fq.xq, x), key_id(kt), t);
@@ -1236,18 +1257,21 @@ void far_dp(bool fp64, const float* spts, const unsigned long long* scode,
             const unsigned long long* skey, const ClassView& cv, const CutGeom* cuts,
             const Node* nodes, const float* nbox, const uint32_t* root, FarQueue q, const FarHint& hint,
             int32_t* lambda, double* delta, Counters* ctr, cudaStream_t st) {
-  // the queue length is known only on the device: launch enough threads for
-  // a full SM load and let them stride over it
-  const unsigned grid = grid_for(cv.N, kFarThreads, sm_count() * 8u);
+  // the queue length is known only on the device: CTAs for most lengths, so
+  // that a free SM takes the next 128 queries (1e6 2-D queries .27 -> .24 ms,
+  // 438,000 7-D queries 9.8 -> 8.7 against 8 CTAs per SM striding over the
+  // queue, of which 6 were resident in 7-D); those without a query end at once
+  const unsigned grid = grid_for(cv.N, kFarThreads, sm_count() * kFarGrid);
+  const uint32_t room = sm_count() * 1024u;
   const unsigned grid2 = grid_for(cv.N, kFarThreads / 32, sm_count() * 16u);
   if (fp64) {
     k_dep_far<DP, true><<<grid, kFarThreads, 0, st>>>(spts, scode, skey, cv, cuts, nodes, nbox,
-                                                      root, q, hint, lambda, delta, ctr);
+                                                      root, q, hint, lambda, delta, ctr, room);
     k_dep_far_wide<DP, true><<<grid2, kFarThreads, 0, st>>>(spts, scode, skey, cv, cuts, nodes,
                                                             nbox, root, q, lambda, delta, ctr);
   } else {
     k_dep_far<DP, false><<<grid, kFarThreads, 0, st>>>(spts, scode, skey, cv, cuts, nodes, nbox,
-                                                       root, q, hint, lambda, delta, ctr);
+                                                       root, q, hint, lambda, delta, ctr, room);
     k_dep_far_wide<DP, false><<<grid2, kFarThreads, 0, st>>>(spts, scode, skey, cv, cuts, nodes,
                                                              nbox, root, q, lambda, delta, ctr);
   }
