@@ -247,7 +247,6 @@ struct Workspace {
   Node* nodes = nullptr;
   float* nbox = nullptr;    // per-node child records of the radix tree (dpc_device.cuh)
   bool boxes_ready = false; // nbox matches the current binning
-  uint32_t* leaf_parent = nullptr;
   uint32_t* visit = nullptr;
   uint4* pieces = nullptr;        // pieces of up to 128 points (tensor-core layouts)
   uint32_t* qpos = nullptr;
@@ -397,7 +396,7 @@ struct Workspace {
     const size_t o_hk = take(8 * (size_t)hc), o_hv = take(8 * (size_t)hc);
     const size_t o_nodes = take(sizeof(Node) * N);
     const size_t o_nbox = take(4 * (size_t)kRecWordsMax * N);
-    const size_t o_lp = take(4 * N), o_visit = take(4 * N);
+    const size_t o_visit = take(4 * N);
     const size_t o_pieces = take(sizeof(uint4) * N);
     const size_t o_qpos = take(4 * N), o_qs1 = take(4 * N), o_qs1d = take(8 * N);
     const size_t o_qpos2 = take(4 * N), o_qs1_2 = take(4 * N), o_qs1d2 = take(8 * N);
@@ -436,7 +435,6 @@ struct Workspace {
     hcap = hc;
     nodes = (Node*)(b + o_nodes);
     nbox = (float*)(b + o_nbox);
-    leaf_parent = (uint32_t*)(b + o_lp);
     visit = (uint32_t*)(b + o_visit);
     pieces = (uint4*)(b + o_pieces);
     qpos = (uint32_t*)(b + o_qpos);
@@ -759,7 +757,7 @@ FarQueue queue_of(Workspace* w) {
 
 void tree_step(Workspace* w, const ClassView& cv) {
   Phase ph(w, DPC_PHASE_TREE);
-  launch_tree_build(w->scode, cv, w->nodes, w->leaf_parent, w->roots, w->stream);
+  launch_tree_build(w->scode, cv, w->nodes, w->roots, w->stream);
 }
 
 void cells_step(Workspace* w, const ClassPlan& c, const ClassView& cv, const CutGeom* cuts) {
@@ -790,7 +788,7 @@ void dependent_step(Workspace* w, const ClassPlan& c, const ClassView& cv, CutGe
   cudaStream_t st = w->stream;
   {
     Phase ph(w, DPC_PHASE_MAXKEY);
-    launch_tree_maxkey(w->skey, w->spts, c.dp, cv.N, w->nodes, w->leaf_parent, w->visit, w->nbox,
+    launch_tree_maxkey(w->skey, w->spts, c.dp, c.dmax, cv.N, w->nodes, w->visit, w->nbox,
                        !w->boxes_ready, st);
     w->boxes_ready = true;
   }
@@ -804,13 +802,13 @@ void dependent_step(Workspace* w, const ClassPlan& c, const ClassView& cv, CutGe
       launch_dep_near_tc(c.dmax, w->spts, w->scode, w->sid, w->skey, cv, rho_skip, pts, dtype, cuts, w->hinfo,
                          w->hkeys, w->hvals, w->pieces, lambda, delta, queue_of(w), w->ctr, min_fill, st);
       if (min_fill)  // sparse cells
-        launch_dep_near(c.dp, c.g, fp64, kLayoutTree, w->spts, w->scode, w->skey, cv, rho_skip, pts, dtype, cuts,
+        launch_dep_near(c.dp, c.g, c.dmax, fp64, kLayoutTree, w->spts, w->scode, w->skey, cv, rho_skip, pts, dtype, cuts,
                         w->hinfo, w->hkeys, w->hvals, lambda, delta, queue_of(w), w->ctr, st, w->nbox, w->roots, seg_cells,
                         min_fill);
     } else {
       // the tensor layout exists for 5-8 dimensions with the float32 filter
       if (layout == kLayoutTensor) layout = kLayoutUnion;
-      launch_dep_near(c.dp, c.g, fp64, layout, w->spts, w->scode, w->skey, cv, rho_skip, pts, dtype,
+      launch_dep_near(c.dp, c.g, c.dmax, fp64, layout, w->spts, w->scode, w->skey, cv, rho_skip, pts, dtype,
                       cuts, w->hinfo, w->hkeys, w->hvals, lambda, delta, queue_of(w), w->ctr, st,
                       w->nbox, w->roots, seg_cells);
     }
@@ -819,7 +817,7 @@ void dependent_step(Workspace* w, const ClassPlan& c, const ClassView& cv, CutGe
   }
   {
     Phase ph(w, DPC_PHASE_FAR);
-    launch_dep_far(c.dp, fp64, w->spts, w->scode, w->skey, cv, cuts, w->nodes, w->nbox, w->roots,
+    launch_dep_far(c.dp, c.dmax, fp64, w->spts, w->scode, w->skey, cv, cuts, w->nodes, w->nbox, w->roots,
                    queue_of(w), hint, lambda, delta, w->ctr, st);
   }
 }
@@ -1014,7 +1012,7 @@ Choice choose(Workspace* w, const ClassPlan& c, const ClassView& cv, CutGeom* cu
         if (timed) cudaEventRecord(w->tune_ev[2 + l], st);
       }
       if (!near) return;
-      launch_tree_maxkey(w->skey, w->spts, c.dp, cv.N, w->nodes, w->leaf_parent, w->visit, w->nbox,
+      launch_tree_maxkey(w->skey, w->spts, c.dp, c.dmax, cv.N, w->nodes, w->visit, w->nbox,
                          !w->boxes_ready, st);
       w->boxes_ready = true;
       if (timed) cudaEventRecord(w->tune_ev[6], st);
@@ -1032,11 +1030,11 @@ Choice choose(Workspace* w, const ClassPlan& c, const ClassView& cv, CutGeom* cu
                                  cuts, w->hinfo, w->hkeys, w->hvals, w->pieces, near->lambda,
                                  near->delta, queue_of(w), w->ctr, 0, st);
             else
-              launch_dep_near(c.dp, c.g, fp64, nlays[l], w->spts, w->scode, w->skey, cv, 0,
+              launch_dep_near(c.dp, c.g, c.dmax, fp64, nlays[l], w->spts, w->scode, w->skey, cv, 0,
                               near->pts, near->dtype, cuts, w->hinfo, w->hkeys, w->hvals,
                               near->lambda, near->delta, queue_of(w), w->ctr, st,
                               w->nbox, w->roots, default_seg_cells(c.g));
-            launch_dep_far(c.dp, fp64, w->spts, w->scode, w->skey, cv, cuts, w->nodes, w->nbox,
+            launch_dep_far(c.dp, c.dmax, fp64, w->spts, w->scode, w->skey, cv, cuts, w->nodes, w->nbox,
                            w->roots, queue_of(w), FarHint(), near->lambda, near->delta, w->ctr, st);
           }
           if (timed) cudaEventRecord(w->tune_ev[8 + (kNL + 1) * sh + l], st);

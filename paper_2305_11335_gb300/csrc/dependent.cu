@@ -605,7 +605,7 @@ k_dep_near_seg(const float* __restrict__ spts, const unsigned long long* __restr
 // 1e6 points in 2-D: near phase and far search 0.53 + 0.21 ms with the blocks
 // scanned, 0.03 + 0.54 with the tree searched unbounded, 0.04 + 0.46 with this
 // bound, 0.04 + 0.29 with the walk of far_walk.
-template <int DP, int ND>
+template <int DP, int ND, int RD>
 __global__ void __launch_bounds__(kNearThreads)
 k_near_to_far(const float* __restrict__ spts, const unsigned long long* __restrict__ skey, ClassView cv,
               const CutGeom* __restrict__ cuts, int32_t rho_skip, int32_t* __restrict__ lambda,
@@ -673,7 +673,7 @@ k_near_to_far(const float* __restrict__ spts, const unsigned long long* __restri
     bool top = false;
     if (valid && !skip && root < cv.N - 1u) {  // (kNoNode: an instance of one point)
       const unsigned long long* rk =
-          reinterpret_cast<const unsigned long long*>(nbox + (size_t)root * rec_words<DP>() + 4);
+          reinterpret_cast<const unsigned long long*>(nbox + (size_t)root * rec_words<RD>() + 4);
       top = rk[0] <= K && rk[1] <= K;
     }
     if (top) {
@@ -701,14 +701,14 @@ k_near_to_far(const float* __restrict__ spts, const unsigned long long* __restri
 // far phase: depth-first priority search of the radix tree
 
 // Squared lower bound between the query and the bounding box of a subtree
-// (all coordinates; box layout [lo(DP) | hi(DP)] per node, tree.cu), scaled
+// (all coordinates; box layout [lo(RD) | hi(RD)] per node, tree.cu), scaled
 // 1e-5 down so that it stays below the float32 distance of every point inside
 // despite the rounding of this evaluation and of dist32.
-template <int DP>
-__device__ __forceinline__ float rec_lb2(const ChildRec<DP>& r, int s, const Pt<DP>& x) {
+template <int DP, int RD>
+__device__ __forceinline__ float rec_lb2(const ChildRec<RD>& r, int s, const Pt<DP>& x) {
   float lb2 = 0.f;
 #pragma unroll
-  for (int a = 0; a < DP; ++a) {
+  for (int a = 0; a < RD; ++a) {
     const float l = fmaxf(fmaxf(r.lo[s][a] - x.x[a], x.x[a] - r.hi[s][a]), 0.f);
     lb2 = fmaf(l, l, lb2);
   }
@@ -716,11 +716,11 @@ __device__ __forceinline__ float rec_lb2(const ChildRec<DP>& r, int s, const Pt<
 }
 
 // A leaf child's point, from its record (its box is the point itself).
-template <int DP>
-__device__ __forceinline__ Pt<DP> rec_point(const ChildRec<DP>& r, int s) {
+template <int DP, int RD>
+__device__ __forceinline__ Pt<DP> rec_point(const ChildRec<RD>& r, int s) {
   Pt<DP> p;
 #pragma unroll
-  for (int a = 0; a < DP; ++a) p.x[a] = r.lo[s][a];
+  for (int a = 0; a < DP; ++a) p.x[a] = a < RD ? r.lo[s][a < RD ? a : 0] : 0.f;
   return p;
 }
 
@@ -732,7 +732,7 @@ enum { kWalkDone = 0, kWalkBudget = 1, kWalkBad = -1 };
 // children's indices, keys and boxes).  Stops with kWalkBudget after `budget` node expansions, and
 // with kWalkBad on a malformed tree or stack overflow (neither happens for a
 // tree built by tree.cu: its depth is at most 64 + 32).
-template <int DP, typename Prune, typename Visit>
+template <int DP, int RD, typename Prune, typename Visit>
 __device__ __noinline__ int tree_walk_from(const Node* __restrict__ nodes,
                                            const float* __restrict__ nbox, uint32_t n,
                                            const unsigned long long* __restrict__ skey,
@@ -752,7 +752,7 @@ __device__ __noinline__ int tree_walk_from(const Node* __restrict__ nodes,
     if (ni + 1 >= n) return kWalkBad;
     if (expanded >= budget) return kWalkBudget;
     ++expanded;
-    const ChildRec<DP> r = load_rec<DP>(nbox, ni);
+    const ChildRec<RD> r = load_rec<RD>(nbox, ni);
     uint32_t keep[2];
     float keepl[2];
     int nk = 0;
@@ -762,9 +762,9 @@ __device__ __noinline__ int tree_walk_from(const Node* __restrict__ nodes,
       if (r.key[s] <= K) continue;  // nothing of higher key below
       if (c & kLeafBit) {
         if ((c & ~kLeafBit) >= n) return kWalkBad;
-        visit(c & ~kLeafBit, r.key[s], rec_point<DP>(r, s));
+        visit(c & ~kLeafBit, r.key[s], rec_point<DP, RD>(r, s));
       } else {
-        const float lbs = rec_lb2<DP>(r, s, xq);
+        const float lbs = rec_lb2<DP, RD>(r, s, xq);
         if (prune(lbs)) continue;
         keep[nk] = c;
         keepl[nk] = lbs;
@@ -793,7 +793,7 @@ struct FastStack {
   float lb[kFastStack][kFarThreads];
 };
 
-template <int DP, typename Prune, typename Visit>
+template <int DP, int RD, typename Prune, typename Visit>
 __device__ __forceinline__ int far_walk(FastStack& fs, const float* __restrict__ nbox, uint32_t n,
                                         unsigned long long K, const Pt<DP>& xq, uint32_t start, uint32_t budget,
                                         uint32_t& expanded, Prune prune, Visit visit) {
@@ -806,12 +806,12 @@ __device__ __forceinline__ int far_walk(FastStack& fs, const float* __restrict__
     if (ni + 1 >= n) return kWalkBad;
     if (expanded >= budget) return kWalkBudget;
     ++expanded;
-    const ChildRec<DP> r = load_rec<DP>(nbox, ni);
+    const ChildRec<RD> r = load_rec<RD>(nbox, ni);
     const bool h0 = r.key[0] > K, h1 = r.key[1] > K;  // something of higher key below
     const bool leaf0 = r.child[0] & kLeafBit, leaf1 = r.child[1] & kLeafBit;
-    if (h0 && leaf0) visit(r.child[0] & ~kLeafBit, r.key[0], rec_point<DP>(r, 0));
-    if (h1 && leaf1) visit(r.child[1] & ~kLeafBit, r.key[1], rec_point<DP>(r, 1));
-    const float l0 = rec_lb2<DP>(r, 0, xq), l1 = rec_lb2<DP>(r, 1, xq);
+    if (h0 && leaf0) visit(r.child[0] & ~kLeafBit, r.key[0], rec_point<DP, RD>(r, 0));
+    if (h1 && leaf1) visit(r.child[1] & ~kLeafBit, r.key[1], rec_point<DP, RD>(r, 1));
+    const float l0 = rec_lb2<DP, RD>(r, 0, xq), l1 = rec_lb2<DP, RD>(r, 1, xq);
     const bool g0 = h0 && !leaf0 && !prune(l0), g1 = h1 && !leaf1 && !prune(l1);
     if (g0 && g1) {
       const bool first = l0 < l1;
@@ -910,7 +910,7 @@ __device__ __forceinline__ uint32_t far_budget(uint32_t qn, uint32_t room) {
 // expansions/s of 160 bytes, 5.1 TB/s).  Letting a lane that is done take the
 // next query while its neighbours go on costs more than the idle lanes (1e6
 // 2-D queries .35 ms for .26).
-template <int DP, bool F64>
+template <int DP, int RD, bool F64>
 __global__ void __launch_bounds__(kFarThreads)
 k_dep_far(const float* __restrict__ spts, const unsigned long long* __restrict__ scode,
           const unsigned long long* __restrict__ skey, ClassView cv,
@@ -943,7 +943,7 @@ k_dep_far(const float* __restrict__ spts, const unsigned long long* __restrict__
         Best<double> best;
         best.init();
         const double s_init = fmin(q.s1d[e], hint_bound<DP, true>(hint, cv, fq));
-        const int r = far_walk<DP>(
+        const int r = far_walk<DP, RD>(
             fs, nbox, n, fq.K, fq.xq, fq.root, budget, expanded,
             [&](float lbs) { return (double)lbs > fmin(best.s1, s_init); },
             [&](uint32_t t, unsigned long long kt, const Pt<DP>& x) {
@@ -964,7 +964,7 @@ k_dep_far(const float* __restrict__ spts, const unsigned long long* __restrict__
         Best<float> best;
         best.init();
         const float s_init = fminf(q.s1[e], (float)hint_bound<DP, false>(hint, cv, fq));
-        const int r = far_walk<DP>(
+        const int r = far_walk<DP, RD>(
             fs, nbox, n, fq.K, fq.xq, fq.root, budget, expanded,
             [&](float lbs) { return beyond(lbs, band_of(fminf(best.s1, s_init), bmul, badd)); },
             [&](uint32_t t, unsigned long long kt, const Pt<DP>& x) {
@@ -984,7 +984,7 @@ k_dep_far(const float* __restrict__ spts, const unsigned long long* __restrict__
           if (best.s2 <= b) {  // near tie: re-rank the band in binary64
             ++rescans;
             uint32_t more = 0;
-            bad |= tree_walk_from<DP>(
+            bad |= tree_walk_from<DP, RD>(
                        nodes, nbox, n, skey, fq.K, fq.xq, fq.root, 0xffffffffu, more,
                        [&](float lbs) { return beyond(lbs, b); },
                        [&](uint32_t t, unsigned long long kt, const Pt<DP>& x) {
@@ -1032,7 +1032,7 @@ k_dep_far(const float* __restrict__ spts, const unsigned long long* __restrict__
 // the warp's shared stack, each lane expands its node, and the survivors are
 // pushed with a warp prefix sum.  Children that do not fit on the stack are
 // searched by their lane alone.
-template <int DP, bool F64>
+template <int DP, int RD, bool F64>
 __global__ void __launch_bounds__(kFarThreads)
 k_dep_far_wide(const float* __restrict__ spts, const unsigned long long* __restrict__ scode,
                const unsigned long long* __restrict__ skey, ClassView cv,
@@ -1085,7 +1085,7 @@ k_dep_far_wide(const float* __restrict__ spts, const unsigned long long* __restr
               bad = true;
             } else {
               ++expanded;
-              const ChildRec<DP> r = load_rec<DP>(nbox, ni);
+              const ChildRec<RD> r = load_rec<RD>(nbox, ni);
 #pragma unroll
               for (int s = 0; s < 2; ++s) {
                 const uint32_t c = r.child[s];
@@ -1095,9 +1095,9 @@ k_dep_far_wide(const float* __restrict__ spts, const unsigned long long* __restr
                     bad = true;
                     continue;
                   }
-                  visit(c & ~kLeafBit, r.key[s], rec_point<DP>(r, s));
+                  visit(c & ~kLeafBit, r.key[s], rec_point<DP, RD>(r, s));
                 } else {
-                  const float l = rec_lb2<DP>(r, s, fq.xq);
+                  const float l = rec_lb2<DP, RD>(r, s, fq.xq);
                   if (prune(l)) continue;
                   keep[nk] = c;
                   keepl[nk] = l;
@@ -1125,7 +1125,7 @@ k_dep_far_wide(const float* __restrict__ spts, const unsigned long long* __restr
             stk[pos + s] = keep[s];
             stl[pos + s] = keepl[s];
           } else {  // no room: this lane searches the subtree alone
-            bad |= tree_walk_from<DP>(nodes, nbox, n, skey, fq.K, fq.xq, keep[s], 0xffffffffu,
+            bad |= tree_walk_from<DP, RD>(nodes, nbox, n, skey, fq.K, fq.xq, keep[s], 0xffffffffu,
                                       expanded, prune, visit) != kWalkDone;
           }
         }
@@ -1252,7 +1252,7 @@ void near_dg(bool fp64, int layout, const float* spts, const unsigned long long*
   }
 }
 
-template <int DP>
+template <int DP, int RD>
 void far_dp(bool fp64, const float* spts, const unsigned long long* scode,
             const unsigned long long* skey, const ClassView& cv, const CutGeom* cuts,
             const Node* nodes, const float* nbox, const uint32_t* root, FarQueue q, const FarHint& hint,
@@ -1265,21 +1265,21 @@ void far_dp(bool fp64, const float* spts, const unsigned long long* scode,
   const uint32_t room = sm_count() * 1024u;
   const unsigned grid2 = grid_for(cv.N, kFarThreads / 32, sm_count() * 16u);
   if (fp64) {
-    k_dep_far<DP, true><<<grid, kFarThreads, 0, st>>>(spts, scode, skey, cv, cuts, nodes, nbox,
+    k_dep_far<DP, RD, true><<<grid, kFarThreads, 0, st>>>(spts, scode, skey, cv, cuts, nodes, nbox,
                                                       root, q, hint, lambda, delta, ctr, room);
-    k_dep_far_wide<DP, true><<<grid2, kFarThreads, 0, st>>>(spts, scode, skey, cv, cuts, nodes,
+    k_dep_far_wide<DP, RD, true><<<grid2, kFarThreads, 0, st>>>(spts, scode, skey, cv, cuts, nodes,
                                                             nbox, root, q, lambda, delta, ctr);
   } else {
-    k_dep_far<DP, false><<<grid, kFarThreads, 0, st>>>(spts, scode, skey, cv, cuts, nodes, nbox,
+    k_dep_far<DP, RD, false><<<grid, kFarThreads, 0, st>>>(spts, scode, skey, cv, cuts, nodes, nbox,
                                                        root, q, hint, lambda, delta, ctr, room);
-    k_dep_far_wide<DP, false><<<grid2, kFarThreads, 0, st>>>(spts, scode, skey, cv, cuts, nodes,
+    k_dep_far_wide<DP, RD, false><<<grid2, kFarThreads, 0, st>>>(spts, scode, skey, cv, cuts, nodes,
                                                              nbox, root, q, lambda, delta, ctr);
   }
 }
 
 }  // namespace
 
-void launch_dep_near(int dp, int g, bool fp64, int layout, const float* spts,
+void launch_dep_near(int dp, int g, int dmax, bool fp64, int layout, const float* spts,
                      const unsigned long long* scode, const unsigned long long* skey,
                      const ClassView& cv, int32_t rho_skip, const void* pts, int dtype,
                      const CutGeom* cuts, const HashInfo* hi, const unsigned long long* hkeys,
@@ -1300,11 +1300,12 @@ void launch_dep_near(int dp, int g, bool fp64, int layout, const float* spts,
       kern<<<grid, kNearThreads, 0, st>>>(spts, skey, cv, cuts, rho_skip, lambda, delta, q, ctr, hi, nbox, roots,
                                           skip_fill);
     };
-    if (g == 1) go(k_near_to_far<2, 1>);
-    else if (g == 2) go(k_near_to_far<2, 2>);
-    else if (g == 3) go(k_near_to_far<4, 3>);
-    else if (dp == 4) go(k_near_to_far<4, 4>);
-    else go(k_near_to_far<8, 8>);
+    if (g == 1) go(k_near_to_far<2, 1, 2>);
+    else if (g == 2) go(k_near_to_far<2, 2, 2>);
+    else if (g == 3) go(k_near_to_far<4, 3, 4>);
+    else if (dp == 4) go(k_near_to_far<4, 4, 4>);
+    else if (rec_dims(dp, dmax) == 6) go(k_near_to_far<8, 6, 6>);
+    else go(k_near_to_far<8, 8, 8>);
   } else if (g == 1) near_dg<2, 1>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, skip_fill, st);
   else if (g == 2) near_dg<2, 2>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, skip_fill, st);
   else if (g == 3) near_dg<4, 3>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, skip_fill, st);
@@ -1313,14 +1314,15 @@ void launch_dep_near(int dp, int g, bool fp64, int layout, const float* spts,
   count_launches(1);
 }
 
-void launch_dep_far(int dp, bool fp64, const float* spts, const unsigned long long* scode,
+void launch_dep_far(int dp, int dmax, bool fp64, const float* spts, const unsigned long long* scode,
                     const unsigned long long* skey, const ClassView& cv, const CutGeom* cuts,
                     const Node* nodes, const float* nbox, const uint32_t* root, FarQueue q,
                     const FarHint& hint, int32_t* lambda, double* delta, Counters* ctr, cudaStream_t st) {
   if (cv.N == 0) return;
-  if (dp == 2) far_dp<2>(fp64, spts, scode, skey, cv, cuts, nodes, nbox, root, q, hint, lambda, delta, ctr, st);
-  else if (dp == 4) far_dp<4>(fp64, spts, scode, skey, cv, cuts, nodes, nbox, root, q, hint, lambda, delta, ctr, st);
-  else far_dp<8>(fp64, spts, scode, skey, cv, cuts, nodes, nbox, root, q, hint, lambda, delta, ctr, st);
+  if (dp == 2) far_dp<2, 2>(fp64, spts, scode, skey, cv, cuts, nodes, nbox, root, q, hint, lambda, delta, ctr, st);
+  else if (dp == 4) far_dp<4, 4>(fp64, spts, scode, skey, cv, cuts, nodes, nbox, root, q, hint, lambda, delta, ctr, st);
+  else if (rec_dims(dp, dmax) == 6) far_dp<8, 6>(fp64, spts, scode, skey, cv, cuts, nodes, nbox, root, q, hint, lambda, delta, ctr, st);
+  else far_dp<8, 8>(fp64, spts, scode, skey, cv, cuts, nodes, nbox, root, q, hint, lambda, delta, ctr, st);
   count_launches(2);
 }
 

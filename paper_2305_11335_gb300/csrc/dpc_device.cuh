@@ -215,28 +215,30 @@ struct __align__(8) Node {
 };
 
 // Child records of the radix tree (tree.cu): internal node i keeps in one
-// 16-byte-aligned record of rec_words<DP>() words what a search needs about
+// 16-byte-aligned record of rec_words<RD>() words what a search needs about
 // both its children -- their indices, their largest order keys and their
 // bounding boxes (a leaf's box is its point) -- so that expanding a node is
 // one load instead of a chain of dependent ones.
 //   words 0, 1                 left, right child (kLeafBit: a sorted point)
 //   words 4..5, 6..7           largest order key below the left, right child
-//   words 8 .. 8+2DP           box of the left child [lo(DP) | hi(DP)]
-//   words 8+2DP .. 8+4DP       box of the right child
-template <int DP>
-constexpr int rec_words() { return 8 + 4 * DP; }
+//   words 8 .. 8+2RD           box of the left child [lo(RD) | hi(RD)]
+//   words 8+2RD .. 8+4RD       box of the right child
+// RD is the class's padded dimension, but 6 where no point has more than six
+// coordinates: the record is then one line of 128 bytes in place of 160.
+template <int RD>
+constexpr int rec_words() { return 8 + 4 * RD; }
 constexpr int kRecWordsMax = 8 + 4 * 8;
 
-template <int DP>
+template <int RD>
 struct ChildRec {
   uint32_t child[2];
   unsigned long long key[2];
-  float lo[2][DP], hi[2][DP];
+  float lo[2][RD], hi[2][RD];
 };
 
-template <int DP>
-__device__ __forceinline__ ChildRec<DP> load_rec(const float* __restrict__ nrec, uint32_t node) {
-  constexpr int W = rec_words<DP>();
+template <int RD>
+__device__ __forceinline__ ChildRec<RD> load_rec(const float* __restrict__ nrec, uint32_t node) {
+  constexpr int W = rec_words<RD>();
   const float4* r = reinterpret_cast<const float4*>(nrec) + (size_t)node * (W / 4);
   float v[W];
 #pragma unroll
@@ -244,16 +246,16 @@ __device__ __forceinline__ ChildRec<DP> load_rec(const float* __restrict__ nrec,
     const float4 q = __ldg(r + k);
     v[4 * k] = q.x; v[4 * k + 1] = q.y; v[4 * k + 2] = q.z; v[4 * k + 3] = q.w;
   }
-  ChildRec<DP> c;
+  ChildRec<RD> c;
   c.child[0] = __float_as_uint(v[0]);
   c.child[1] = __float_as_uint(v[1]);
 #pragma unroll
   for (int s = 0; s < 2; ++s) {
     c.key[s] = ((unsigned long long)__float_as_uint(v[5 + 2 * s]) << 32) | __float_as_uint(v[4 + 2 * s]);
 #pragma unroll
-    for (int a = 0; a < DP; ++a) {
-      c.lo[s][a] = v[8 + 2 * DP * s + a];
-      c.hi[s][a] = v[8 + 2 * DP * s + DP + a];
+    for (int a = 0; a < RD; ++a) {
+      c.lo[s][a] = v[8 + 2 * RD * s + a];
+      c.hi[s][a] = v[8 + 2 * RD * s + RD + a];
     }
   }
   return c;

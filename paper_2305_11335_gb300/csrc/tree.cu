@@ -30,8 +30,7 @@ __device__ __forceinline__ int prefix_len(const unsigned long long* __restrict__
 }
 
 __global__ void k_tree_build(const unsigned long long* __restrict__ code, ClassView cv,
-                             Node* __restrict__ nodes, uint32_t* __restrict__ leaf_parent,
-                             uint32_t* __restrict__ root) {
+                             Node* __restrict__ nodes, uint32_t* __restrict__ root) {
   const uint32_t n = cv.N;
   const int S = cv.cls->S, ib = cv.cls->ib;
   for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t + 1 < n; t += gridDim.x * blockDim.x) {
@@ -60,17 +59,13 @@ __global__ void k_tree_build(const unsigned long long* __restrict__ code, ClassV
     const uint32_t right = (hi == gamma + 1) ? ((uint32_t)(gamma + 1) | kLeafBit) : (uint32_t)(gamma + 1);
     nodes[i].left = left;
     nodes[i].right = right;
-    if (left & kLeafBit) {
-      leaf_parent[left & ~kLeafBit] = (uint32_t)i;
-    } else {
+    if (!(left & kLeafBit)) {
       nodes[left].parent = (uint32_t)i;
       nodes[left].pend = (uint32_t)j;
       nodes[left].sib = right;
       nodes[left].side = 0u;
     }
-    if (right & kLeafBit) {
-      leaf_parent[right & ~kLeafBit] = (uint32_t)i;
-    } else {
+    if (!(right & kLeafBit)) {
       nodes[right].parent = (uint32_t)i;
       nodes[right].pend = (uint32_t)j;
       nodes[right].sib = left;
@@ -91,20 +86,20 @@ __global__ void k_tree_build(const unsigned long long* __restrict__ code, ClassV
 // a leaf's key is its point's and its box the point itself).
 
 // Writes the summary of child `side` of node `node` into its record.
-template <int DP, bool BOX>
+template <int RD, bool BOX>
 __device__ __forceinline__ void put_child(float* nrec, uint32_t node, int side, unsigned long long key,
                                           const float* lo, const float* hi) {
-  constexpr int W = rec_words<DP>();
+  constexpr int W = rec_words<RD>();
   float* r = nrec + (size_t)node * W;
   __stcg(reinterpret_cast<unsigned long long*>(r + 4 + 2 * side), key);
   if constexpr (BOX) {
-    float4* b = reinterpret_cast<float4*>(r + 8 + 2 * DP * side);
+    float4* b = reinterpret_cast<float4*>(r + 8 + 2 * RD * side);
 #pragma unroll
-    for (int k = 0; k < DP / 2; ++k) {
-      const float v0 = (4 * k < DP) ? lo[4 * k] : hi[4 * k - DP];
-      const float v1 = (4 * k + 1 < DP) ? lo[4 * k + 1] : hi[4 * k + 1 - DP];
-      const float v2 = (4 * k + 2 < DP) ? lo[4 * k + 2] : hi[4 * k + 2 - DP];
-      const float v3 = (4 * k + 3 < DP) ? lo[4 * k + 3] : hi[4 * k + 3 - DP];
+    for (int k = 0; k < RD / 2; ++k) {
+      const float v0 = (4 * k < RD) ? lo[4 * k] : hi[4 * k - RD];
+      const float v1 = (4 * k + 1 < RD) ? lo[4 * k + 1] : hi[4 * k + 1 - RD];
+      const float v2 = (4 * k + 2 < RD) ? lo[4 * k + 2] : hi[4 * k + 2 - RD];
+      const float v3 = (4 * k + 3 < RD) ? lo[4 * k + 3] : hi[4 * k + 3 - RD];
       __stcg(b + k, make_float4(v0, v1, v2, v3));
     }
   }
@@ -112,30 +107,30 @@ __device__ __forceinline__ void put_child(float* nrec, uint32_t node, int side, 
 
 // Reads the summary of child `side` of node `node` back from its record
 // (written by another thread's walk before its release).
-template <int DP, bool BOX>
+template <int RD, bool BOX>
 __device__ __forceinline__ void get_child(const float* nrec, uint32_t node, int side,
                                           unsigned long long& key, float* lo, float* hi) {
-  constexpr int W = rec_words<DP>();
+  constexpr int W = rec_words<RD>();
   const float* r = nrec + (size_t)node * W;
   key = __ldcg(reinterpret_cast<const unsigned long long*>(r + 4 + 2 * side));
   if constexpr (BOX) {
-    const float4* b = reinterpret_cast<const float4*>(r + 8 + 2 * DP * side);
-    float v[2 * DP];
+    const float4* b = reinterpret_cast<const float4*>(r + 8 + 2 * RD * side);
+    float v[2 * RD];
 #pragma unroll
-    for (int k = 0; k < DP / 2; ++k) {
+    for (int k = 0; k < RD / 2; ++k) {
       const float4 q = __ldcg(b + k);
       v[4 * k] = q.x; v[4 * k + 1] = q.y; v[4 * k + 2] = q.z; v[4 * k + 3] = q.w;
     }
 #pragma unroll
-    for (int a = 0; a < DP; ++a) {
+    for (int a = 0; a < RD; ++a) {
       lo[a] = v[a];
-      hi[a] = v[DP + a];
+      hi[a] = v[RD + a];
     }
   }
 }
 
 // A leaf's summary: its point's key, and (BOX) the point as its box.
-template <int DP, bool BOX>
+template <int DP, int RD, bool BOX>
 __device__ __forceinline__ void leaf_summary(uint32_t c, const unsigned long long* __restrict__ skey,
                                              const float* __restrict__ spts, unsigned long long& key,
                                              float* lo, float* hi) {
@@ -144,7 +139,7 @@ __device__ __forceinline__ void leaf_summary(uint32_t c, const unsigned long lon
   if constexpr (BOX) {
     const Pt<DP> p = load_pt<DP>(spts, t);
 #pragma unroll
-    for (int a = 0; a < DP; ++a) lo[a] = hi[a] = p.x[a];
+    for (int a = 0; a < RD; ++a) lo[a] = hi[a] = p.x[a];
   }
 }
 
@@ -186,13 +181,13 @@ __device__ __forceinline__ uint32_t arrive_cta(uint32_t* counter) {
 // and only nodes whose range crosses a block boundary (a few percent) take
 // the global acq_rel counter.  Every node's record gets its children's
 // indices, keys and (BOX) boxes on the way.
-template <int DP, bool BOX>
+template <int DP, int RD, bool BOX>
 __global__ void __launch_bounds__(kUpThreads) k_tree_up(const unsigned long long* __restrict__ skey,
                                                         const float* __restrict__ spts, uint32_t n,
                                                         const Node* __restrict__ nodes,
                                                         uint32_t* visit, float* nrec) {
-  constexpr int W = rec_words<DP>();
-  constexpr int SB = BOX ? 2 * DP : 1;
+  constexpr int W = rec_words<RD>();
+  constexpr int SB = BOX ? 2 * RD : 1;
   __shared__ uint32_t s_cnt[kUpThreads];
   __shared__ unsigned long long s_key[2 * kUpThreads];  // [node - base][side]
   __shared__ float s_box[2 * kUpThreads * SB];          // [node - base][side][lo | hi]
@@ -207,19 +202,19 @@ __global__ void __launch_bounds__(kUpThreads) k_tree_up(const unsigned long long
   if (!((l0 & kLeafBit) && (r0 & kLeafBit))) return;
   // this node from its two leaves
   unsigned long long key;
-  float lo[DP], hi[DP];
+  float lo[RD], hi[RD];
   {
     unsigned long long kr;
-    float lo2[DP], hi2[DP];
-    leaf_summary<DP, BOX>(l0, skey, spts, key, lo, hi);
-    leaf_summary<DP, BOX>(r0, skey, spts, kr, lo2, hi2);
+    float lo2[RD], hi2[RD];
+    leaf_summary<DP, RD, BOX>(l0, skey, spts, key, lo, hi);
+    leaf_summary<DP, RD, BOX>(r0, skey, spts, kr, lo2, hi2);
     __stcg(reinterpret_cast<uint2*>(nrec + (size_t)node * W), make_uint2(l0, r0));
-    put_child<DP, BOX>(nrec, node, 0, key, lo, hi);
-    put_child<DP, BOX>(nrec, node, 1, kr, lo2, hi2);
+    put_child<RD, BOX>(nrec, node, 0, key, lo, hi);
+    put_child<RD, BOX>(nrec, node, 1, kr, lo2, hi2);
     key = key > kr ? key : kr;
     if constexpr (BOX) {
 #pragma unroll
-      for (int a = 0; a < DP; ++a) {
+      for (int a = 0; a < RD; ++a) {
         lo[a] = fminf(lo[a], lo2[a]);
         hi[a] = fmaxf(hi[a], hi2[a]);
       }
@@ -236,11 +231,11 @@ __global__ void __launch_bounds__(kUpThreads) k_tree_up(const unsigned long long
     const uint32_t sib = ps.x;
     const uint32_t pl = side == 0 ? node : sib, pr = side == 0 ? sib : node;
     unsigned long long ks;
-    float lo2[DP], hi2[DP];
+    float lo2[RD], hi2[RD];
     if (sib & kLeafBit) {
-      put_child<DP, BOX>(nrec, par, side, key, lo, hi);
-      leaf_summary<DP, BOX>(sib, skey, spts, ks, lo2, hi2);
-      put_child<DP, BOX>(nrec, par, 1 - side, ks, lo2, hi2);
+      put_child<RD, BOX>(nrec, par, side, key, lo, hi);
+      leaf_summary<DP, RD, BOX>(sib, skey, spts, ks, lo2, hi2);
+      put_child<RD, BOX>(nrec, par, 1 - side, ks, lo2, hi2);
     } else {
       const uint32_t plo = par < pp.y ? par : pp.y, phi = par < pp.y ? pp.y : par;
       if (plo >= base && phi < base + kUpThreads) {
@@ -251,27 +246,27 @@ __global__ void __launch_bounds__(kUpThreads) k_tree_up(const unsigned long long
         s_key[2 * k + side] = key;
         if constexpr (BOX) {
 #pragma unroll
-          for (int a = 0; a < DP; ++a) {
+          for (int a = 0; a < RD; ++a) {
             s_box[(2 * k + side) * SB + a] = lo[a];
-            s_box[(2 * k + side) * SB + DP + a] = hi[a];
+            s_box[(2 * k + side) * SB + RD + a] = hi[a];
           }
         }
         const uint32_t old = arrive_cta(&s_cnt[k]);
-        put_child<DP, BOX>(nrec, par, side, key, lo, hi);
+        put_child<RD, BOX>(nrec, par, side, key, lo, hi);
         if (old == 0u) break;  // the sibling's walk continues
         ks = s_key[2 * k + 1 - side];
         if constexpr (BOX) {
 #pragma unroll
-          for (int a = 0; a < DP; ++a) {
+          for (int a = 0; a < RD; ++a) {
             lo2[a] = s_box[(2 * k + 1 - side) * SB + a];
-            hi2[a] = s_box[(2 * k + 1 - side) * SB + DP + a];
+            hi2[a] = s_box[(2 * k + 1 - side) * SB + RD + a];
           }
         }
       } else {
         // this node's summary into the parent's record, before the release
-        put_child<DP, BOX>(nrec, par, side, key, lo, hi);
+        put_child<RD, BOX>(nrec, par, side, key, lo, hi);
         if (arrive(&visit[par]) == 0u) break;  // the sibling's walk continues
-        get_child<DP, BOX>(nrec, par, 1 - side, ks, lo2, hi2);
+        get_child<RD, BOX>(nrec, par, 1 - side, ks, lo2, hi2);
       }
     }
     // the parent from this node (registers) and its sibling
@@ -279,7 +274,7 @@ __global__ void __launch_bounds__(kUpThreads) k_tree_up(const unsigned long long
     key = key > ks ? key : ks;
     if constexpr (BOX) {
 #pragma unroll
-      for (int a = 0; a < DP; ++a) {
+      for (int a = 0; a < RD; ++a) {
         lo[a] = fminf(lo[a], lo2[a]);
         hi[a] = fmaxf(hi[a], hi2[a]);
       }
@@ -304,33 +299,31 @@ inline unsigned grid_all(uint64_t n) {
 
 }  // namespace
 
-void launch_tree_build(const unsigned long long* scode, const ClassView& cv, Node* nodes,
-                       uint32_t* leaf_parent, uint32_t* root, cudaStream_t st) {
+void launch_tree_build(const unsigned long long* scode, const ClassView& cv, Node* nodes, uint32_t* root,
+                       cudaStream_t st) {
   cudaMemsetAsync(root, 0xff, sizeof(uint32_t) * cv.ninst, st);
   if (cv.N < 2) return;
-  k_tree_build<<<grid_for(cv.N - 1), kThreads, 0, st>>>(scode, cv, nodes, leaf_parent, root);
+  k_tree_build<<<grid_for(cv.N - 1), kThreads, 0, st>>>(scode, cv, nodes, root);
   count_launches(1);
 }
 
-template <int DP>
+template <int DP, int RD>
 void tree_up_dp(const unsigned long long* skey, const float* spts, uint32_t n, Node* nodes,
-                const uint32_t* leaf_parent, uint32_t* visit, float* nbox, bool boxes,
-                cudaStream_t st) {
-  (void)leaf_parent;
+                uint32_t* visit, float* nbox, bool boxes, cudaStream_t st) {
   if (boxes)
-    k_tree_up<DP, true><<<grid_all(n - 1), kUpThreads, 0, st>>>(skey, spts, n, nodes, visit, nbox);
+    k_tree_up<DP, RD, true><<<grid_all(n - 1), kUpThreads, 0, st>>>(skey, spts, n, nodes, visit, nbox);
   else
-    k_tree_up<DP, false><<<grid_all(n - 1), kUpThreads, 0, st>>>(skey, spts, n, nodes, visit, nbox);
+    k_tree_up<DP, RD, false><<<grid_all(n - 1), kUpThreads, 0, st>>>(skey, spts, n, nodes, visit, nbox);
 }
 
-void launch_tree_maxkey(const unsigned long long* skey, const float* spts, int dp, uint32_t n,
-                        Node* nodes, const uint32_t* leaf_parent, uint32_t* visit, float* nrec,
-                        bool boxes, cudaStream_t st) {
+void launch_tree_maxkey(const unsigned long long* skey, const float* spts, int dp, int dmax, uint32_t n,
+                        Node* nodes, uint32_t* visit, float* nrec, bool boxes, cudaStream_t st) {
   if (n < 2) return;
   cudaMemsetAsync(visit, 0, sizeof(uint32_t) * (n - 1), st);
-  if (dp == 2) tree_up_dp<2>(skey, spts, n, nodes, leaf_parent, visit, nrec, boxes, st);
-  else if (dp == 4) tree_up_dp<4>(skey, spts, n, nodes, leaf_parent, visit, nrec, boxes, st);
-  else tree_up_dp<8>(skey, spts, n, nodes, leaf_parent, visit, nrec, boxes, st);
+  if (dp == 2) tree_up_dp<2, 2>(skey, spts, n, nodes, visit, nrec, boxes, st);
+  else if (dp == 4) tree_up_dp<4, 4>(skey, spts, n, nodes, visit, nrec, boxes, st);
+  else if (rec_dims(dp, dmax) == 6) tree_up_dp<8, 6>(skey, spts, n, nodes, visit, nrec, boxes, st);
+  else tree_up_dp<8, 8>(skey, spts, n, nodes, visit, nrec, boxes, st);
   count_launches(1);
 }
 
