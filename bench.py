@@ -427,7 +427,7 @@ def run_ours(args, rank, world, dev):
     dom = max(single, key=lambda p: single[p][0]) if single else None
     kernels = {"density": {2: "k_density_seg", 4: "k_density_tc", 5: "k_density_pairs", 6: "k_density_cell"}.get(
         stats.get("density_layout"), "k_density"),
-               "near": {2: "k_dep_near_seg", 3: "k_near_to_far", 6: "k_dep_near_cell"}.get(stats.get("near_layout"),
+               "near": {2: "k_dep_near_seg", 3: "k_near_to_far", 4: "k_dep_near_tc", 6: "k_dep_near_cell"}.get(stats.get("near_layout"),
                                                                                           "k_dep_near")}
     model_phase = dom if dom in kernels else max(("density", "near"), key=lambda p: phases[p][0])
     work, mean_rho = block_work(job, out["rho"])

@@ -239,13 +239,10 @@ __device__ __forceinline__ void block_union(const uint32_t* c0, int R, int cmax,
 }
 
 // This lane's candidates w0 + lane + 32 v (v < V) of the run table, NaN
-// coordinates past the end (a NaN distance fails every comparison); with
-// KEYS also their order keys (0 past the end: below every query's key).
-template <int DP, int V, bool KEYS = false>
+// coordinates past the end (a NaN distance fails every comparison).
+template <int DP, int V>
 __device__ __forceinline__ void load_window(const RunTable& rt, int nr, uint32_t w0, uint32_t total,
-                                            const float* __restrict__ spts, int lane, Pt<DP>* cand,
-                                            const unsigned long long* __restrict__ skey = nullptr,
-                                            unsigned long long* ck = nullptr) {
+                                            const float* __restrict__ spts, int lane, Pt<DP>* cand) {
   const uint32_t e0 = w0 + lane;
   int lo = 0, hi = nr - 1;
   while (lo < hi) {
@@ -262,39 +259,6 @@ __device__ __forceinline__ void load_window(const RunTable& rt, int nr, uint32_t
       while (r + 1 < nr && rt.pre[r + 1] <= e) ++r;
       const uint32_t src = rt.start[r] + (e - rt.pre[r]);
       cand[v] = load_pt<DP>(spts, src);
-      if constexpr (KEYS) ck[v] = __ldg(skey + src);
-    } else {
-#pragma unroll
-      for (int a = 0; a < DP; ++a) cand[v].x[a] = __int_as_float(0x7fffffff);
-      if constexpr (KEYS) ck[v] = 0ull;
-    }
-  }
-}
-
-// load_window with the sorted position of every candidate (0xffffffff past
-// the end).
-template <int DP, int V>
-__device__ __forceinline__ void load_window_pos(const RunTable& rt, int nr, uint32_t w0, uint32_t total,
-                                                const float* __restrict__ spts, int lane, Pt<DP>* cand,
-                                                uint32_t* pos) {
-  const uint32_t e0 = w0 + lane;
-  int lo = 0, hi = nr - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (rt.pre[mid] <= e0) lo = mid;
-    else hi = mid - 1;
-  }
-  int r = lo;
-#pragma unroll
-  for (int v = 0; v < V; ++v) {
-    const uint32_t e = e0 + 32u * v;
-    pos[v] = 0xffffffffu;
-    if (w0 + 32u * v >= total) break;
-    if (e < total) {
-      while (r + 1 < nr && rt.pre[r + 1] <= e) ++r;
-      const uint32_t src = rt.start[r] + (e - rt.pre[r]);
-      cand[v] = load_pt<DP>(spts, src);
-      pos[v] = src;
     } else {
 #pragma unroll
       for (int a = 0; a < DP; ++a) cand[v].x[a] = __int_as_float(0x7fffffff);
