@@ -1476,7 +1476,7 @@ int dpc_decision_graph(const dpc_batch* b, const int32_t* rho, const double* del
   for (const ClassPlan& c : P.classes) {
     const ClassView cv = view_of(w, c, insts);
     if (k > 0 &&
-        (rc = w->reserve_buf(&w->scr, &w->scr_bytes, decision_scratch_bytes(cv.ninst, k))))
+        (rc = w->reserve_buf(&w->scr, &w->scr_bytes, decision_scratch_bytes(cv.ninst, cv.N, k))))
       return rc;
     launch_chunks(cv, w->chunk_inst, w->chunk_pos, w->stream);
     if (launch_decision(rho, delta, cv, k, top, gamma, rho_bins, delta_bins, delta_lo,

@@ -38,20 +38,28 @@ constexpr int kMaxTopK = 1024;
 constexpr int kDgCap = 4096;   // candidates the sort CTA can hold (48 KB of shared memory)
 constexpr unsigned kFullMask = 0xffffffffu;
 
-// Bins of the first pass and candidates kept per instance, by the number of
-// instances: a single large set gets fine bins (2048: a factor 1.09 of gamma
-// each) and the whole sort buffer; with many instances the scratch per
-// instance stays near 1 KB of bins and twice the k asked for.
+// Bins of the first pass and candidates kept per instance: up to 256 instances
+// get fine bins (2048: a factor 1.09 of gamma each) and the whole sort buffer.
+// With more the scratch is bounded by 24 bytes per point of the class and 1 KB
+// and two or three times the k asked for per instance: 4 bins per octave and 1024
+// candidates where the mean instance has 4096 points, 2 and 512 from 512
+// points, and below that a buffer that takes the mean instance twice.  With one
+// bin per octave and 2 k candidates most of 4,096 instances of 38,000 points
+// overflowed into the radix select (k = 16: 50 ms; 2.6 now).
 struct DgShape {
   int shift;     // bin = bits of the float32 lower bound >> shift
   int nbins;
   uint32_t cap;  // candidates per instance
 };
-inline DgShape dg_shape(uint32_t ninst, int k) {
+inline DgShape dg_shape(uint32_t ninst, uint32_t n, int k) {
   DgShape z;
-  z.shift = ninst <= 256u ? 20 : 23;
+  const uint32_t mean = n / (ninst > 0u ? ninst : 1u) + 1u;
+  z.shift = ninst <= 256u ? 20 : (mean >= 4096u ? 21 : (mean >= 512u ? 22 : 23));
   z.nbins = 1 << (31 - z.shift);
-  z.cap = ninst <= 256u ? (uint32_t)kDgCap : (uint32_t)(2 * k);
+  const uint32_t room = ninst <= 256u ? (uint32_t)kDgCap : (mean >= 4096u ? 1024u : (mean >= 512u ? 512u : 2u * mean));
+  const uint32_t want = (ninst > 256u && mean >= 4096u ? 3u : 2u) * (uint32_t)k;
+  z.cap = room > want ? room : want;
+  if (z.cap > (uint32_t)kDgCap) z.cap = (uint32_t)kDgCap;
   return z;
 }
 
@@ -165,6 +173,7 @@ __device__ __forceinline__ bool dg_bins(int32_t r, double dl, const DgBins& B, i
 
 constexpr int kHistSmemBins = 4096;  // (rho, delta) bins counted in shared memory at most
 constexpr int kScanThreads = 256;
+constexpr int kSelectBlocks = 4;  // CTAs per SM of the radix select, co-resident by its launch bounds
 
 // First pass, every point once: counts of the lower bound's bins (TOP) and of
 // the (rho, delta) bins (HIST).  Shared-memory counts for the CTA's first and
@@ -469,10 +478,14 @@ __device__ void dg_hist(const int32_t* __restrict__ rho, const double* __restric
   for (int e = threadIdx.x; e < 512; e += blockDim.x) (&sh[0][0])[e] = 0u;
   const ChunkRange R = chunk_range(cv);
   __syncthreads();
+  uint32_t cur = 0xffffffffu;
+  DgState S;
+#pragma unroll 2
   for (uint32_t c = R.c0 + (threadIdx.x >> 5); c < R.c1; c += blockDim.x >> 5) {
     uint32_t inst, p0, end;
     cv.chunk(c, inst, p0, end);
-    const DgState S = dg_load(st + inst);
+    if (inst != cur) S = dg_load(st + inst);
+    cur = inst;
     if (!S.exact || S.all || (IDS && !S.tie)) continue;  // warp-uniform
     const InstDev I = cv.instance(inst);
     const uint32_t p = p0 + lane;
@@ -586,7 +599,7 @@ __device__ void dg_pick(DgState* st, uint32_t* hist, uint32_t ninst, int dg) {
 // are needed): a histogram over all points of the class, a grid barrier, a
 // pick per instance, a grid barrier; then the winners -- gamma above T, or at
 // T with an id no larger than the tie limit -- replace the candidates.
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, kSelectBlocks)
 k_dg_select(const int32_t* __restrict__ rho, const double* __restrict__ delta, ClassView cv, DgState* st,
             DgShared* gs, uint32_t* hist, uint32_t cap, unsigned long long* __restrict__ cand_key,
             uint32_t* __restrict__ cand_id, uint32_t limit, int* status) {
@@ -728,9 +741,9 @@ void launch_decision_init(int n_inst, int k, bool pad, int32_t* top, double* gam
 struct DgScratch {
   size_t shared, hist, zeroed, key, id, bytes;
 };
-static DgScratch dg_scratch(uint32_t ninst, int k) {
+static DgScratch dg_scratch(uint32_t ninst, uint32_t n, int k) {
   auto al = [](size_t x) { return (x + 255) / 256 * 256; };
-  const DgShape z = dg_shape(ninst, k);
+  const DgShape z = dg_shape(ninst, n, k);
   DgScratch o;
   o.shared = al(sizeof(DgState) * ninst);
   o.hist = o.shared + al(sizeof(DgShared));
@@ -741,7 +754,7 @@ static DgScratch dg_scratch(uint32_t ninst, int k) {
   return o;
 }
 
-size_t decision_scratch_bytes(uint32_t ninst, int k) { return dg_scratch(ninst, k).bytes; }
+size_t decision_scratch_bytes(uint32_t ninst, uint32_t n, int k) { return dg_scratch(ninst, n, k).bytes; }
 
 template <bool SINGLE>
 static void dg_scan(bool top, bool hist, bool smem, unsigned grid, size_t sh_bytes, const int32_t* rho,
@@ -764,8 +777,8 @@ int launch_decision(const int32_t* rho, const double* delta, const ClassView& cv
   const bool want_top = k > 0 && top && gamma && cv.ninst > 0;
   const bool want_hist = hist && rho_bins > 0 && delta_bins > 0 && cv.ninst > 0;
   const bool single = cv.inst == nullptr;
-  const DgShape z = dg_shape(cv.ninst, k > 0 ? k : 1);
-  const DgScratch o = dg_scratch(cv.ninst, k > 0 ? k : 1);
+  const DgShape z = dg_shape(cv.ninst, cv.N, k > 0 ? k : 1);
+  const DgScratch o = dg_scratch(cv.ninst, cv.N, k > 0 ? k : 1);
   char* b = (char*)scratch;
   DgState* S = (DgState*)b;
   DgShared* G = (DgShared*)(b + o.shared);
@@ -794,9 +807,8 @@ int launch_decision(const int32_t* rho, const double* delta, const ClassView& cv
   else k_dg_gather<false><<<grid, kScanThreads, 0, st>>>(rho, delta, cv, S, G, z.cap, ck, ci);
   count_launches(2);
   if (!(single && cv.N <= z.cap)) {
-    // one block per SM: co-resident for certain, enough for a rare path
     const uint32_t limit = wait_limit(kDgSpinLimit);
-    const unsigned sg = sm_count();
+    const unsigned sg = sm_count() * kSelectBlocks;
     uint32_t cap = z.cap;
     ClassView v = cv;
     void* args[] = {(void*)&rho, (void*)&delta, (void*)&v,  (void*)&S,  (void*)&G,     (void*)&H,

@@ -252,7 +252,7 @@ int launch_decision(const int32_t* rho, const double* delta, const ClassView& cv
                      int32_t* top, double* gamma, int rho_bins, int delta_bins, double delta_lo,
                      unsigned long long* hist, void* scratch, int* status, cudaStream_t st);
 // device scratch launch_decision needs for a class of ninst instances
-size_t decision_scratch_bytes(uint32_t ninst, int k);
+size_t decision_scratch_bytes(uint32_t ninst, uint32_t n, int k);
 // ---- priority range search (range.cu) -------------------------------------------
 struct PrangeArgs {
   uint32_t nq;              // queries

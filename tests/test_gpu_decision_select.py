@@ -1,6 +1,6 @@
 """Top-k selection of the decision graph at the edges of its candidate buffer
-(4096 points per instance up to 256 instances, 2 k beyond): instance sizes
-around the buffer, masses of equal gamma that overflow it (the exact radix
+(4096 points per instance up to 256 instances, by their mean size beyond):
+instance sizes around the buffer, masses of equal gamma that overflow it (the exact radix
 select), gammas outside the float32 range, and more than 256 instances.
 Bit for bit against the oracle (no tolerance)."""
 import math
@@ -43,3 +43,10 @@ def test_gammas_outside_float32(scale):
 def test_many_instances():
     sizes = [0, 1] + [40 + 7 * (i % 50) for i in range(300)]
     check(sizes, [synthetic(n, 900 + i, ties=i % 2 == 0) for i, n in enumerate(sizes)], 24, 6, 9, 0.02)
+
+
+@pytest.mark.parametrize("k", [3, 200, 1000])
+@pytest.mark.parametrize("n", [9, 511, 512, 1500, 4095, 4200])
+def test_many_instances_of_every_mean_size(n, k):
+    sizes = [n + (i * 7) % 5 - 2 for i in range(260)]
+    check(sizes, [synthetic(m, 50 + i, ties=i % 3 == 0) for i, m in enumerate(sizes)], k, 6, 9, 0.02)
