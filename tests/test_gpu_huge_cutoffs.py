@@ -1,0 +1,55 @@
+"""Cutoffs and coordinates at the top of the accepted range, against the
+oracle, for sets above the all-pairs limits whose sizes leave the last tile
+partly empty: a padding candidate must never count, however large the cutoff.
+One cutoff and sweeps of one to four cutoffs per grid level, the tensor tiles
+of 5 to 8 dimensions and the allocation-free density.  Exact."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2305_11335_gb300 as dpc
+from _gpu_util import parity
+
+pytestmark = pytest.mark.gpu
+
+
+def densities(pts, cuts, **kw):
+    t = torch.from_numpy(pts).cuda()
+    batch = dpc.Batch.single(len(pts), pts.shape[1], cuts)
+    return dpc.dpc_density(t, batch, sync=True, **kw).cpu().numpy()
+
+
+def far_blobs(n, d, center, spread, seed):
+    """Blobs around +-center: every distance is a small multiple of `spread`
+    within a blob, about 2 center between blobs."""
+    rng = np.random.default_rng(seed)
+    c = center * rng.choice([-1.0, 1.0], (4, d))
+    return (c[rng.integers(0, 4, n)] + rng.normal(0.0, spread, (n, d))).astype(np.float32)
+
+
+@pytest.mark.parametrize("d", [5, 6, 7, 8])
+@pytest.mark.parametrize("layout", ["auto", "tensor"])
+def test_tensor_tiles_everything_within_the_cutoff(d, layout):
+    n = 17009
+    pts = np.random.default_rng(d).random((n, d), dtype=np.float32)
+    for cuts in ([1e16], [1e20], [1e16, 1.5e16, 1.9e16, 1e15, 0.2]):
+        got = densities(pts, cuts, layout=layout)
+        for c, dc in enumerate(cuts):
+            want = oracle.density(pts, dc) if dc < 10.0 else np.full(n, n)
+            assert np.array_equal(got[c], want), (cuts, c)
+
+
+@pytest.mark.parametrize("d", [5, 8])
+@pytest.mark.parametrize("center,spread", [(1e17, 1e15), (1e18, 2e16)])
+def test_tensor_tiles_far_coordinates(d, center, spread):
+    pts = far_blobs(9013, d, center, spread, d)
+    for cuts in ([2.0 * spread], [2.0 * spread, 2.5 * spread, 3.0 * spread, 2.2 * spread]):
+        parity(pts, cuts, rho_noise=3, rho_min=50, delta_min=4.0 * spread)
+
+
+def test_static_density_in_tensor_tiles():
+    for n, dc in ((20000, 1e16), (20011, 1e16), (20011, 1e20)):
+        pts = np.random.default_rng(n).random((n, 7), dtype=np.float32)
+        got = dpc.dpc_density_static(torch.from_numpy(pts).cuda(), dc, sync=True).cpu().numpy()
+        assert (got == n).all(), (n, dc)
