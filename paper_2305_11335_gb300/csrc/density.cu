@@ -287,9 +287,11 @@ k_density_seg(const float* __restrict__ spts, const unsigned long long* __restri
           for (uint32_t i = 4u * part; i < tn; i += step) {
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
+              // (padding is at distance +inf, which an infinite d_cut^2 would count)
+              const bool real = i + v < tn;
               const double d = dist64<DP, ND>(me, tile_pt<DP>(tile, i + v));
 #pragma unroll
-              for (int c = 0; c < M; ++c) cnt[c] += d <= dc2s[c] ? 1 : 0;
+              for (int c = 0; c < M; ++c) cnt[c] += real && d <= dc2s[c] ? 1 : 0;
             }
           }
         } else {
@@ -322,7 +324,7 @@ k_density_seg(const float* __restrict__ spts, const unsigned long long* __restri
 #pragma unroll 1
                 for (uint32_t i = 4u * part; i < tn; i += step) {
 #pragma unroll 1
-                  for (uint32_t v = i; v < i + 4u; ++v) {
+                  for (uint32_t v = i; v < i + 4u && v < tn; ++v) {
                     const Pt<DP> x = tile_pt<DP>(tile, v);
                     const float s32 = dist32<DP, ND>(me, x);
                     if (s32 > t_in && s32 <= t_out && mine < nq) {

@@ -53,3 +53,37 @@ def test_static_density_in_tensor_tiles():
         pts = np.random.default_rng(n).random((n, 7), dtype=np.float32)
         got = dpc.dpc_density_static(torch.from_numpy(pts).cuda(), dc, sync=True).cpu().numpy()
         assert (got == n).all(), (n, dc)
+
+
+CUTS = [1e18, 1e20, 1e200, 1.7e308]  # squares beyond 2^122, past float32, past binary64
+
+
+@pytest.mark.parametrize("d", [1, 2, 3, 4, 7])
+@pytest.mark.parametrize("dtype", [np.float32, np.int32])
+def test_segments_everything_within_the_cutoff(d, dtype):
+    n = 17003
+    rng = np.random.default_rng(40 + d)
+    pts = rng.random((n, d), dtype=np.float32) if dtype == np.float32 else rng.integers(0, 1000, (n, d), dtype=np.int32)
+    small = 0.05 if dtype == np.float32 else 30.0
+    want = oracle.density(pts, small)
+    for prec in ("fp32", "fp64"):
+        for layout in ("auto", "segment"):
+            for cuts in [[c] for c in CUTS] + [CUTS, [1e200, 1.1e200, small], [1e20, 1.1e20, 1.2e20, 1.3e20, 1.4e20]]:
+                got = densities(pts, cuts, precision=prec, layout=layout)
+                for c, dc in enumerate(cuts):
+                    assert np.array_equal(got[c], want if dc == small else np.full(n, n)), (prec, layout, cuts, c)
+
+
+def test_segments_count_no_band_pairs_beyond_float32():
+    """Every squared distance is finite in float32, so none is undecided by a
+    filter whose outer threshold is infinite."""
+    pts = np.random.default_rng(3).random((17003, 3), dtype=np.float32)
+    for cuts in ([1e20], [1e20, 1.1e20]):
+        densities(pts, cuts)
+        assert dpc.dpc_get_stats()["band_pairs"] == 0, cuts
+
+
+@pytest.mark.parametrize("d", [2, 3])
+def test_run_with_an_infinite_square(d):
+    pts = np.random.default_rng(50 + d).random((17003, d), dtype=np.float32)
+    parity(pts, [1e200, 1e199, 0.03], rho_noise=2, rho_min=5, delta_min=0.1)
