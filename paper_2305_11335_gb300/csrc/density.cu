@@ -463,9 +463,10 @@ k_density_pairs(const float* __restrict__ spts, const unsigned long long* __rest
                 const uint32_t pv = pbase + 32u * v;
                 const float sa0 = dist32<DP, ND>(xa, cand[v]);
                 const float sb0 = dist32<DP, ND>(xb, cand[v]);
-                // a pair that does not count is moved past every threshold
-                const float sa = (!OWN || pv > qa) ? sa0 : INFINITY;
-                const float sb = (two && (!OWN || pv > qb)) ? sb0 : INFINITY;
+                // a pair that does not count is NaN, which no threshold (+inf
+                // among them) reaches
+                const float sa = (!OWN || pv > qa) ? sa0 : NAN;
+                const float sb = (two && (!OWN || pv > qb)) ? sb0 : NAN;
                 const bool ia = sa <= t_in, ib2 = sb <= t_in;
                 ci += (ia ? 1u : 0u) + (ib2 ? 0x10000u : 0u);
                 co += (sa <= t_out ? 1u : 0u) + (sb <= t_out ? 0x10000u : 0u);
@@ -481,8 +482,8 @@ k_density_pairs(const float* __restrict__ spts, const unsigned long long* __rest
                 for (int v = 0; v < V; ++v) {
                   if (v >= vn) break;
                   const uint32_t pv = pbase + 32u * v;
-                  const float sa = (!OWN || pv > qa) ? dist32<DP, ND>(xa, cand[v]) : INFINITY;
-                  const float sb = (two && (!OWN || pv > qb)) ? dist32<DP, ND>(xb, cand[v]) : INFINITY;
+                  const float sa = (!OWN || pv > qa) ? dist32<DP, ND>(xa, cand[v]) : NAN;
+                  const float sb = (two && (!OWN || pv > qb)) ? dist32<DP, ND>(xb, cand[v]) : NAN;
                   if (sa > t_in && sa <= t_out) {
                     ++seen;
                     const bool x = dist64<DP, ND>(xa, cand[v]) <= dc2;

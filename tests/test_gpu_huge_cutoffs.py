@@ -87,3 +87,15 @@ def test_segments_count_no_band_pairs_beyond_float32():
 def test_run_with_an_infinite_square(d):
     pts = np.random.default_rng(50 + d).random((17003, d), dtype=np.float32)
     parity(pts, [1e200, 1e199, 0.03], rho_noise=2, rho_min=5, delta_min=0.1)
+
+
+@pytest.mark.parametrize("layout", ["union", "pairs", "cell"])
+@pytest.mark.parametrize("d", [1, 2, 3, 4, 7])
+def test_other_layouts_everything_within_the_cutoff(d, layout):
+    n = 1003 if layout == "cell" else 5003
+    rng = np.random.default_rng(60 + d)
+    for pts in (rng.random((n, d), dtype=np.float32), rng.integers(0, 1000, (n, d), dtype=np.int32)):
+        for prec in ("fp32", "fp64"):
+            for cut in CUTS:
+                got = densities(pts, [cut], precision=prec, layout=layout)
+                assert (got[0] == n).all(), (prec, cut)
