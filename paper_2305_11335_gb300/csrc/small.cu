@@ -103,16 +103,16 @@ __device__ __forceinline__ const CutHost& small_cut(const CutHost* __restrict__ 
   return hc ? hc[(size_t)i * ncut + k] : args.h[k];
 }
 
-// Densities of every cutoff (grid y).
+// Densities of cutoffs cut0 .. (grid y).
 template <int D, bool F64>
 __global__ void __launch_bounds__(kThreads)
 k_small_density(const void* __restrict__ pts, int dtype, ClassView cv, const CutHost* __restrict__ hc,
-                const __grid_constant__ CutArgs args, int ncut, int32_t* __restrict__ rho, uint64_t rho_stride,
+                const __grid_constant__ CutArgs args, int ncut, int cut0, int32_t* __restrict__ rho, uint64_t rho_stride,
                 uint32_t ngroup, Counters* ctr, int* status) {
   constexpr int Q = small_q<D>();
   __shared__ uint32_t s_cnt[kWarps][Q];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int cut = blockIdx.y;
+  const int cut = cut0 + (int)blockIdx.y;
   for (uint32_t g = blockIdx.x; g < ngroup; g += gridDim.x) {
     uint32_t inst, q0;
     int nq;
@@ -472,13 +472,17 @@ template <int D>
 void density_d(bool fp64, const void* pts, int dtype, const ClassView& cv, const CutHost* hc, const CutArgs& a,
                int ncut, int32_t* rho, uint64_t stride, Counters* ctr, int* status, cudaStream_t st) {
   const uint64_t ng = (uint64_t)cv.nchunk * (32 / small_q<D>());
-  const dim3 grid((unsigned)(ng < (1u << 20) ? ng : (1u << 20)), (unsigned)ncut);
-  if (fp64)
-    k_small_density<D, true><<<grid, kThreads, 0, st>>>(pts, dtype, cv, hc, a, ncut, rho, stride, (uint32_t)ng, ctr,
-                                                       status);
-  else
-    k_small_density<D, false><<<grid, kThreads, 0, st>>>(pts, dtype, cv, hc, a, ncut, rho, stride, (uint32_t)ng, ctr,
-                                                        status);
+  // a launch takes at most 65,535 cutoffs in its grid's second dimension
+  for (int c0 = 0; c0 < ncut; c0 += 65535) {
+    const dim3 grid((unsigned)(ng < (1u << 20) ? ng : (1u << 20)), (unsigned)(ncut - c0 < 65535 ? ncut - c0 : 65535));
+    if (fp64)
+      k_small_density<D, true><<<grid, kThreads, 0, st>>>(pts, dtype, cv, hc, a, ncut, c0, rho, stride, (uint32_t)ng,
+                                                         ctr, status);
+    else
+      k_small_density<D, false><<<grid, kThreads, 0, st>>>(pts, dtype, cv, hc, a, ncut, c0, rho, stride, (uint32_t)ng,
+                                                          ctr, status);
+    count_launches(1);
+  }
 }
 
 template <int D>
@@ -519,7 +523,6 @@ void launch_small_density(int d, bool fp64, const void* pts, int dtype, const Cl
     case 7: density_d<7>(fp64, pts, dtype, cv, hc_dev, a, ncut, rho, rho_stride, ctr, status, st); break;
     default: density_d<8>(fp64, pts, dtype, cv, hc_dev, a, ncut, rho, rho_stride, ctr, status, st); break;
   }
-  count_launches(1);
 }
 
 void launch_small_dependent(int d, bool fp64, const void* pts, int dtype, const ClassView& cv,
