@@ -48,7 +48,10 @@ constexpr int kTcN = 256;            // candidates per MMA (columns)
 constexpr float kTcErr = 0x1p-14f;
 // one candidate row per thread: warp w stages columns 32w .. 32w + 31
 static_assert(kTcN == kTcThreads, "candidate rows per thread");
-constexpr float kTcFar = 1e30f;      // |c|^2 of a padding candidate (dropped by its column, whatever the cutoff)
+// |c|^2 of a padding candidate, which must never count: above every threshold
+// (make_cut_host keeps t_in at or below 3.0e38), and finite as a sum of two TF32
+// numbers.  (A mask of the last columns instead costs the density 0.7-1%.)
+constexpr float kTcFar = 3.2e38f;
 constexpr uint32_t kTcWaitLimit = 1u << 26;  // mbarrier polls before giving up
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
@@ -545,9 +548,6 @@ k_density_tc(const float* __restrict__ spts, const unsigned long long* __restric
             sg = __funnelshift_l(x1, sg, 1);
             lowest = min(lowest, min(x0, x1));
           }
-          // column i is bit 31 - i; those past the last candidate never count:
-          // against a cutoff above sqrt(kTcFar) they are negative too
-          if (ncol - cb < 32) sg >>= 32 - (ncol - cb);
           if (inq) {
             cnt[j] += __popc(sg);
             if (lowest <= wbits) {
