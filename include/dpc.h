@@ -138,8 +138,8 @@ enum {
 #define DPC_FLAG_LAYOUT(v) ((uint32_t)(v) << 16)
 #define DPC_FLAG_LAYOUT_MASK (0x7u << 16)
 /* dpc_run only: capture the call's kernels into a CUDA graph the first time a
- * (pointers, batch, thresholds, precision, radius) combination is seen, and on
- * later calls with the same combination launch that graph instead of one
+ * (pointers, batch, thresholds, precision, fixed radius, layout or near level,
+ * noise skipping) combination is seen, and on later calls with the same combination launch that graph instead of one
  * kernel at a time.  Each call still resets the status word and copies the
  * instance tables (outside the graph), so the point coordinates may change
  * between calls; a different combination, or a workspace that had to grow,

@@ -1616,7 +1616,10 @@ static std::string graph_key(const void* pts, int dtype, const dpc_batch* b,
   auto put = [&](const void* p, size_t n) { k.append((const char*)p, n); };
   const void* ptrs[5] = {pts, rho, lambda, delta, label};
   put(ptrs, sizeof(ptrs));
-  const uint32_t f = flags & (DPC_PREC_MASK | DPC_FLAG_RADIUS_MASK | DPC_FLAG_LAYOUT_MASK);
+  // every flag that changes a kernel or its arguments (the skip threshold of a
+  // single instance is one)
+  const uint32_t f = flags & (DPC_PREC_MASK | DPC_FLAG_RADIUS_MASK | DPC_FLAG_LAYOUT_MASK |
+                              DPC_FLAG_NEAR_SHIFT_MASK | DPC_FLAG_SKIP_NOISE);
   put(&dtype, sizeof(dtype));
   put(&f, sizeof(f));
   put(&b->n_inst, sizeof(b->n_inst));
