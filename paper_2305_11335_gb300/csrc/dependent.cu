@@ -54,6 +54,11 @@ __device__ __forceinline__ bool beyond(float lbs, float bound) {
   return lbs > __fadd_ru(bound, kPruneAbs);
 }
 
+// 1e-5 of a bound covers its relative error, but below 2^-126 a float32 bound is
+// off by up to 2^-150 per axis whatever its size; in binary64 mode, where
+// distances that small are told apart, bounds are lowered by this as well.
+constexpr float kPruneTiny = 0x1p-140f;
+
 // Running minimum of (s, id), the second smallest s, and the sorted position
 // of the minimum (tree phase).
 template <typename S>
@@ -296,7 +301,7 @@ k_dep_near(const float* __restrict__ spts, const unsigned long long* __restrict_
             lb2 = fmaf(l, l, lb2);
           }
           const float lbs = lb2 * f2lo;
-          if constexpr (F64) need = (double)lbs <= acc64.s;
+          if constexpr (F64) need = (double)(lbs - kPruneTiny) <= acc64.s;
           else need = !beyond(lbs, band_of(acc.s1, bmul, badd));
         }
         return __any_sync(kFull, need) != 0;
@@ -519,7 +524,7 @@ k_dep_near_seg(const float* __restrict__ spts, const unsigned long long* __restr
                 lb2 = fmaf(l, l, lb2);
               }
               const float lbs = lb2 * f2lo;
-              if constexpr (F64) need = (double)lbs <= ex.s;
+              if constexpr (F64) need = (double)(lbs - kPruneTiny) <= ex.s;
               else need = !beyond(lbs, bnd);
             }
             return __any_sync(kFull, need) != 0;
@@ -702,8 +707,9 @@ k_near_to_far(const float* __restrict__ spts, const unsigned long long* __restri
 
 // Squared lower bound between the query and the bounding box of a subtree
 // (all coordinates; box layout [lo(RD) | hi(RD)] per node, tree.cu), scaled
-// 1e-5 down so that it stays below the float32 distance of every point inside
-// despite the rounding of this evaluation and of dist32.
+// 1e-5 down (and kPruneTiny less) so that it stays below the float32 and the
+// binary64 distance of every point inside despite the rounding of this
+// evaluation and of dist32.
 template <int DP, int RD>
 __device__ __forceinline__ float rec_lb2(const ChildRec<RD>& r, int s, const Pt<DP>& x) {
   float lb2 = 0.f;
@@ -712,7 +718,7 @@ __device__ __forceinline__ float rec_lb2(const ChildRec<RD>& r, int s, const Pt<
     const float l = fmaxf(fmaxf(r.lo[s][a] - x.x[a], x.x[a] - r.hi[s][a]), 0.f);
     lb2 = fmaf(l, l, lb2);
   }
-  return lb2 * (1.f - 1e-5f);
+  return fmaf(lb2, 1.f - 1e-5f, -kPruneTiny);
 }
 
 // A leaf child's point, from its record (its box is the point itself).
