@@ -830,11 +830,10 @@ void labels_step(Workspace* w, const ClassPlan& c, const ClassView& cv, int k_in
       c.uploaded()
           ? (const LabelParams*)((char*)w->up_dev + c.off_par) + (size_t)k_in_call * c.members.size()
           : nullptr;
-  // instances that fit a CTA's shared memory: one launch, a CTA per instance
-  if (c.nmax <= kSmallLabelPoints)
+  if (labels_by_instance(c.N, (uint32_t)c.members.size(), c.nmax))
     launch_small_labels(rho, lambda, delta, cv, c.nmax, par, one, label, w->status, w->stream);
   else
-    launch_labels(rho, lambda, delta, cv, c.nmax, par, one, label, w->flags, w->stream);
+    launch_labels(rho, lambda, delta, cv, c.nmax, par, one, label, w->flags, w->status, w->stream);
 }
 
 LabelParams one_params(const dpc_params* params, const ClassPlan& c, int ncut_all, int cut) {
@@ -1362,10 +1361,7 @@ int dpc_cluster(const dpc_batch* b, int32_t dcut_index, const dpc_params* params
   if ((rc = prepare(w, P, b, insts, params, flags))) return rc;
   for (const ClassPlan& c : P.classes) {
     const ClassView cv = view_of(w, c, insts);
-    if (c.nmax > kSmallLabelPoints) {
-      launch_class_init(cv, c.g, c.ib, c.bcap, w->status, w->stream);
-      launch_chunks(cv, w->chunk_inst, w->chunk_pos, w->stream);
-    }
+    if (!labels_by_instance(c.N, cv.ninst, c.nmax)) launch_chunks(cv, w->chunk_inst, w->chunk_pos, w->stream);
     labels_step(w, c, cv, 0, one_params(params, c, P.ncut_all, dcut_index), rho, lambda, delta,
                 label);
   }

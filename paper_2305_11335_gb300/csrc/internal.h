@@ -306,8 +306,20 @@ void launch_small_dependent(int d, bool fp64, const void* pts, int dtype, const 
 constexpr uint32_t small_limit(int d, bool fp64, bool density_only) {
   return fp64 ? (d <= 3 ? 2048u : 4096u) : (density_only && d <= 5 ? 16384u : 8192u);
 }
-// labels of a class whose instances have at most kSmallLabelPoints points
+// Points of an instance whose pointers fit a CTA's shared memory (k_small_labels).
 constexpr uint32_t kSmallLabelPoints = 32768;
+// Whether the labels of a class take one launch with a CTA per instance, or the
+// launches of labels.cu over all points.  A CTA costs a few microseconds however
+// small its instance, and one CTA alone falls behind at 24,000 points.  Labels
+// phase of a run, launches -> CTA per instance (us): one instance of 8,000 points
+// 38 -> 18, 16,000 40 -> 31, 24,000 42 -> 43, 32,000 42 -> 63 (4 of them 42 -> 63,
+// 40 of them 126 -> 80); 1,000 instances of 20 points 26 -> 14, 10,000 of them
+// 32 -> 82, 100,000 62 -> 740; 10,000 of 300 points 87 -> 117, 4,000 of 1,000
+// 108 -> 64, 2,000 of 2,000 119 -> 55.
+inline bool labels_by_instance(uint32_t n, uint32_t ninst, uint32_t nmax) {
+  if (nmax > kSmallLabelPoints || (nmax > 20480u && (uint64_t)n < 16ull * nmax)) return false;
+  return ninst <= 4096u || (uint64_t)n >= 1024ull * ninst;
+}
 void launch_small_labels(const int32_t* rho, const int32_t* lambda, const double* delta,
                          const ClassView& cv, uint32_t nmax, const LabelParams* params,
                          LabelParams one, int32_t* label, int* status, cudaStream_t st);
@@ -321,6 +333,6 @@ int label_rounds(uint32_t n);
 // nmax: the largest instance; flags needs label_rounds(nmax) + 1 ints.
 void launch_labels(const int32_t* rho, const int32_t* lambda, const double* delta,
                    const ClassView& cv, uint32_t nmax, const LabelParams* params,
-                   LabelParams one, int32_t* label, int32_t* flags, cudaStream_t st);
+                   LabelParams one, int32_t* label, int32_t* flags, int* status, cudaStream_t st);
 
 }  // namespace dpc

@@ -103,8 +103,8 @@ __global__ void k_label_local(int32_t* par, ClassView cv) {
   });
 }
 
-__global__ void k_label_check(const int32_t* __restrict__ flags, int last, ClassGeom* cls) {
-  if (flags[last]) set_status(cls->status, kStatusCycle);
+__global__ void k_label_check(const int32_t* __restrict__ flags, int last, int* status) {
+  if (flags[last]) set_status(status, kStatusCycle);
 }
 
 inline unsigned grid_for(uint64_t n) {
@@ -133,7 +133,7 @@ int label_rounds(uint32_t n) {
 // `label` doubles as the pointer array; `flags` needs label_rounds(nmax) + 1 ints.
 void launch_labels(const int32_t* rho, const int32_t* lambda, const double* delta,
                    const ClassView& cv, uint32_t nmax, const LabelParams* params,
-                   LabelParams one, int32_t* label, int32_t* flags, cudaStream_t st) {
+                   LabelParams one, int32_t* label, int32_t* flags, int* status, cudaStream_t st) {
   if (cv.N == 0) return;
   const int rounds = label_rounds(nmax);
   cudaMemsetAsync(flags, 0, sizeof(int32_t) * (rounds + 1), st);
@@ -141,7 +141,7 @@ void launch_labels(const int32_t* rho, const int32_t* lambda, const double* delt
   k_label_init<<<grid, kThreads, 0, st>>>(rho, lambda, delta, cv, params, one, label, flags);
   for (int r = 1; r <= rounds; ++r) k_label_jump<<<grid, kThreads, 0, st>>>(label, cv, flags, r);
   k_label_local<<<grid, kThreads, 0, st>>>(label, cv);
-  k_label_check<<<1, 1, 0, st>>>(flags, rounds, cv.cls);
+  k_label_check<<<1, 1, 0, st>>>(flags, rounds, status);
   count_launches(rounds + 3);
 }
 
