@@ -792,7 +792,8 @@ __device__ __noinline__ int tree_walk_from(const Node* __restrict__ nodes,
 // child kept in a register (only the farther one is pushed) and the stack in
 // shared memory, [entry][thread]: lanes of a warp stand at different depths, so
 // entries in local memory cost a sector per lane and access.  Entries past
-// kFastStack (deep trees) go to a local array.
+// kFastStack (deep trees) go to a local array.  Leaves are visited by their record
+// (the point is in it); a caller that reads memory at a leaf's index checks it.
 constexpr int kFastStack = 24;
 struct FastStack {
   uint32_t node[kFastStack][kFarThreads];
@@ -980,7 +981,8 @@ k_dep_far(const float* __restrict__ spts, const unsigned long long* __restrict__
         if (r == kWalkBudget) {
           pass_on = true;
           s_next = fminf(best.s1, s_init);
-        } else if (best.t1 == 0xffffffffu) {
+        } else if (best.t1 >= n) {  // nothing higher (or a malformed tree: far_walk checks no leaf)
+          bad |= best.t1 != 0xffffffffu;
           lambda[fq.id] = -1;
           delta[fq.id] = INFINITY;
         } else {
