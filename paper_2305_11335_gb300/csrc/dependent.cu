@@ -56,7 +56,9 @@ __device__ __forceinline__ bool beyond(float lbs, float bound) {
 
 // 1e-5 of a bound covers its relative error, but below 2^-126 a float32 bound is
 // off by up to 2^-150 per axis whatever its size; in binary64 mode, where
-// distances that small are told apart, bounds are lowered by this as well.
+// distances that small are told apart, bounds are lowered by this as well (the
+// float32 comparisons have kPruneAbs; with it in both modes a run of 1e6 points
+// in 2-D took 0.25% longer).
 constexpr float kPruneTiny = 0x1p-140f;
 
 // Running minimum of (s, id), the second smallest s, and the sorted position
@@ -707,10 +709,10 @@ k_near_to_far(const float* __restrict__ spts, const unsigned long long* __restri
 
 // Squared lower bound between the query and the bounding box of a subtree
 // (all coordinates; box layout [lo(RD) | hi(RD)] per node, tree.cu), scaled
-// 1e-5 down (and kPruneTiny less) so that it stays below the float32 and the
-// binary64 distance of every point inside despite the rounding of this
+// 1e-5 down (F64: and kPruneTiny less) so that it stays below the float32 (F64: the
+// binary64) distance of every point inside despite the rounding of this
 // evaluation and of dist32.
-template <int DP, int RD>
+template <int DP, int RD, bool F64>
 __device__ __forceinline__ float rec_lb2(const ChildRec<RD>& r, int s, const Pt<DP>& x) {
   float lb2 = 0.f;
 #pragma unroll
@@ -718,7 +720,7 @@ __device__ __forceinline__ float rec_lb2(const ChildRec<RD>& r, int s, const Pt<
     const float l = fmaxf(fmaxf(r.lo[s][a] - x.x[a], x.x[a] - r.hi[s][a]), 0.f);
     lb2 = fmaf(l, l, lb2);
   }
-  return fmaf(lb2, 1.f - 1e-5f, -kPruneTiny);
+  return F64 ? fmaf(lb2, 1.f - 1e-5f, -kPruneTiny) : lb2 * (1.f - 1e-5f);
 }
 
 // A leaf child's point, from its record (its box is the point itself).
@@ -738,7 +740,7 @@ enum { kWalkDone = 0, kWalkBudget = 1, kWalkBad = -1 };
 // children's indices, keys and boxes).  Stops with kWalkBudget after `budget` node expansions, and
 // with kWalkBad on a malformed tree or stack overflow (neither happens for a
 // tree built by tree.cu: its depth is at most 64 + 32).
-template <int DP, int RD, typename Prune, typename Visit>
+template <int DP, int RD, bool F64, typename Prune, typename Visit>
 __device__ __noinline__ int tree_walk_from(const Node* __restrict__ nodes,
                                            const float* __restrict__ nbox, uint32_t n,
                                            const unsigned long long* __restrict__ skey,
@@ -770,7 +772,7 @@ __device__ __noinline__ int tree_walk_from(const Node* __restrict__ nodes,
         if ((c & ~kLeafBit) >= n) return kWalkBad;
         visit(c & ~kLeafBit, r.key[s], rec_point<DP, RD>(r, s));
       } else {
-        const float lbs = rec_lb2<DP, RD>(r, s, xq);
+        const float lbs = rec_lb2<DP, RD, F64>(r, s, xq);
         if (prune(lbs)) continue;
         keep[nk] = c;
         keepl[nk] = lbs;
@@ -800,7 +802,7 @@ struct FastStack {
   float lb[kFastStack][kFarThreads];
 };
 
-template <int DP, int RD, typename Prune, typename Visit>
+template <int DP, int RD, bool F64, typename Prune, typename Visit>
 __device__ __forceinline__ int far_walk(FastStack& fs, const float* __restrict__ nbox, uint32_t n,
                                         unsigned long long K, const Pt<DP>& xq, uint32_t start, uint32_t budget,
                                         uint32_t& expanded, Prune prune, Visit visit) {
@@ -818,7 +820,7 @@ __device__ __forceinline__ int far_walk(FastStack& fs, const float* __restrict__
     const bool leaf0 = r.child[0] & kLeafBit, leaf1 = r.child[1] & kLeafBit;
     if (h0 && leaf0) visit(r.child[0] & ~kLeafBit, r.key[0], rec_point<DP, RD>(r, 0));
     if (h1 && leaf1) visit(r.child[1] & ~kLeafBit, r.key[1], rec_point<DP, RD>(r, 1));
-    const float l0 = rec_lb2<DP, RD>(r, 0, xq), l1 = rec_lb2<DP, RD>(r, 1, xq);
+    const float l0 = rec_lb2<DP, RD, F64>(r, 0, xq), l1 = rec_lb2<DP, RD, F64>(r, 1, xq);
     const bool g0 = h0 && !leaf0 && !prune(l0), g1 = h1 && !leaf1 && !prune(l1);
     if (g0 && g1) {
       const bool first = l0 < l1;
@@ -950,7 +952,7 @@ k_dep_far(const float* __restrict__ spts, const unsigned long long* __restrict__
         Best<double> best;
         best.init();
         const double s_init = fmin(q.s1d[e], hint_bound<DP, true>(hint, cv, fq));
-        const int r = far_walk<DP, RD>(
+        const int r = far_walk<DP, RD, F64>(
             fs, nbox, n, fq.K, fq.xq, fq.root, budget, expanded,
             [&](float lbs) { return (double)lbs > fmin(best.s1, s_init); },
             [&](uint32_t t, unsigned long long kt, const Pt<DP>& x) {
@@ -971,7 +973,7 @@ k_dep_far(const float* __restrict__ spts, const unsigned long long* __restrict__
         Best<float> best;
         best.init();
         const float s_init = fminf(q.s1[e], (float)hint_bound<DP, false>(hint, cv, fq));
-        const int r = far_walk<DP, RD>(
+        const int r = far_walk<DP, RD, F64>(
             fs, nbox, n, fq.K, fq.xq, fq.root, budget, expanded,
             [&](float lbs) { return beyond(lbs, band_of(fminf(best.s1, s_init), bmul, badd)); },
             [&](uint32_t t, unsigned long long kt, const Pt<DP>& x) {
@@ -992,7 +994,7 @@ k_dep_far(const float* __restrict__ spts, const unsigned long long* __restrict__
           if (best.s2 <= b) {  // near tie: re-rank the band in binary64
             ++rescans;
             uint32_t more = 0;
-            bad |= tree_walk_from<DP, RD>(
+            bad |= tree_walk_from<DP, RD, F64>(
                        nodes, nbox, n, skey, fq.K, fq.xq, fq.root, 0xffffffffu, more,
                        [&](float lbs) { return beyond(lbs, b); },
                        [&](uint32_t t, unsigned long long kt, const Pt<DP>& x) {
@@ -1105,7 +1107,7 @@ k_dep_far_wide(const float* __restrict__ spts, const unsigned long long* __restr
                   }
                   visit(c & ~kLeafBit, r.key[s], rec_point<DP, RD>(r, s));
                 } else {
-                  const float l = rec_lb2<DP, RD>(r, s, fq.xq);
+                  const float l = rec_lb2<DP, RD, F64>(r, s, fq.xq);
                   if (prune(l)) continue;
                   keep[nk] = c;
                   keepl[nk] = l;
@@ -1133,7 +1135,7 @@ k_dep_far_wide(const float* __restrict__ spts, const unsigned long long* __restr
             stk[pos + s] = keep[s];
             stl[pos + s] = keepl[s];
           } else {  // no room: this lane searches the subtree alone
-            bad |= tree_walk_from<DP, RD>(nodes, nbox, n, skey, fq.K, fq.xq, keep[s], 0xffffffffu,
+            bad |= tree_walk_from<DP, RD, F64>(nodes, nbox, n, skey, fq.K, fq.xq, keep[s], 0xffffffffu,
                                       expanded, prune, visit) != kWalkDone;
           }
         }
