@@ -817,7 +817,7 @@ void dependent_step(Workspace* w, const ClassPlan& c, const ClassView& cv, CutGe
   }
   {
     Phase ph(w, DPC_PHASE_FAR);
-    launch_dep_far(c.dp, c.dmax, fp64, w->spts, w->scode, w->skey, cv, cuts, w->nodes, w->nbox, w->roots,
+    launch_dep_far(c.dp, c.dmax, fp64, w->spts, w->scode, w->skey, cv, cuts, w->nbox, w->roots,
                    queue_of(w), hint, lambda, delta, w->ctr, st);
   }
 }
@@ -1033,7 +1033,7 @@ Choice choose(Workspace* w, const ClassPlan& c, const ClassView& cv, CutGeom* cu
                               near->pts, near->dtype, cuts, w->hinfo, w->hkeys, w->hvals,
                               near->lambda, near->delta, queue_of(w), w->ctr, st,
                               w->nbox, w->roots, default_seg_cells(c.g));
-            launch_dep_far(c.dp, c.dmax, fp64, w->spts, w->scode, w->skey, cv, cuts, w->nodes, w->nbox,
+            launch_dep_far(c.dp, c.dmax, fp64, w->spts, w->scode, w->skey, cv, cuts, w->nbox,
                            w->roots, queue_of(w), FarHint(), near->lambda, near->delta, w->ctr, st);
           }
           if (timed) cudaEventRecord(w->tune_ev[8 + (kNL + 1) * sh + l], st);

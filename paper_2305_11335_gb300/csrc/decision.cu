@@ -544,7 +544,6 @@ __device__ void dg_pick(DgState* st, uint32_t* hist, uint32_t ninst, int dg) {
         const uint32_t t = __shfl_up_sync(kFullMask, incl, o);
         if (lane >= o) incl += t;
       }
-      const uint32_t total = __shfl_sync(kFullMask, incl, 31);
       const uint32_t need = IDS ? S.idneed : S.need;
       // the digit where the running count reaches `need`
       uint32_t before = incl - sum;
@@ -585,7 +584,6 @@ __device__ void dg_pick(DgState* st, uint32_t* hist, uint32_t ninst, int dg) {
           S.idneed = need - bl;
         }
       }
-      (void)total;
     }
     __syncwarp();
     if (lane == 0) st[inst] = S;

@@ -178,8 +178,7 @@ k_dep_near(const float* __restrict__ spts, const unsigned long long* __restrict_
            const void* __restrict__ pts, int dtype, const CutGeom* __restrict__ cuts,
            const HashInfo* __restrict__ hi, const unsigned long long* __restrict__ hkeys,
            const uint2* __restrict__ hvals, int32_t* __restrict__ lambda,
-           double* __restrict__ delta, FarQueue q, Counters* ctr, uint32_t skip_fill) {
-  if (skip_fill && tensor_fill(cv.N, hi, skip_fill)) return;  // the tensor tiles' part
+           double* __restrict__ delta, FarQueue q, Counters* ctr) {
   constexpr int kNearCap = DP == 8 ? 128 : 256;
   __shared__ __align__(16) float s_pts[kNearWarps * kNearCap * DP];
   __shared__ unsigned long long s_key[kNearWarps * kNearCap];
@@ -741,9 +740,7 @@ enum { kWalkDone = 0, kWalkBudget = 1, kWalkBad = -1 };
 // with kWalkBad on a malformed tree or stack overflow (neither happens for a
 // tree built by tree.cu: its depth is at most 64 + 32).
 template <int DP, int RD, bool F64, typename Prune, typename Visit>
-__device__ __noinline__ int tree_walk_from(const Node* __restrict__ nodes,
-                                           const float* __restrict__ nbox, uint32_t n,
-                                           const unsigned long long* __restrict__ skey,
+__device__ __noinline__ int tree_walk_from(const float* __restrict__ nbox, uint32_t n,
                                            unsigned long long K, const Pt<DP>& xq,
                                            uint32_t start, uint32_t budget, uint32_t& expanded,
                                            Prune prune, Visit visit) {
@@ -923,7 +920,7 @@ template <int DP, int RD, bool F64>
 __global__ void __launch_bounds__(kFarThreads)
 k_dep_far(const float* __restrict__ spts, const unsigned long long* __restrict__ scode,
           const unsigned long long* __restrict__ skey, ClassView cv,
-          const CutGeom* __restrict__ cuts, const Node* __restrict__ nodes,
+          const CutGeom* __restrict__ cuts,
           const float* __restrict__ nbox, const uint32_t* __restrict__ roots, FarQueue q, FarHint hint,
           int32_t* __restrict__ lambda, double* __restrict__ delta, Counters* ctr, uint32_t room) {
   __shared__ FastStack fs;
@@ -995,7 +992,7 @@ k_dep_far(const float* __restrict__ spts, const unsigned long long* __restrict__
             ++rescans;
             uint32_t more = 0;
             bad |= tree_walk_from<DP, RD, F64>(
-                       nodes, nbox, n, skey, fq.K, fq.xq, fq.root, 0xffffffffu, more,
+                       nbox, n, fq.K, fq.xq, fq.root, 0xffffffffu, more,
                        [&](float lbs) { return beyond(lbs, b); },
                        [&](uint32_t t, unsigned long long kt, const Pt<DP>& x) {
                          if (dist32<DP>(fq.xq, x) <= b) ex.add(dist64<DP>(fq.xq, x), key_id(kt));
@@ -1046,7 +1043,7 @@ template <int DP, int RD, bool F64>
 __global__ void __launch_bounds__(kFarThreads)
 k_dep_far_wide(const float* __restrict__ spts, const unsigned long long* __restrict__ scode,
                const unsigned long long* __restrict__ skey, ClassView cv,
-               const CutGeom* __restrict__ cuts, const Node* __restrict__ nodes,
+               const CutGeom* __restrict__ cuts,
                const float* __restrict__ nbox, const uint32_t* __restrict__ roots, FarQueue q,
                int32_t* __restrict__ lambda, double* __restrict__ delta, Counters* ctr) {
   constexpr int kWarpsPerBlock = kFarThreads / 32;
@@ -1135,7 +1132,7 @@ k_dep_far_wide(const float* __restrict__ spts, const unsigned long long* __restr
             stk[pos + s] = keep[s];
             stl[pos + s] = keepl[s];
           } else {  // no room: this lane searches the subtree alone
-            bad |= tree_walk_from<DP, RD, F64>(nodes, nbox, n, skey, fq.K, fq.xq, keep[s], 0xffffffffu,
+            bad |= tree_walk_from<DP, RD, F64>(nbox, n, fq.K, fq.xq, keep[s], 0xffffffffu,
                                       expanded, prune, visit) != kWalkDone;
           }
         }
@@ -1239,7 +1236,7 @@ void near_dg(bool fp64, int layout, const float* spts, const unsigned long long*
              const unsigned long long* skey, const ClassView& cv, int32_t rho_skip,
              const void* pts, int dtype, const CutGeom* cuts, const HashInfo* hi,
              const unsigned long long* hkeys, const uint2* hvals, int32_t* lambda, double* delta,
-             FarQueue q, Counters* ctr, int seg_cells, uint32_t skip_fill, cudaStream_t st) {
+             FarQueue q, Counters* ctr, int seg_cells, cudaStream_t st) {
   const unsigned grid = grid_for(cv.nchunk, kNearWarps, sm_count() * 64u);
   if (layout == kLayoutSegment) {
     if (fp64)
@@ -1254,18 +1251,18 @@ void near_dg(bool fp64, int layout, const float* spts, const unsigned long long*
     if (fp64)
       k_dep_near<DP, G, true><<<grid, kNearThreads, 0, st>>>(spts, scode, skey, cv, rho_skip, pts,
                                                              dtype, cuts, hi, hkeys, hvals, lambda,
-                                                             delta, q, ctr, skip_fill);
+                                                             delta, q, ctr);
     else
       k_dep_near<DP, G, false><<<grid, kNearThreads, 0, st>>>(spts, scode, skey, cv, rho_skip, pts,
                                                               dtype, cuts, hi, hkeys, hvals, lambda,
-                                                              delta, q, ctr, skip_fill);
+                                                              delta, q, ctr);
   }
 }
 
 template <int DP, int RD>
 void far_dp(bool fp64, const float* spts, const unsigned long long* scode,
             const unsigned long long* skey, const ClassView& cv, const CutGeom* cuts,
-            const Node* nodes, const float* nbox, const uint32_t* root, FarQueue q, const FarHint& hint,
+            const float* nbox, const uint32_t* root, FarQueue q, const FarHint& hint,
             int32_t* lambda, double* delta, Counters* ctr, cudaStream_t st) {
   // the queue length is known only on the device: CTAs for most lengths, so
   // that a free SM takes the next 128 queries (1e6 2-D queries .27 -> .24 ms,
@@ -1275,14 +1272,14 @@ void far_dp(bool fp64, const float* spts, const unsigned long long* scode,
   const uint32_t room = sm_count() * 1024u;
   const unsigned grid2 = grid_for(cv.N, kFarThreads / 32, sm_count() * 16u);
   if (fp64) {
-    k_dep_far<DP, RD, true><<<grid, kFarThreads, 0, st>>>(spts, scode, skey, cv, cuts, nodes, nbox,
+    k_dep_far<DP, RD, true><<<grid, kFarThreads, 0, st>>>(spts, scode, skey, cv, cuts, nbox,
                                                       root, q, hint, lambda, delta, ctr, room);
-    k_dep_far_wide<DP, RD, true><<<grid2, kFarThreads, 0, st>>>(spts, scode, skey, cv, cuts, nodes,
+    k_dep_far_wide<DP, RD, true><<<grid2, kFarThreads, 0, st>>>(spts, scode, skey, cv, cuts,
                                                             nbox, root, q, lambda, delta, ctr);
   } else {
-    k_dep_far<DP, RD, false><<<grid, kFarThreads, 0, st>>>(spts, scode, skey, cv, cuts, nodes, nbox,
+    k_dep_far<DP, RD, false><<<grid, kFarThreads, 0, st>>>(spts, scode, skey, cv, cuts, nbox,
                                                        root, q, hint, lambda, delta, ctr, room);
-    k_dep_far_wide<DP, RD, false><<<grid2, kFarThreads, 0, st>>>(spts, scode, skey, cv, cuts, nodes,
+    k_dep_far_wide<DP, RD, false><<<grid2, kFarThreads, 0, st>>>(spts, scode, skey, cv, cuts,
                                                              nbox, root, q, lambda, delta, ctr);
   }
 }
@@ -1297,7 +1294,8 @@ void launch_dep_near(int dp, int g, int dmax, bool fp64, int layout, const float
                      cudaStream_t st, const float* nbox, const uint32_t* roots, int seg_cells,
                      uint32_t skip_fill) {
   if (cv.N == 0) return;
-  // (beside the tensor form the queue is cleared and may be filled already)
+  // (skip_fill, tree layout only: beside the tensor form, which has cleared the
+  // queue and may have filled it)
   if (!skip_fill) cudaMemsetAsync(&ctr->queue_n, 0, 2 * sizeof(unsigned int), st);  // queue_n and queue2_n
   if (layout == kLayoutCell) {
     launch_dep_near_cell(dp, g, fp64, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys,
@@ -1316,23 +1314,23 @@ void launch_dep_near(int dp, int g, int dmax, bool fp64, int layout, const float
     else if (dp == 4) go(k_near_to_far<4, 4, 4>);
     else if (rec_dims(dp, dmax) == 6) go(k_near_to_far<8, 6, 6>);
     else go(k_near_to_far<8, 8, 8>);
-  } else if (g == 1) near_dg<2, 1>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, skip_fill, st);
-  else if (g == 2) near_dg<2, 2>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, skip_fill, st);
-  else if (g == 3) near_dg<4, 3>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, skip_fill, st);
-  else if (dp == 4) near_dg<4, 4>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, skip_fill, st);
-  else near_dg<8, 4>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, skip_fill, st);
+  } else if (g == 1) near_dg<2, 1>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, st);
+  else if (g == 2) near_dg<2, 2>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, st);
+  else if (g == 3) near_dg<4, 3>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, st);
+  else if (dp == 4) near_dg<4, 4>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, st);
+  else near_dg<8, 4>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, st);
   count_launches(1);
 }
 
 void launch_dep_far(int dp, int dmax, bool fp64, const float* spts, const unsigned long long* scode,
                     const unsigned long long* skey, const ClassView& cv, const CutGeom* cuts,
-                    const Node* nodes, const float* nbox, const uint32_t* root, FarQueue q,
+                    const float* nbox, const uint32_t* root, FarQueue q,
                     const FarHint& hint, int32_t* lambda, double* delta, Counters* ctr, cudaStream_t st) {
   if (cv.N == 0) return;
-  if (dp == 2) far_dp<2, 2>(fp64, spts, scode, skey, cv, cuts, nodes, nbox, root, q, hint, lambda, delta, ctr, st);
-  else if (dp == 4) far_dp<4, 4>(fp64, spts, scode, skey, cv, cuts, nodes, nbox, root, q, hint, lambda, delta, ctr, st);
-  else if (rec_dims(dp, dmax) == 6) far_dp<8, 6>(fp64, spts, scode, skey, cv, cuts, nodes, nbox, root, q, hint, lambda, delta, ctr, st);
-  else far_dp<8, 8>(fp64, spts, scode, skey, cv, cuts, nodes, nbox, root, q, hint, lambda, delta, ctr, st);
+  if (dp == 2) far_dp<2, 2>(fp64, spts, scode, skey, cv, cuts, nbox, root, q, hint, lambda, delta, ctr, st);
+  else if (dp == 4) far_dp<4, 4>(fp64, spts, scode, skey, cv, cuts, nbox, root, q, hint, lambda, delta, ctr, st);
+  else if (rec_dims(dp, dmax) == 6) far_dp<8, 6>(fp64, spts, scode, skey, cv, cuts, nbox, root, q, hint, lambda, delta, ctr, st);
+  else far_dp<8, 8>(fp64, spts, scode, skey, cv, cuts, nbox, root, q, hint, lambda, delta, ctr, st);
   count_launches(2);
 }
 

@@ -239,9 +239,8 @@ void launch_dep_near_tc(int d, const float* spts, const unsigned long long* scod
                         cudaStream_t st);
 void launch_dep_far(int dp, int dmax, bool fp64, const float* spts, const unsigned long long* scode,
                     const unsigned long long* skey, const ClassView& cv, const CutGeom* cuts,
-                    const Node* nodes, const float* nbox, const uint32_t* root, FarQueue q,
-                    const FarHint& hint, int32_t* lambda, double* delta, Counters* ctr,
-                    cudaStream_t st);
+                    const float* nbox, const uint32_t* root, FarQueue q, const FarHint& hint,
+                    int32_t* lambda, double* delta, Counters* ctr, cudaStream_t st);
 
 // ---- decision graph (decision.cu) -------------------------------------------------
 // top-k by gamma = rho * delta and the (rho, delta) histogram of every instance
