@@ -162,7 +162,8 @@ k_small_density(const void* __restrict__ pts, int dtype, ClassView cv, const Cut
           mband = min(mband, band_min2(s, bb.lo));
         }
       }
-      // a band pair anywhere: count this warp's band pairs in binary64
+      // a band pair anywhere: this warp's candidates again, every band pair in
+      // binary64
       if (__any_sync(kFull, mband < bb.width)) {
         uint32_t seen = 0;
         for (uint32_t e0 = warp * 64; e0 < I.n; e0 += kStep) {
@@ -170,12 +171,36 @@ k_small_density(const void* __restrict__ pts, int dtype, ClassView cv, const Cut
           for (uint32_t e = e0 + lane; e < e0 + 64u && e < I.n; e += 32u) {
             float x[D];
             load_row<D>(pts, dtype, I.coord, e, x);
+            if constexpr (D == 1) {
+              // a 1-D binary64 distance is so short that it would run under a
+              // predicate for every pair, through the binary64 pipe (13,000 integer
+              // points with a cutoff that many pairs meet: 1.32 ms, 0.12 with the
+              // float32 tests first and a loop over the pairs that need it)
+              uint32_t bm = 0;
 #pragma unroll
-            for (int j = 0; j < Q; ++j) {
-              const float s = row_dist32<D>(xq[j], x);
-              if (s > C.t_in && s <= C.t_out && j < nq) {
-                ++seen;
-                cnt[j] += row_dist64<D>(xq[j], x) <= C.dc2 ? 1u : 0u;
+              for (int j = 0; j < Q; ++j) {
+                const float s = row_dist32<D>(xq[j], x);
+                bm |= (s > C.t_in && s <= C.t_out && j < nq) ? 1u << j : 0u;
+              }
+              seen += __popc(bm);
+#pragma unroll 1
+              while (bm) {
+                const int j = __ffs((int)bm) - 1;
+                bm &= bm - 1u;
+                float y[D];
+                load_row<D>(pts, dtype, I.coord, q0 + (uint32_t)j, y);
+                const uint32_t in = row_dist64<D>(y, x) <= C.dc2 ? 1u : 0u;
+#pragma unroll
+                for (int k = 0; k < Q; ++k) cnt[k] += k == j ? in : 0u;
+              }
+            } else {
+#pragma unroll
+              for (int j = 0; j < Q; ++j) {
+                const float s = row_dist32<D>(xq[j], x);
+                if (s > C.t_in && s <= C.t_out && j < nq) {
+                  ++seen;
+                  cnt[j] += row_dist64<D>(xq[j], x) <= C.dc2 ? 1u : 0u;
+                }
               }
             }
           }
