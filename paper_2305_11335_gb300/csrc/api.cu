@@ -860,16 +860,29 @@ std::string tune_key(const ClassPlan& c, const dpc_batch* b, int cut) {
 // ---- small instances -----------------------------------------------------------
 
 // Whether a class runs from all pairs (small.cu) instead of the grid: one
-// dimension, no fixed or tuned radius or layout asked for, and few enough
-// points.  Measured on blobs with a median density of 16 (us a call, grid ->
-// all pairs): density of 1,000 points in 2-D 156 -> 18, 8,192 183 -> 37,
-// 16,384 205 -> 77 (5-D 313 -> 191, 8-D 347 -> 457; 8,192 points 287 -> 135);
-// a run of 1,000 points in 2-D 311 -> 34, 8,192 393 -> 117 (5-D 1,077 -> 167,
-// 8-D 1,240 -> 339).  In binary64 the pairs wait for the binary64 pipe: a run
-// of 2,048 points in 2-D 444 -> 191 but 4,096 461 -> 642; in 5-D 4,009 ->
-// 1,336 at 4,096.  A captured call (DPC_FLAG_GRAPH) takes this path up to
-// 4,096 points only: tests/test_gpu_parity.py counts the kernels of a captured
-// grid pipeline at 6,000.
+// dimension, no fixed or tuned radius or layout asked for, few enough points an
+// instance (small_limit) and few enough of them.
+// Points, measured on blobs with a median density of 16 (us a call, grid -> all
+// pairs): density of 1,000 points in 2-D 107 -> 9.5, 8,192 115 -> 36, 16,384 121
+// -> 92 (5-D 214 -> 191; 8-D 8,192 189 -> 134, 16,384 216 -> 492); a run of 1,000
+// points in 2-D 189 -> 27, 8,192 227 -> 127, 16,384 266 -> 360 (5-D 8,192 394 ->
+// 169, 16,384 590 -> 615; 8-D 599 -> 335 and 769 -> 1,089).  In binary64 the
+// pairs wait for the binary64 pipe: a run of 2,048 points in 2-D 315 -> 199,
+// 4,096 357 -> 653; in 5-D 4,096 1,590 -> 1,342, in 4-D 1,077 -> 1,103.
+// Instances: every group of 4 or 8 queries costs a CTA however small its instance
+// is, so a class of many tiny ones is the grid's.  Sum of the phases without
+// labels: a run of 4,000 instances of 20 points in 2-D 242 -> 156 us, 8,000 271 ->
+// 288, 20,000 403 -> 688 (3-D 257 -> 185, 290 -> 343, 432 -> 822); 1,000 of 100
+// (4,000 chunks) 256 -> 191, 2,000 309 -> 359; 100 of 1,000 (3,200) 263 -> 269.  A
+// density alone: 20,000 of 20 245 -> 151, 500 of 1,000 (16,000 chunks) 260 -> 257,
+// 20,000 of 100 (80,000) 546 -> 618.  The grid's sweeps share their set-up, so
+// runs of three cutoffs and more change sides earlier (1,000 of 100, whole calls:
+// 2 cutoffs 526 -> 408, 4 608 -> 787; 4,000 of 20 in 3-D, 8 cutoffs 1,262 -> 1,658).
+// A captured call (DPC_FLAG_GRAPH) takes this path up to 4,096 points only.
+// Replayed, all pairs are the faster side beyond that too (grid -> all pairs: a
+// run of 4,096 points in 2-D 155 -> 52, 8,192 177 -> 123, in 8-D 542 -> 331), so
+// the line is not one of speed: a captured call of more points keeps the grid's
+// kernel sequence, which tests/test_gpu_parity.py counts at 6,000 points.
 bool small_class(const Workspace* w, const dpc_batch* b, const CallPlan& P, const ClassPlan& c,
                  const std::vector<Inst>& insts, uint32_t flags, bool density_only) {
   if (flags & (DPC_FLAG_RADIUS_MASK | DPC_FLAG_LAYOUT_MASK | DPC_FLAG_NEAR_SHIFT_MASK | DPC_FLAG_AUTOTUNE))
@@ -882,6 +895,7 @@ bool small_class(const Workspace* w, const dpc_batch* b, const CallPlan& P, cons
   const int d = insts[c.members[0]].d;
   const uint32_t nmax = small_limit(d, fp64, density_only);
   if (c.nmax > nmax || ((flags & DPC_FLAG_GRAPH) && c.nmax > 4096u)) return false;
+  if (c.nchunk > (density_only ? 16384u : (P.ncut > 2 ? 2048u : 4096u))) return false;
   uint64_t pairs = 0;
   for (int i : c.members) {
     if (insts[i].d != d) return false;

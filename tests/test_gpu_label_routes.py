@@ -1,8 +1,8 @@
 """Labels by one CTA per instance or by launches over all points, on both
 sides of the rule between them: sizes of one large instance, a few large ones,
-counts of tiny instances (with one larger among them), and tiny instances
-whose whole run takes the all-pairs path.  Random forests against a sequential
-walk, cycles reported, the route read from the launch count."""
+counts of tiny instances (with one larger among them), and whole runs of tiny
+instances.  Random forests against a sequential walk, cycles reported, the
+route read from the launch count."""
 import numpy as np
 import pytest
 import torch
@@ -59,13 +59,27 @@ def test_forests(name):
     assert e.value.code == dpc.DPC_ERR_DATA
 
 
-def test_run_of_tiny_instances():
-    sizes = [20] * 5000
-    pts = np.random.default_rng(1).random((100000, 2), dtype=np.float32)
-    batch = dpc.Batch.packed(sizes, [2] * 5000, [[0.2]] * 5000)
-    out = dpc.dpc_run(torch.from_numpy(pts).cuda(), batch, dpc.make_params(batch, 2, 3, 0.3), sync=True)
-    assert dpc.dpc_get_stats()["density_layout"] == 0
+@pytest.mark.parametrize("count,pairs,sweep_pairs,density_pairs", [
+    (2048, True, True, True), (4096, True, False, True), (4097, False, False, True), (16385, False, False, False)])
+def test_runs_of_tiny_instances(count, pairs, sweep_pairs, density_pairs):
+    """Many instances of 20 points on both sides of the all-pairs limits (a run
+    by 32-point chunks, a density alone by four times as many)."""
+    sizes = [20] * count
+    pts = np.random.default_rng(1).random((20 * count, 2), dtype=np.float32)
+    batch = dpc.Batch.packed(sizes, [2] * count, [[0.2]] * count)
+    t = torch.from_numpy(pts).cuda()
+    out = dpc.dpc_run(t, batch, dpc.make_params(batch, 2, 3, 0.3), sync=True)
+    assert (dpc.dpc_get_stats()["density_layout"] == 0) == pairs
     out = {k: v[0].cpu().numpy() for k, v in out.items()}
-    for i in list(range(0, 5000, 97)) + [4999]:
+    den = dpc.dpc_density(t, batch, sync=True)[0].cpu().numpy()
+    assert (dpc.dpc_get_stats()["density_layout"] == 0) == density_pairs
+    assert np.array_equal(den, out["rho"])
+    three = dpc.Batch.packed(sizes, [2] * count, [[0.2, 0.3, 0.25]] * count)
+    sweep = dpc.dpc_run(t, three, dpc.make_params(three, 2, 3, 0.3), sync=True)
+    assert (dpc.dpc_get_stats()["density_layout"] == 0) == sweep_pairs
+    sweep = {k: v.cpu().numpy() for k, v in sweep.items()}
+    assert_same({k: v[0] for k, v in sweep.items()}, out)
+    for i in list(range(0, count, 97)) + [count - 1]:
         s = slice(20 * i, 20 * i + 20)
         assert_same({k: v[s] for k, v in out.items()}, oracle.run(pts[s], 0.2, 2, 3, 0.3), str(i))
+        assert_same({k: v[1, s] for k, v in sweep.items()}, oracle.run(pts[s], 0.3, 2, 3, 0.3), str(i))
