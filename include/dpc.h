@@ -116,10 +116,10 @@ enum {
 #define DPC_FLAG_RADIUS_MASK (0x7u << 12)
 /* Fixed work layout of the density and near-dependent kernels instead of the
  * default rule (density: tensor tiles in 5-8 dimensions with
- * DPC_PREC_FP32_CERT from 2 points per occupied cell on, pairs in binary64,
- * segments otherwise, union in 1-D; near phase: tensor tiles in 5-8 dimensions
- * from 4 points per cell on, else the tree, union in 1-D above 1e6 points) or
- * the autotuned choice:
+ * DPC_PREC_FP32_CERT from 2 points per occupied cell on, pairs for float32 points
+ * in binary64 from 800 chunks of 32 points on, segments otherwise, union in 1-D;
+ * near phase: tensor tiles in 5-8 dimensions from 4 points per cell on, else the
+ * tree, union in 1-D above 1e6 points) or the autotuned choice:
  * 1 = union (a warp's 32 consecutive points, one query per lane, the union of
  * their blocks streamed as broadcast reads), 2 = segment (the points around a
  * few consecutive cells staged once, the cells' queries spread over the lanes),

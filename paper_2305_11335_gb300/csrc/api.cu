@@ -942,9 +942,8 @@ struct NearTrial {
 };
 
 // Default layouts (measured on the GB300).  Density: tensor tiles in 5-8
-// dimensions with the float32 filter, segments otherwise, pairs in binary64
-// (the binary64 pipe is the bound, so half the pairs: 1e5 points in 2-D 0.45 ms
-// against 1.34, in 3-D 3.7 against 5.7, in 7-D 12.2 against 20.5), union in 1-D.
+// dimensions with the float32 filter, segments otherwise, pairs in binary64 from
+// kBinary64Pairs chunks on, union in 1-D.
 // Near phase: tensor tiles again; else the tree search (near phase + far search,
 // ms, blocks scanned -> tree: 1e6 points in 2-D 0.74 -> 0.34, blobs of 1e6 in 3-D
 // 2.21 -> 0.66, in 4-D 4.6 -> 1.9, binary64 1e5 in 5-D 62.9 -> 2.6; against it
@@ -954,7 +953,8 @@ inline bool tensor_class(const ClassPlan& c, bool fp64) { return c.dp == 8 && !f
 inline int default_dlayout(const ClassPlan& c, int prec) {
   if (tensor_class(c, prec != 0)) return kLayoutTensor;
   if (prec == 2) return kLayoutSegment;  // 64-bit integers
-  return c.g < 2 ? kLayoutUnion : (prec == 1 ? kLayoutPairs : kLayoutSegment);
+  if (c.g < 2) return kLayoutUnion;
+  return prec == 1 && c.nchunk >= kBinary64Pairs ? kLayoutPairs : kLayoutSegment;
 }
 inline int default_nlayout(const ClassPlan& c, bool fp64) {
   if (tensor_class(c, fp64)) return kLayoutTensor;
@@ -1222,7 +1222,7 @@ void group_density_step(Workspace* w, const ClassPlan& c, const ClassView& cv, i
     // cutoff alone (on top of four in one pass, segments / pairs in ms: 1e6 points
     // in 2-D 14.4 / 6.8, in 3-D 79 / 35, 1e5 in 5-D 10.9 / 9.3, in 7-D 17.6 /
     // 15.7; in 1-D .88 / 1.07 with that one's union layout)
-    if (prec == 1 && c.g >= 2 && i + 1 == g.cuts.size()) {
+    if (i + 1 == g.cuts.size() && default_dlayout(c, prec) == kLayoutPairs) {
       launch_adopt_geometry(cv, w->geo, w->cuts + (size_t)g.cuts[i] * cv.ninst, w->stream);
       single(g.cuts[i]);
       return;

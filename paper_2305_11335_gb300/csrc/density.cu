@@ -688,10 +688,8 @@ void launch_density(int dp, int g, int d, int prec, int layout, const float* spt
     }
     layout = kLayoutSegment;
   }
-  // float32 points in binary64: the segments' work with every pair once (the
-  // segment kernel's tiles are made for packed float32).  1e6 points, density in
-  // ms, segments / pairs: 2-D 13.4 / 6.1, 3-D 70 / 34; 5-D, 1e5 points 25.8 / 18.6
-  if (layout == kLayoutSegment && prec == 1) layout = kLayoutPairs;
+  // float32 points in binary64: the segments' work with every pair once
+  if (layout == kLayoutSegment && prec == 1 && cv.nchunk >= kBinary64Pairs) layout = kLayoutPairs;
   if (layout == kLayoutCell) {
     launch_density_cell(dp, g, prec != 0, spts, scode, sid, cv, cuts, hi, hkeys, hvals, rho_out, skey, ctr,
                         st);

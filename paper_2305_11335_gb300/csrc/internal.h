@@ -148,6 +148,15 @@ enum { kLayoutUnion = 1, kLayoutSegment = 2, kLayoutTree = 3, kLayoutTensor = 4,
        kLayoutCell = 6 };
 
 // ---- density (density.cu) -------------------------------------------------------
+// Chunks from which float32 points in binary64 are counted pair by pair (every
+// pair once) and not in segments (every query's block, but a chunk's queries
+// spread over several warps).  The binary64 pipe is the bound where the chip is
+// full; below that the longest chunk is.  Density in ms, segments / pairs, uniform
+// points: 2-D 1e4 .041 / .070, 2e4 .063 / .080, 4e4 .132 / .121, 3e5 1.35 / .54;
+// 3-D 1e4 .078 / .134, 2e4 .133 / .150, 4e4 .29 / .22, 3e5 3.0 / 1.1; 5-D 1e4 .56 /
+// 1.07, 2e4 1.29 / 1.33, 4e4 3.4 / 2.4; 7-D 2e4 3.8 / 5.4, 4e4 10.4 / 11.8, 1e5
+// 45 / 28.
+constexpr uint32_t kBinary64Pairs = 800;
 // Cutoffs evaluated in one density launch: they share the block geometry of
 // the largest of them; cut[j] is the [ninst] thresholds of cutoff j, rho[j]
 // its output row.
