@@ -119,7 +119,8 @@ enum {
  * DPC_PREC_FP32_CERT from 2 points per occupied cell on, pairs for float32 points
  * in binary64 from 800 chunks of 32 points on, segments otherwise, union in 1-D;
  * near phase: tensor tiles in 5-8 dimensions from 4 points per cell on, else the
- * tree, union in 1-D above 1e6 points) or the autotuned choice:
+ * tree, but union in 1-D above 1e6 points, and from 131,072 points on where the
+ * cells hold 512 points and more with DPC_PREC_FP32_CERT) or the autotuned choice:
  * 1 = union (a warp's 32 consecutive points, one query per lane, the union of
  * their blocks streamed as broadcast reads), 2 = segment (the points around a
  * few consecutive cells staged once, the cells' queries spread over the lanes),

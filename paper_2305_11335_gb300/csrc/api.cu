@@ -211,6 +211,7 @@ struct Choice {
   int ns = 0;    // near-phase grid levels below the density's
   int sc = 0;    // segment layouts: cells a segment's union may hold (0: one cell)
   uint32_t dfill = 0, nfill = 0;  // points per cell from which a tensor layout runs (0: always)
+  uint32_t ufill = 0;  // near phase in the tree layout: points per cell from which union runs (0: never)
 };
 
 struct Workspace {
@@ -744,6 +745,18 @@ void bin_class(Workspace* w, const void* pts, int dtype, const CallPlan& P, cons
 // 118 without.
 constexpr uint32_t kTensorDensityFill = 2, kTensorNearFill = 4;
 
+// Points per occupied cell from which the default near phase in 1-D scans the
+// block (union) instead of searching the tree, with the float32 filter and for
+// sets of some size: on smooth dense data the tree search meets long runs of
+// higher points (near phase + far search, us, union / tree: 300,000 points in
+// blobs, 882 a cell, 1,235 / 2,641; 1e6, 2,874 a cell, 9,758 / 20,729; 100,000,
+// 346 a cell, 529 / 516; 300,000, 49 a cell, 255 / 148; uniform, 18 a cell, 100 /
+// 99; integer clusters, where both search on through ties, 300 a cell 2,501 /
+// 2,250, 940 a cell 17,161 / 14,621; in binary64 the tree everywhere, 882 a cell
+// 13,678 / 6,661).
+constexpr uint32_t kUnionNearPoints = 1u << 17;
+constexpr uint32_t kUnionNearFill = 512;
+
 FarQueue queue_of(Workspace* w) {
   FarQueue q;
   q.pos = w->qpos;
@@ -798,6 +811,7 @@ void dependent_step(Workspace* w, const ClassPlan& c, const ClassView& cv, CutGe
   }
   {
     Phase ph(w, DPC_PHASE_NEAR);
+    uint32_t dense = 0;
     if (layout == kLayoutTensor && c.dp == 8 && !fp64) {
       launch_dep_near_tc(c.dmax, w->spts, w->scode, w->sid, w->skey, cv, rho_skip, pts, dtype, cuts, w->hinfo,
                          w->hkeys, w->hvals, w->pieces, lambda, delta, queue_of(w), w->ctr, min_fill, st);
@@ -808,11 +822,18 @@ void dependent_step(Workspace* w, const ClassPlan& c, const ClassView& cv, CutGe
     } else {
       // the tensor layout exists for 5-8 dimensions with the float32 filter
       if (layout == kLayoutTensor) layout = kLayoutUnion;
+      // 1-D by default: the block scan on dense cells, the tree elsewhere
+      if (layout == kLayoutTree && c.g == 1 && !fp64 && min_fill && cv.N >= kUnionNearPoints) dense = kUnionNearFill;
+      if (dense)
+        launch_dep_near(c.dp, c.g, c.dmax, fp64, kLayoutUnion, w->spts, w->scode, w->skey, cv, rho_skip, pts, dtype,
+                        cuts, w->hinfo, w->hkeys, w->hvals, lambda, delta, queue_of(w), w->ctr, st, w->nbox, w->roots,
+                        seg_cells, 0, dense);
       launch_dep_near(c.dp, c.g, c.dmax, fp64, layout, w->spts, w->scode, w->skey, cv, rho_skip, pts, dtype,
                       cuts, w->hinfo, w->hkeys, w->hvals, lambda, delta, queue_of(w), w->ctr, st,
-                      w->nbox, w->roots, seg_cells);
+                      w->nbox, w->roots, seg_cells, dense);
     }
     w->last_choice.nlay = layout;
+    w->last_choice.ufill = dense;
     w->last_choice.nfill = min_fill;
   }
   {
@@ -1838,6 +1859,7 @@ int dpc_get_stats(void* stream, dpc_stats* out) {
     auto sparse = [&](uint32_t fill) { return (uint64_t)w->last_points < (uint64_t)fill * hi.m; };
     out->density_layout = ch.dlay == kLayoutTensor && sparse(ch.dfill) ? kLayoutSegment : ch.dlay;
     out->near_layout = ch.nlay == kLayoutTensor && sparse(ch.nfill) ? kLayoutTree : ch.nlay;
+    if (ch.nlay == kLayoutTree && ch.ufill && !sparse(ch.ufill)) out->near_layout = kLayoutUnion;
     out->near_shift = w->last_choice.ns;
     out->bits_per_axis = g.B;
   }

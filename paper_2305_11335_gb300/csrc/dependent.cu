@@ -178,7 +178,8 @@ k_dep_near(const float* __restrict__ spts, const unsigned long long* __restrict_
            const void* __restrict__ pts, int dtype, const CutGeom* __restrict__ cuts,
            const HashInfo* __restrict__ hi, const unsigned long long* __restrict__ hkeys,
            const uint2* __restrict__ hvals, int32_t* __restrict__ lambda,
-           double* __restrict__ delta, FarQueue q, Counters* ctr) {
+           double* __restrict__ delta, FarQueue q, Counters* ctr, uint32_t min_fill) {
+  if (min_fill && !tensor_fill(cv.N, hi, min_fill)) return;  // the tree layout's part
   constexpr int kNearCap = DP == 8 ? 128 : 256;
   __shared__ __align__(16) float s_pts[kNearWarps * kNearCap * DP];
   __shared__ unsigned long long s_key[kNearWarps * kNearCap];
@@ -1236,8 +1237,9 @@ void near_dg(bool fp64, int layout, const float* spts, const unsigned long long*
              const unsigned long long* skey, const ClassView& cv, int32_t rho_skip,
              const void* pts, int dtype, const CutGeom* cuts, const HashInfo* hi,
              const unsigned long long* hkeys, const uint2* hvals, int32_t* lambda, double* delta,
-             FarQueue q, Counters* ctr, int seg_cells, cudaStream_t st) {
-  const unsigned grid = grid_for(cv.nchunk, kNearWarps, sm_count() * 64u);
+             FarQueue q, Counters* ctr, int seg_cells, uint32_t min_fill, cudaStream_t st) {
+  // (a launch that most sets leave at once: fewer CTAs)
+  const unsigned grid = grid_for(cv.nchunk, kNearWarps, sm_count() * (min_fill ? 16u : 64u));
   if (layout == kLayoutSegment) {
     if (fp64)
       k_dep_near_seg<DP, G, true><<<grid, kNearThreads, 0, st>>>(spts, scode, skey, cv, rho_skip, pts,
@@ -1251,11 +1253,11 @@ void near_dg(bool fp64, int layout, const float* spts, const unsigned long long*
     if (fp64)
       k_dep_near<DP, G, true><<<grid, kNearThreads, 0, st>>>(spts, scode, skey, cv, rho_skip, pts,
                                                              dtype, cuts, hi, hkeys, hvals, lambda,
-                                                             delta, q, ctr);
+                                                             delta, q, ctr, min_fill);
     else
       k_dep_near<DP, G, false><<<grid, kNearThreads, 0, st>>>(spts, scode, skey, cv, rho_skip, pts,
                                                               dtype, cuts, hi, hkeys, hvals, lambda,
-                                                              delta, q, ctr);
+                                                              delta, q, ctr, min_fill);
   }
 }
 
@@ -1292,10 +1294,10 @@ void launch_dep_near(int dp, int g, int dmax, bool fp64, int layout, const float
                      const CutGeom* cuts, const HashInfo* hi, const unsigned long long* hkeys,
                      const uint2* hvals, int32_t* lambda, double* delta, FarQueue q, Counters* ctr,
                      cudaStream_t st, const float* nbox, const uint32_t* roots, int seg_cells,
-                     uint32_t skip_fill) {
+                     uint32_t skip_fill, uint32_t min_fill) {
   if (cv.N == 0) return;
-  // (skip_fill, tree layout only: beside the tensor form, which has cleared the
-  // queue and may have filled it)
+  // (skip_fill: beside a form for dense cells, which has cleared the queue and may
+  // have filled it)
   if (!skip_fill) cudaMemsetAsync(&ctr->queue_n, 0, 2 * sizeof(unsigned int), st);  // queue_n and queue2_n
   if (layout == kLayoutCell) {
     launch_dep_near_cell(dp, g, fp64, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys,
@@ -1314,11 +1316,11 @@ void launch_dep_near(int dp, int g, int dmax, bool fp64, int layout, const float
     else if (dp == 4) go(k_near_to_far<4, 4, 4>);
     else if (rec_dims(dp, dmax) == 6) go(k_near_to_far<8, 6, 6>);
     else go(k_near_to_far<8, 8, 8>);
-  } else if (g == 1) near_dg<2, 1>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, st);
-  else if (g == 2) near_dg<2, 2>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, st);
-  else if (g == 3) near_dg<4, 3>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, st);
-  else if (dp == 4) near_dg<4, 4>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, st);
-  else near_dg<8, 4>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, st);
+  } else if (g == 1) near_dg<2, 1>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, min_fill, st);
+  else if (g == 2) near_dg<2, 2>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, min_fill, st);
+  else if (g == 3) near_dg<4, 3>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, min_fill, st);
+  else if (dp == 4) near_dg<4, 4>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, min_fill, st);
+  else near_dg<8, 4>(fp64, layout, spts, scode, skey, cv, rho_skip, pts, dtype, cuts, hi, hkeys, hvals, lambda, delta, q, ctr, seg_cells, min_fill, st);
   count_launches(1);
 }
 

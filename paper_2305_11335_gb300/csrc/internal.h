@@ -224,13 +224,15 @@ struct FarHint {
 };
 // lambda and delta are indexed by output index; lambda values are
 // instance-local ids
+// (skip_fill, tree layout: nothing from that many points per occupied cell on;
+// min_fill, union layout: nothing below it)
 void launch_dep_near(int dp, int g, int dmax, bool fp64, int layout, const float* spts,
                      const unsigned long long* scode, const unsigned long long* skey,
                      const ClassView& cv, int32_t rho_skip, const void* pts, int dtype,
                      const CutGeom* cuts, const HashInfo* hi, const unsigned long long* hkeys,
                      const uint2* hvals, int32_t* lambda, double* delta, FarQueue q, Counters* ctr,
                      cudaStream_t st, const float* nbox, const uint32_t* roots, int seg_cells = 0,
-                     uint32_t skip_fill = 0);
+                     uint32_t skip_fill = 0, uint32_t min_fill = 0);
 // the cell layout of the near phase (cell_tile.cu)
 void launch_dep_near_cell(int dp, int g, bool fp64, const float* spts,
                           const unsigned long long* scode, const unsigned long long* skey,
