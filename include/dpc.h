@@ -90,7 +90,10 @@ enum { DPC_I32 = 0, DPC_F32 = 1 };
 
 /* precision modes (flags & DPC_PREC_MASK).  Both give identical results. */
 enum {
-  DPC_PREC_FP64 = 0,     /* every distance evaluated in binary64              */
+  DPC_PREC_FP64 = 0,     /* every distance that counts or is compared evaluated
+                            in binary64 (densities of int32 points in 64-bit
+                            integers, the same values; the tree search's first
+                            bound is a float32 distance widened by its error) */
   DPC_PREC_FP32_CERT = 1 /* float32 filter + binary64 recheck of the band     */
 };
 #define DPC_PREC_MASK 0xFu
@@ -106,8 +109,11 @@ enum {
  * 0, 1 and 2 grid levels below the density's, timing each with CUDA events
  * and synchronizing the stream, and keeps the fastest for that shape in the
  * workspace; later calls (with or without the flag) reuse the choice without
- * synchronizing.  Results do not depend on the choice.  Do not set it on a
- * call that is being captured into a CUDA graph. */
+ * synchronizing.  A call with several cutoffs is not tuned and takes no tuned
+ * choice: its cutoffs share their passes, which beats one tuned pass per cutoff
+ * (1e7 points in 3-D at 2 cutoffs 30.6 -> 25.3 ms, 1e6 in 2-D at 3 4.3 -> 2.7).
+ * Results do not depend on the choice.  Do not set it on a call that is being
+ * captured into a CUDA graph. */
 #define DPC_FLAG_AUTOTUNE (1u << 10)
 /* Fixed block radius r = 1..5 instead of the default rule or the autotuned
  * choice (larger radii are clamped to the largest the dimension allows: 5 for
@@ -134,8 +140,7 @@ enum {
  * lane one query -- or a share of one query's candidates in cells of fewer than
  * 32 points -- against all of it).  Without a fixed radius, layout or near
  * shift small instances are compared in full (see dpc_stats.density_layout),
- * and the cutoffs of a sweep share their passes: neither autotuning nor its
- * choices apply to a call with several cutoffs.  Results do not depend on it. */
+ * and the cutoffs of a sweep share their passes.  Results do not depend on it. */
 #define DPC_FLAG_LAYOUT(v) ((uint32_t)(v) << 16)
 #define DPC_FLAG_LAYOUT_MASK (0x7u << 16)
 /* dpc_run only: capture the call's kernels into a CUDA graph the first time a
@@ -348,7 +353,9 @@ typedef struct {
   int32_t block_radius;   /* block radius R of the last cutoff (cells per side
                              of the (2R+1)^g block around a query's cell)     */
   int32_t density_layout; /* layout the last density launch ran: 1 union,
-                             2 segment, 4 tensor, 5 pairs, 6 cell
+                             2 segment (asked for with float32 points in
+                             binary64: pair by pair from 800 chunks on),
+                             4 tensor, 5 pairs, 6 cell
                              (see DPC_FLAG_LAYOUT); 0: small instances, all
                              pairs (no grid: its fields are 0 too)            */
   int32_t near_layout;    /* layout of the last near-dependent launch: 1 union,

@@ -738,11 +738,13 @@ void bin_class(Workspace* w, const void* pts, int dtype, const CallPlan& P, cons
 // Points per occupied cell from which the default layouts of 5-8 dimensions use
 // tensor tiles: a tile serves up to 128 queries at the cost of one, but sparse
 // cells leave its rows empty and every piece pays its lookups and waits.
-// Densities of 1e5 points in 5-D at 4 cutoffs (2-4 points per cell): 1.17 ms
-// with tiles from 1 point on, 1.47 from 4, 1.92 without; near phase of 1.6e6
-// points in 5-D at 8 cutoffs (3 points per cell): 60 ms with tiles, 48 with one
-// query per lane; of 2e6 points in 7-D (17 points per cell): 50 ms with tiles,
-// 118 without.
+// Densities of 1e5 points in 5-D at 4 cutoffs with tiles from 1 / 2 / 3 / 4 points
+// on / without, ms: 1.9 points per cell at the smallest cutoff 1.53 / 1.18 / 1.26 /
+// 1.25 / 1.24, 2.6 a cell 1.32 / 1.32 / 1.41 / 1.43 / 1.96, 3.1 a cell 1.38 / 1.38 /
+// 1.38 / 1.57 / 1.94; 128 instances of 2, 3 and 5 dimensions, 8 cutoffs, whole call
+// 84.4 / 84.4 / 81.6 / 81.6 (81.0 from 8 on).  Near phase, the same batch: 141 with
+// tiles from 1 or 2 points on, 84.5 from anything between 3 and 16; of 2e6 points
+// in 7-D (17 points per cell) 50 ms with tiles, 118 without.
 constexpr uint32_t kTensorDensityFill = 2, kTensorNearFill = 4;
 
 // Points per occupied cell from which the default near phase in 1-D scans the
@@ -981,10 +983,10 @@ inline int default_nlayout(const ClassPlan& c, bool fp64) {
   if (tensor_class(c, fp64)) return kLayoutTensor;
   return c.g == 1 && c.N > 1000000u ? kLayoutUnion : kLayoutTree;
 }
-// segments of the segment layouts span cells while their union fits this
-// (1e7 points in 3-D, density + near phase: 7.04 ms at 48 cells, 6.98 at 64,
-// 7.11 at 80, 7.41 at 128; 1e6 in 2-D, density: 0.43 ms one cell, 0.365 at 36,
-// 0.356 at 49, 0.545 at 81)
+// segments of the segment layouts span cells while their union fits this: the
+// middle of a flat range (1e7 points in 3-D, density + near phase: 7.78 ms at 40
+// cells, 7.10 at 48, 7.10 at 56, 7.03 at 64, 7.02 at 72, 7.17 at 80; 1e6 in 2-D,
+// density: .436 ms one cell, .371 at 25, .360 at 36, .364 at 49, .364 at 56)
 inline int default_seg_cells(int g) { return g == 3 ? 56 : (g == 2 ? 36 : 0); }
 
 // The grid level and kernel layouts of one (class, cutoff): a fixed radius or

@@ -170,10 +170,13 @@ k_density(const float* __restrict__ spts, const unsigned long long* __restrict__
 // the chip has enough warps to hide the lookups (1e4 points in 2-D: 83 us with
 // one warp per chunk; a replayed run 101 -> 70 us with this, the sort's small
 // tiles and the merged set-up launches).
-// What bounds it: issue slots; about half of them are the segment's set-up
-// (cell lookups, staging).  1e7 points in 3-D: 3.60 ms with the candidates in
-// registers across the lanes and one warp reduction per query pair and window
-// of 128 candidates, 2.65 with queries across the lanes.
+// What bounds it: issue slots (65% of them busy, 1.5 warps ready per cycle; DRAM 3%):
+// 16 instructions per lane and scanned pair, of which the loop over candidates
+// takes about 6 with every lane on a query, the rest the segment's set-up (cell
+// lookups, staging) and lanes without one (profiles/, 4e6 points in 3-D, 1.11 ms).
+// 1e7 points in 3-D: 3.60 ms with the candidates in registers across the lanes and
+// one warp reduction per query pair and window of 128 candidates, 2.65 with
+// queries across the lanes.
 // M cutoffs of a sweep that share the block geometry `geo` (M = 1: one cutoff)
 // are counted in one pass: the distances, lookups and staging are paid once,
 // every cutoff adds its own compare and count.
@@ -364,10 +367,10 @@ template <int DP>
 constexpr int pairs_v() { return DP == 2 ? 8 : (DP == 4 ? 8 : 4); }
 
 // Pair layout (symmetric): every unordered pair within d_cut is evaluated
-// once and counted for both points.  The work layout is k_density_seg's
-// (segments of equal cell, the block's candidates spread over the lanes, two
-// queries per pass), but a segment in cell A only takes the cells B of its
-// block that follow A in Morton order, plus the points of A itself that
+// once and counted for both points.  Segments are the points of one cell in a
+// chunk; the block's candidates are spread over the lanes, in registers, and the
+// segment's queries taken two per pass.  A segment in cell A only takes the cells
+// B of its block that follow A in Morton order, plus the points of A itself that
 // follow the query in sorted order.  A query's count stays in a register and
 // each candidate's in a register per slot; both go to a position-indexed
 // counter with one atomic add per window (candidates) or per chunk (queries).

@@ -358,11 +358,12 @@ k_dep_near(const float* __restrict__ spts, const unsigned long long* __restrict_
 // tile, four candidates at a time as broadcast reads.  The parts are merged with
 // shuffles at the end; lane j then settles the chunk's query j or queues it
 // for the far phase exactly as k_dep_near does.
-// What bounds it: issue slots (about 13 instructions per candidate and lane,
-// and the segment's set-up).  1e7 points in 3-D: 6.09 ms with the candidates in
-// registers across the lanes and a warp reduction per query and window, 5.6 with
-// those reductions only where a window could still matter, 4.4 with queries
-// across the lanes.
+// What bounds it: issue slots and the ALU pipe in them (61% and 62% busy, DRAM 5%):
+// 25 instructions per lane and scanned pair, set-up and idle lanes included
+// (profiles/, 4e6 points in 3-D, 1.74 ms).  1e7 points in 3-D: 6.09 ms with the
+// candidates in registers across the lanes and a warp reduction per query and
+// window, 5.6 with those reductions only where a window could still matter, 4.4
+// with queries across the lanes.
 template <int DP, int G>
 constexpr int near_cap() { return DP == 2 ? 512 : (DP == 4 && G < 4 ? 384 : (DP == 4 ? 256 : 128)); }
 

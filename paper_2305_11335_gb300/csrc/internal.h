@@ -128,15 +128,15 @@ inline int rec_dims(int dp, int dmax) { return dp == 8 && dmax <= 6 ? 6 : dp; }
 //   union    a warp owns 32 consecutive sorted points (one query per lane) and
 //            streams the union of their blocks through shared memory, every
 //            candidate a broadcast read (block.cuh)
-//   segment  the 32 points are split into segments of equal cell; the block's
-//            candidates are spread over the lanes (in registers) and the
-//            segment's queries are taken one at a time, one warp reduction each
+//   segment  the 32 points are split into segments of a cell or of a few
+//            consecutive ones; the points around a segment are staged in shared
+//            memory once and its queries spread over the lanes (CandTile)
 //   tree     (near phase only) no block scan: every query goes to the tree
 //            search of the far phase
 //   tensor   (density, 5-8 dimensions, float32 filter) the distance tiles on the
 //            tensor cores (tc_density.cu); other cases fall back to segment
-//   pairs    (density only) the segment layout counting every unordered pair
-//            once, for both of its points (density.cu, k_density_pairs)
+//   pairs    (density only) segments of one cell, every unordered pair counted
+//            once for both of its points (density.cu, k_density_pairs)
 // seg_cells (segment layouts): a segment may span several consecutive cells
 // while their bounding box grown by R holds at most seg_cells cells (0: one
 // cell per segment)

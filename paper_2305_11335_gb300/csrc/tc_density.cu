@@ -27,8 +27,10 @@
 // float32 filter on the original coordinates and, inside its own band, by the
 // canonical binary64 distance, so rho is exactly the binary64 count.
 //
-// What bounds it: the epilogue's ALU work and the barriers between staging, MMA
-// and epilogue (two CTAs per SM overlap them); the tensor pipe is 10-17% busy.
+// What bounds it: the epilogue's ALU work (ALU pipe 62% busy with three cutoffs in a
+// pass, 43% with one) and the barriers between staging, MMA and epilogue (two CTAs
+// per SM overlap them); the tensor pipe is 10% busy with three cutoffs in a pass,
+// 18% with one, 11% in the near phase (profiles/, 663,000 points in 7-D).
 // 2e6 points in 7-D: three cutoffs of one level in one pass 40 ms where three
 // passes of two separate operands, one cutoff each and one cell per piece took
 // about 35 each; the recount alone, unrolled per column and in binary64 for every
